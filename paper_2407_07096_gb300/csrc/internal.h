@@ -90,8 +90,12 @@ struct stag_kde {
     int64_t n_tiles = 0;
     int d_pad = 0;
 
-    // FP64 form: row-major points
+    // FP64 form: row-major points; partial sums, and per query tile a counter of the blocks
+    // that have stored theirs (both behind the points; a view has its own, view_scratch)
     double *x64 = nullptr;
+    double *f64_part = nullptr;
+    unsigned *tickets = nullptr;
+    void *view_scratch = nullptr;
 
     // tensor-core form
     stagkde::TcData *tc = nullptr;
@@ -131,8 +135,6 @@ void prof_stop(stag_kde *h, cudaStream_t s, double pairs);
 int simt_prepare_points(stag_kde *h, const float *dX);  // dX: device row-major n x d
 int simt_query_f32(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaStream_t s,
                    int *dflag);
-int simt_query_f64(stag_kde *h, const double *dQ, int64_t m, double *dOut, cudaStream_t s,
-                   int *dflag);
 int ensure_partials(stag_kde *h, int64_t entries);
 // The point set in its original order, row-major (from the plain form's tiled copy).
 int simt_points_rows(stag_kde *h, float *out, cudaStream_t s);
@@ -161,6 +163,12 @@ int subset_prepare(stag_kde *h, cudaStream_t s);
 int subset_check_entries(const int64_t *dIdx, const float *dW, int64_t nnz, int64_t n, int *dflag, cudaStream_t s);
 int subset_query(stag_kde *h, const float *dQ, int64_t m, const int64_t *dOff, const int64_t *dIdx, const float *dW,
                  double *dOut, cudaStream_t s, double entries);
+
+// kde_f64.cu
+constexpr int64_t kF64MaxD = 6144;  // coordinates the FP64 form takes
+size_t f64_scratch_bytes(const stag_kde *h);
+int f64_set_scratch(stag_kde *h, void *p);  // p: f64_scratch_bytes, owned by the caller
+int f64_query(stag_kde *h, const double *dQ, int64_t m, double *dOut, cudaStream_t s, int *dflag);
 
 // kde_combine.cu
 int launch_combine(const double *part_sum, const float *part_shift, int64_t m, int splits,

@@ -107,8 +107,6 @@ int reserve_all(BatchPlan *p) {
             rc = tc_reserve(h, m, p->tiles_per_unit);
         } else if (h->form == STAG_KDE_FORM_SIMT_F32) {
             rc = simt_reserve(h, m);
-        } else if (h->normalise) {
-            rc = ensure_partials(h, m);
         }
         if (rc) return rc;
     }
@@ -195,7 +193,7 @@ int enqueue(BatchPlan *p, cudaStream_t s) {
         else if (h->form == STAG_KDE_FORM_SIMT_F32)
             rc = simt_query_f32(h, (const float *)p->qs[i], p->ms[i], p->outs[i], si, nullptr);
         else
-            rc = simt_query_f64(h, (const double *)p->qs[i], p->ms[i], p->outs[i], si, nullptr);
+            rc = f64_query(h, (const double *)p->qs[i], p->ms[i], p->outs[i], si, nullptr);
     }
     if (!rc) rc = join();
     return rc;

@@ -1,4 +1,4 @@
-// Plain CUDA-core forms of exact KDE (Sec. 3: K(q) = sum_i k(||q - x_i||), by default the
+// Plain CUDA-core FP32 form of exact KDE (Sec. 3: K(q) = sum_i k(||q - x_i||), by default the
 // Gaussian kernel k(r) = exp(-a r^2); also the exponential and logistic kernels of Sec. 3),
 // evaluated over every data point, the "naive" exact method of Sec. 3 / Sec. 6.1.
 //
@@ -6,7 +6,6 @@
 //    4 queries x 4 points per thread, 64 x 64 pairs per 256-thread block, shared-memory
 //    chunks of 32 coordinates fed by cp.async; the exp and the row sum are fused, so no
 //    m x n matrix is ever written.
-//  * kde_simt_f64_kernel: FP64 direct differences and FP64 exp, for FP64 inputs.
 //
 // Exponent arithmetic (FP32 form). With c = a log2(e), every term is evaluated as
 //     e = 2^(-c d2 - s)      (one fused multiply-add, then ex2.approx)
@@ -354,40 +353,6 @@ __global__ void check_finite_kernel(const T *__restrict__ p, int64_t count, int 
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, bit);
 }
 
-// FP64 form: one thread per query, points staged through shared memory, summed in
-// index order with FP64 exp (plain double arithmetic, for FP64 inputs).
-__global__ void __launch_bounds__(128)
-kde_simt_f64_kernel(const double *__restrict__ X, int64_t n, const double *__restrict__ Q,
-                    int64_t m, int64_t d, double a, int kern, double *__restrict__ out) {
-    extern __shared__ double sx[];
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t tp = max((int64_t)1, (int64_t)(4096 / d));  // points per staged tile
-    double s = 0.0;
-    for (int64_t i0 = 0; i0 < n; i0 += tp) {
-        const int64_t cnt = min(tp, n - i0);
-        __syncthreads();
-        for (int64_t e = threadIdx.x; e < cnt * d; e += blockDim.x) sx[e] = X[i0 * d + e];
-        __syncthreads();
-        if (j < m) {
-            const double *q = Q + j * d;
-            for (int64_t i = 0; i < cnt; ++i) {
-                double d2 = 0.0;
-                for (int64_t k = 0; k < d; ++k) {
-                    const double t = q[k] - sx[i * d + k];
-                    d2 = fma(t, t, d2);
-                }
-                if (kern == STAG_KDE_KERNEL_GAUSSIAN) {
-                    s += exp(-a * d2);
-                } else {
-                    const double x = a * sqrt(d2);
-                    s += kern == STAG_KDE_KERNEL_EXPONENTIAL ? exp(-x) : 4.0 / (2.0 + exp(x) + exp(-x));
-                }
-            }
-        }
-    }
-    if (j < m) out[j] = s;
-}
-
 // Rows idx[0 .. *count) of the row-major Q, in that order, into the tile-transposed
 // layout (rows past *count are zero).
 __global__ void gather_rows_tiles_kernel(const float *__restrict__ Q, int64_t d, int d_pad,
@@ -589,31 +554,6 @@ int simt_tiles_from_rows(const stag_kde *h, const float *rows, float *out, cudaS
     count_launch();
     to_tiles_kernel<float><<<grid_for(total, 256), 256, 0, s>>>(rows, h->n, h->d, h->d_pad, h->n_tiles, out);
     STAG_CUDA_TRY(cudaGetLastError());
-    return 0;
-}
-
-int simt_query_f64(stag_kde *h, const double *dQ, int64_t m, double *dOut, cudaStream_t s, int *dflag) {
-    if (dflag) {
-        int rc = launch_check_finite_f64(dQ, m * h->d, dflag, s);
-        if (rc) return rc;
-    }
-    const int64_t tp = std::max<int64_t>(1, 4096 / h->d);
-    const size_t smem = (size_t)(tp * h->d) * sizeof(double);
-    if (smem > 48 * 1024) return fail(STAG_KDE_EUNSUPPORTED, "FP64 form: d too large");
-    count_launch();
-    prof_start(h, s);
-    kde_simt_f64_kernel<<<(unsigned)ceil_div(m, 128), 128, smem, s>>>(h->x64, h->n, dQ, m, h->d, h->a, h->kernel,
-                                                                       dOut);
-    prof_stop(h, s, (double)m * (double)h->n);
-    STAG_CUDA_TRY(cudaGetLastError());
-    if (h->normalise) {
-        // (1/n) applied by the combine kernel with a single split of FP64 partials
-        int rc = ensure_partials(h, m);
-        if (rc) return rc;
-        STAG_CUDA_TRY(cudaMemcpyAsync(h->part.sum, dOut, m * sizeof(double), cudaMemcpyDeviceToDevice, s));
-        STAG_CUDA_TRY(cudaMemsetAsync(h->part.shift, 0, m * sizeof(float), s));
-        return launch_combine(h->part.sum, h->part.shift, m, 1, 1.0 / (double)h->n, dOut, s);
-    }
     return 0;
 }
 

@@ -145,6 +145,7 @@ void free_handle(stag_kde *h) {
     cudaFree(h->out_dev);
     cudaFree(h->part.sum);
     cudaFree(h->part.shift);
+    cudaFree(h->view_scratch);
     cudaFree(h->flag_dev);
     if (h->flag_host) cudaFreeHost(h->flag_host);
     for (int i = 0; i < 2; ++i) {
@@ -188,6 +189,18 @@ stag_kde *make_view(stag_kde *base) {
         cuda_fail(e, "view set-up");
         free_handle(v);
         return nullptr;
+    }
+    if (v->x64) {
+        if ((e = dev_malloc(&v->view_scratch, f64_scratch_bytes(v))) != cudaSuccess) {
+            cuda_fail(e, "view set-up");
+            free_handle(v);
+            return nullptr;
+        }
+        // (the slots' streams do not wait for this one)
+        if (f64_set_scratch(v, v->view_scratch) || cudaStreamSynchronize(v->stream) != cudaSuccess) {
+            free_handle(v);
+            return nullptr;
+        }
     }
     if (tc_make_view(base, v)) {
         free_handle(v);
@@ -244,7 +257,7 @@ int run_query(stag_kde *h, const void *dQ, int64_t m, double *dOut, cudaStream_t
         case STAG_KDE_FORM_SIMT_F32:
             return simt_query_f32(h, (const float *)dQ, m, dOut, s, dflag);
         case STAG_KDE_FORM_SIMT_F64:
-            return simt_query_f64(h, (const double *)dQ, m, dOut, s, dflag);
+            return f64_query(h, (const double *)dQ, m, dOut, s, dflag);
         case STAG_KDE_FORM_TC:
             return tc_query(h, (const float *)dQ, m, dOut, s, dflag);
     }
@@ -322,9 +335,11 @@ stag_kde_t *stag_kde_create_ex(const void *X, int dtype, int64_t n, int64_t d, d
 
     const size_t bytes = (size_t)(n * d) * elem_size(dtype);
     if (dtype == STAG_KDE_F64) {
-        if ((e = dev_malloc(&h->x64, bytes)) != cudaSuccess) return bail("dev_malloc(X)", e);
+        const size_t off = (bytes + 255) / 256 * 256;
+        if ((e = dev_malloc(&h->x64, off + f64_scratch_bytes(h))) != cudaSuccess) return bail("dev_malloc(X)", e);
         if ((e = cudaMemcpyAsync(h->x64, X, bytes, cudaMemcpyHostToDevice, h->stream)) != cudaSuccess)
             return bail("cudaMemcpy(X)", e);
+        if (f64_set_scratch(h, reinterpret_cast<char *>(h->x64) + off)) return bail("prepare", cudaSuccess);
     } else {
         float *dX = nullptr;
         if ((e = dev_malloc(&dX, bytes)) != cudaSuccess) return bail("dev_malloc(X)", e);
@@ -369,7 +384,6 @@ int stag_kde_reserve(stag_kde_t *h, int64_t m) {
     if (rc) return rc;
     if (h->form == STAG_KDE_FORM_SIMT_F32) rc = simt_reserve(h, std::max<int64_t>(m, 1));
     if (h->form == STAG_KDE_FORM_TC) rc = tc_reserve(h, std::max<int64_t>(m, 1), h->tune_tiles_per_unit);
-    if (h->form == STAG_KDE_FORM_SIMT_F64 && h->normalise) rc = ensure_partials(h, std::max<int64_t>(m, 1));
     return rc;
 }
 
