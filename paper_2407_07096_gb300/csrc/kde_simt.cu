@@ -3,7 +3,7 @@
 // evaluated over every data point, the "naive" exact method of Sec. 3 / Sec. 6.1.
 //
 //  * kde_simt_f32_kernel: FP32 direct differences sum_k (q_k - x_k)^2, register-tiled
-//    4 queries x 4 points per thread, 64 x 64 pairs per 256-thread block, shared-memory
+//    8 queries x 4 points per thread, 64 x 64 pairs per 128-thread block, shared-memory
 //    chunks of 32 coordinates fed by cp.async; the exp and the row sum are fused, so no
 //    m x n matrix is ever written.
 //
@@ -40,6 +40,9 @@ constexpr float kShiftFloor = -0x1p100f;  // initial shift (an exact integer)
 constexpr float kOverflowGuard = 0x1p64f;
 constexpr int kFlushTiles = 16;
 constexpr int kSumBlock = 16;  // coordinates per partial chain of a squared distance
+constexpr int kThreads = 128;  // threads per block: 8 row groups x 16 point groups
+constexpr int kRows = 8;       // query rows per thread
+constexpr int kStages = 3;     // ring of staged chunks
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -104,128 +107,202 @@ __device__ __forceinline__ void merge(RowAcc &r, double oacc, float oshift) {
     r.shift = sm;
 }
 
-// One work item: a query tile of 64 rows (qbase, tile-transposed) against `ntiles` point
-// tiles, tile_at(i) giving the index of the i-th. Rows at or past rows_valid are
-// computed on zero padding and not stored; the partials of row r go to out_sum[r] and
-// out_shift[r].
-template <bool kQResident, int KERN, class TileAt>
-__device__ __forceinline__ void simt_item(float (*sX)[kSimtKC * kSimtTile], float (*sQ)[kSimtKC * kSimtTile],
-                                          const float *__restrict__ xt, int64_t n, const float *__restrict__ qbase,
-                                          int d_pad, float negc, int64_t ntiles, TileAt tile_at, int64_t rows_valid,
-                                          double *__restrict__ out_sum, float *__restrict__ out_shift) {
+// One work item: a query tile of 64 rows (qbase, tile-transposed with every value stored
+// twice) against `ntiles` point tiles, tile_at(i) giving the index of the i-th. Rows at or
+// past rows_valid are computed on zero padding and not stored; the partials of row r go
+// to out_sum[r] and out_shift[r]. `smem`: the block's dynamic shared memory (simt_smem).
+//
+// What bounds it: the FP32 pipe, two lane operations per coordinate and pair (a packed
+// instruction holds it for two cycles). The register tile of 8 rows x 4 points per thread
+// spends, per coordinate, 32 packed instructions on 5 shared-memory loads and nothing
+// else: the queries are stored duplicated, (q, q), so that a loaded 64-bit register is the
+// broadcast operand (building it took 8 moves per 16 packed instructions in the 4 x 4
+// tile before). Six shared-memory wavefronts per 64 pipe cycles. The stages are a ring of three
+// with one barrier per chunk: the barrier that publishes chunk i also shows that every
+// thread is done with chunk i - 1, whose stage then takes chunk i + 2.
+// Measured (before: 4 x 4 pairs per thread, 256 threads, two stages): n = 70000, m = 10000,
+// d = 784: 42.7 -> 34.8 ms (78 % of the FP32 pipe counting two operations per coordinate;
+// 5 % more is the last wave of blocks); exponential kernel, n = m = 1e5, d = 16: 17.6 ->
+// 12.1 ms. Four blocks per SM (128 registers) measured 4 % slower at d = 784, the same at
+// d = 16. Of the inner loop's form: a remainder loop beside the unrolled one 41.5 ms, steps
+// of 4 coordinates 40.9, of 8 38.5, of 16 36.9, with constant-trip copies 34.8.
+// A row's arithmetic depends on its 16 point lanes and the order of the tiles only, not on
+// how many rows a thread or a block takes.
+template <bool kQResident, bool kOneBlock, int KERN, class TileAt>
+__device__ __forceinline__ void simt_item(float *__restrict__ smem, const float *__restrict__ xt, int64_t n,
+                                          const float *__restrict__ qbase, int d_pad, float negc, int64_t ntiles,
+                                          TileAt tile_at, int64_t rows_valid, double *__restrict__ out_sum,
+                                          float *__restrict__ out_shift) {
     const int tid = threadIdx.x;
     const int tx = tid & 15;  // point group: points 4*tx .. 4*tx+3 of the tile
-    const int ty = tid >> 4;  // query group: rows 4*ty .. 4*ty+3 of the block
-    const int nch = (d_pad + kSimtKC - 1) / kSimtKC;
+    const int ty = tid >> 4;  // query group: rows 8*ty .. 8*ty+7 of the block
+    const int nch = kOneBlock ? 1 : (d_pad + kSimtKC - 1) / kSimtKC;
+    constexpr int kXStage = kSimtKC * kSimtTile, kQStage = 2 * kXStage;  // floats
+    float *sX = smem, *sQ = smem + kStages * kXStage;
 
-    RowAcc row[4];
+    RowAcc row[kRows];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) row[i] = RowAcc{kShiftFloor, 0.f, 0.0};
+    for (int i = 0; i < kRows; ++i) row[i] = RowAcc{kShiftFloor, 0.f, 0.0};
 
-    auto load = [&](int stage, int64_t t, int ch) {
-        const int k0 = ch * kSimtKC;
-        const int klen = min(kSimtKC, d_pad - k0);
-        const int nvec = klen * (kSimtTile / 4);
-        const float *src = xt + (t * d_pad + k0) * kSimtTile;
-        for (int v = tid; v < nvec; v += 256) cp_async16(&sX[stage][v * 4], src + v * 4);
-        if (!kQResident) {
-            const float *qs = qbase + (int64_t)k0 * kSimtTile;
-            for (int v = tid; v < nvec; v += 256) cp_async16(&sQ[kQResident ? 0 : stage][v * 4], qs + v * 4);
+    const int64_t iters = ntiles * nch;
+    // chunk lch of the tile with list index lt is the next one to load, into stage ls
+    int64_t lt = 0;
+    int lch = 0, ls = 0;
+    auto load_next = [&]() {
+        if (lt < ntiles) {
+            const int k0 = lch * kSimtKC;
+            const int nvec = min(kSimtKC, d_pad - k0) * (kSimtTile / 4);
+            const float *src = xt + (tile_at(lt) * d_pad + k0) * kSimtTile;
+            float *dst = sX + ls * kXStage;
+            if (nvec == kSimtKC * (kSimtTile / 4)) {  // a whole chunk: constant trip count
+#pragma unroll
+                for (int v = 0; v < kSimtKC * (kSimtTile / 4); v += kThreads)
+                    cp_async16(dst + (v + tid) * 4, src + (v + tid) * 4);
+            } else {
+                for (int v = tid; v < nvec; v += kThreads) cp_async16(dst + v * 4, src + v * 4);
+            }
+            if (!kQResident) {
+                const float *qs = qbase + (int64_t)k0 * kSimtTile * 2;
+                float *qd = sQ + ls * kQStage;
+                if (nvec == kSimtKC * (kSimtTile / 4)) {
+#pragma unroll
+                    for (int v = 0; v < kSimtKC * (kSimtTile / 2); v += kThreads)
+                        cp_async16(qd + (v + tid) * 4, qs + (v + tid) * 4);
+                } else {
+                    for (int v = tid; v < 2 * nvec; v += kThreads) cp_async16(qd + v * 4, qs + v * 4);
+                }
+            }
+            if (++lch == nch) {
+                lch = 0;
+                ++lt;
+            }
         }
+        ls = ls + 1 == kStages ? 0 : ls + 1;
+        cp_async_commit();
     };
 
     if (kQResident) {
-        const int nvec = d_pad * (kSimtTile / 4);
-        for (int v = tid; v < nvec; v += 256) cp_async16(&sQ[0][v * 4], qbase + v * 4);
+        const int nvec = d_pad * (kSimtTile / 2);
+        for (int v = tid; v < nvec; v += kThreads) cp_async16(sQ + v * 4, qbase + v * 4);
     }
-    const int64_t iters = ntiles * nch;
-    if (iters > 0) load(0, tile_at(0), 0);
-    cp_async_commit();
+    load_next();
+    load_next();
 
-    // squared distances of the 4 x 4 pairs, as packed column pairs (4*tx+0,1) and (+2,3)
-    uint64_t d2p[4][2];
+    // squared distances of the 8 x 4 pairs, as packed column pairs (4*tx+0,1) and (+2,3)
+    uint64_t d2p[kRows][2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) d2p[i][0] = d2p[i][1] = 0ull;
+    for (int i = 0; i < kRows; ++i) d2p[i][0] = d2p[i][1] = 0ull;
+    const uint64_t negc2 = f2::pack(negc, negc);
 
-    int group = 0;
+    int group = 0, ch = 0, cs = 0;
+    int64_t ct = 0;
     for (int64_t it = 0; it < iters; ++it) {
-        const int stage = (int)(it & 1);
-        if (it + 1 < iters) {
-            load(stage ^ 1, tile_at((it + 1) / nch), (int)((it + 1) % nch));
-            cp_async_commit();
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
+        cp_async_wait<1>();
         __syncthreads();
+        load_next();
 
-        const int ch = (int)(it % nch);
         const int klen = min(kSimtKC, d_pad - ch * kSimtKC);
-        const float *xs = sX[stage];
-        const float *qs = kQResident ? sQ[0] + ch * kSimtKC * kSimtTile : sQ[kQResident ? 0 : stage];
+        const float *xs = sX + cs * kXStage + tx * 4;
+        const float *qs = (kQResident ? sQ + ch * kQStage : sQ + cs * kQStage) + ty * (2 * kRows);
         // blocks of kSumBlock coordinates: each block's squares are summed in a chain of
         // its own and the block sum is added to the pair's total, which keeps the
         // accumulated rounding error of d2 about half that of one chain over all d
         for (int kb = 0; kb < klen; kb += kSumBlock) {
             const int ke = min(klen, kb + kSumBlock);
-            uint64_t b2p[4][2];
+            uint64_t b2p[kRows][2];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) b2p[i][0] = b2p[i][1] = 0ull;
-#pragma unroll 4
-            for (int k = kb; k < ke; ++k) {
-                const float4 qv = *reinterpret_cast<const float4 *>(&qs[k * kSimtTile + ty * 4]);
-                const float4 xv = *reinterpret_cast<const float4 *>(&xs[k * kSimtTile + tx * 4]);
-                const float qa[4] = {qv.x, qv.y, qv.z, qv.w};
-                const uint64_t x01 = f2::pack(xv.x, xv.y), x23 = f2::pack(xv.z, xv.w);
+            for (int i = 0; i < kRows; ++i) b2p[i][0] = b2p[i][1] = 0ull;
+            auto step = [&](int k) {
+                const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(xs + k * kSimtTile);
+                uint64_t qq[kRows];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint64_t qq = f2::pack(qa[i], qa[i]);
-                    const uint64_t df0 = f2::sub(qq, x01), df1 = f2::sub(qq, x23);
+                for (int i = 0; i < kRows; i += 2) {
+                    const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(qs + k * 2 * kSimtTile + i * 2);
+                    qq[i] = t.x;
+                    qq[i + 1] = t.y;
+                }
+#pragma unroll
+                for (int i = 0; i < kRows; ++i) {
+                    const uint64_t df0 = f2::sub(qq[i], xv.x), df1 = f2::sub(qq[i], xv.y);
                     b2p[i][0] = f2::fma(df0, df0, b2p[i][0]);
                     b2p[i][1] = f2::fma(df1, df1, b2p[i][1]);
                 }
+            };
+            // whole blocks unrolled, the rest in steps of 4 (d_pad is a multiple of 4): no
+            // remainder loop, whose copies of the body cost 15 instructions per coordinate
+            if (ke - kb == kSumBlock) {
+#pragma unroll
+                for (int k = 0; k < kSumBlock; ++k) step(kb + k);
+            } else {
+#pragma unroll 1
+                for (int k1 = kb; k1 < ke; k1 += 4) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) step(k1 + k);
+                }
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                d2p[i][0] = f2::add(d2p[i][0], b2p[i][0]);
-                d2p[i][1] = f2::add(d2p[i][1], b2p[i][1]);
+            for (int i = 0; i < kRows; ++i) {
+                // (one block in all: its sums are the totals)
+                d2p[i][0] = kOneBlock ? b2p[i][0] : f2::add(d2p[i][0], b2p[i][0]);
+                d2p[i][1] = kOneBlock ? b2p[i][1] : f2::add(d2p[i][1], b2p[i][1]);
             }
         }
-        __syncthreads();
+        cs = cs + 1 == kStages ? 0 : cs + 1;
 
-        if (ch == nch - 1) {
-            const int64_t t = tile_at(it / nch);
-            const int64_t col0 = t * kSimtTile + tx * 4;
+        if (++ch == nch) {
+            ch = 0;
+            const int64_t col0 = tile_at(ct++) * kSimtTile + tx * 4;
             const int valid = (int)max((int64_t)0, min((int64_t)4, n - col0));
+            // the common case, a full tile whose terms fit the rows' shifts: no selects and
+            // one branch for all rows
+            float ts[kRows];
+            bool slow = valid < 4;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float d2[4];
-                f2::unpack(d2p[i][0], d2[0], d2[1]);
-                f2::unpack(d2p[i][1], d2[2], d2[3]);
-                add_terms<KERN>(row[i], d2, negc, valid);
-                d2p[i][0] = d2p[i][1] = 0ull;
+            for (int i = 0; i < kRows; ++i) {
+                float e0, e1, e2, e3;
+                kfn::term2<KERN>(negc, negc2, d2p[i][0], row[i].shift, e0, e1);
+                kfn::term2<KERN>(negc, negc2, d2p[i][1], row[i].shift, e2, e3);
+                ts[i] = ((e0 + e1) + e2) + e3;
+                slow = slow || !(ts[i] <= kOverflowGuard);
+            }
+            if (slow) {
+#pragma unroll
+                for (int i = 0; i < kRows; ++i) {
+                    float d2[4];
+                    f2::unpack(d2p[i][0], d2[0], d2[1]);
+                    f2::unpack(d2p[i][1], d2[2], d2[3]);
+                    add_terms<KERN>(row[i], d2, negc, valid);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < kRows; ++i) row[i].acc32 += ts[i];
+            }
+            if (!kOneBlock) {
+#pragma unroll
+                for (int i = 0; i < kRows; ++i) d2p[i][0] = d2p[i][1] = 0ull;
             }
             if (++group == kFlushTiles) {
                 group = 0;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < kRows; ++i) {
                     row[i].acc64 += (double)row[i].acc32;
                     row[i].acc32 = 0.f;
                 }
             }
         }
     }
+    cp_async_wait<0>();
 
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kRows; ++i) {
         row[i].acc64 += (double)row[i].acc32;
         row[i].acc32 = 0.f;
     }
-    // Combine the 16 threads of the half-warp that share rows 4*ty..4*ty+3.
+    // Combine the 16 threads of the half-warp that share rows 8*ty..8*ty+7.
 #pragma unroll
     for (int off = 8; off >= 1; off >>= 1) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < kRows; ++i) {
             const double oa = __shfl_xor_sync(0xffffffffu, row[i].acc64, off);
             const float os = __shfl_xor_sync(0xffffffffu, row[i].shift, off);
             merge(row[i], oa, os);
@@ -233,8 +310,8 @@ __device__ __forceinline__ void simt_item(float (*sX)[kSimtKC * kSimtTile], floa
     }
     if (tx == 0) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = ty * 4 + i;
+        for (int i = 0; i < kRows; ++i) {
+            const int r = ty * kRows + i;
             if (r < rows_valid) {
                 out_sum[r] = row[i].acc64;
                 out_shift[r] = row[i].shift;
@@ -243,37 +320,21 @@ __device__ __forceinline__ void simt_item(float (*sX)[kSimtKC * kSimtTile], floa
     }
 }
 
-// The contiguous point tiles of split `split` against query tile `qtile`; partials of
-// query q at part_sum[split * m + q] (rows from m_real on are not stored).
-template <bool kQResident, int KERN>
-__device__ __forceinline__ void simt_split_item(float (*sX)[kSimtKC * kSimtTile], float (*sQ)[kSimtKC * kSimtTile],
-                                                const float *__restrict__ xt, int64_t n, int64_t n_tiles,
-                                                const float *__restrict__ qt, int64_t m, int64_t m_real, int d_pad,
-                                                float negc, int64_t tiles_per_split, double *__restrict__ part_sum,
-                                                float *__restrict__ part_shift, int64_t qtile, int64_t split) {
-    const int64_t t0 = split * tiles_per_split;
-    const int64_t t1 = min(n_tiles, t0 + tiles_per_split);
-    const int64_t off = split * m + qtile * kSimtTile;
-    simt_item<kQResident, KERN>(sX, sQ, xt, n, qt + qtile * (int64_t)d_pad * kSimtTile, d_pad, negc,
-                                  max((int64_t)0, t1 - t0), [t0](int64_t i) { return t0 + i; },
-                                  m_real - qtile * kSimtTile, part_sum + off, part_shift + off);
-}
-
-template <bool kQResident, int KERN>
-__global__ void __launch_bounds__(256, 2)
+// One block per (query tile, contiguous range of point tiles); the partials of query q of
+// range s go to part_sum[s * m + q].
+template <bool kQResident, bool kOneBlock, int KERN>
+__global__ void __launch_bounds__(kThreads, 3)
 kde_simt_f32_kernel(const float *__restrict__ xt, int64_t n, int64_t n_tiles, const float *__restrict__ qt, int64_t m,
                     int d_pad, float negc, int64_t tiles_per_split, double *__restrict__ part_sum,
                     float *__restrict__ part_shift) {
-    __shared__ __align__(16) float sX[2][kSimtKC * kSimtTile];
-    // resident query tile: all d_pad coordinates (dynamic, d_pad x 64 floats); otherwise
-    // double-buffered chunks of the query tile
-    extern __shared__ __align__(16) float sQres[];
-    __shared__ __align__(16) float sQchunk[kQResident ? 1 : 2][kQResident ? 4 : kSimtKC * kSimtTile];
-    auto sQ = kQResident ? reinterpret_cast<float (*)[kSimtKC * kSimtTile]>(sQres)
-                         : reinterpret_cast<float (*)[kSimtKC * kSimtTile]>(&sQchunk[0][0]);
-    // one block per (query tile, split)
-    simt_split_item<kQResident, KERN>(sX, sQ, xt, n, n_tiles, qt, m, m, d_pad, negc, tiles_per_split, part_sum,
-                                        part_shift, blockIdx.x, blockIdx.y);
+    extern __shared__ __align__(16) float smem[];
+    const int64_t qtile = blockIdx.x, split = blockIdx.y;
+    const int64_t t0 = split * tiles_per_split;
+    const int64_t t1 = min(n_tiles, t0 + tiles_per_split);
+    const int64_t off = split * m + qtile * kSimtTile;
+    simt_item<kQResident, kOneBlock, KERN>(
+        smem, xt, n, qt + qtile * (int64_t)d_pad * (2 * kSimtTile), d_pad, negc, max((int64_t)0, t1 - t0),
+        [t0](int64_t i) { return t0 + i; }, m - qtile * kSimtTile, part_sum + off, part_shift + off);
 }
 
 // The grouped recompute of the tensor-core form's flagged queries (kde_tc.cu): work item
@@ -282,20 +343,14 @@ kde_simt_f32_kernel(const float *__restrict__ xt, int64_t n, int64_t n_tiles, co
 // list kept[g * kstride ..], s = w - item_off[g]; each kept tile is `per` consecutive
 // 64-point tiles of xt. Query group g is tile g of qt (64 gathered rows). The partials of
 // row r go to part_sum[w * 64 + r]. A fixed grid walks the items (counts on the device).
-template <bool kQResident, int KERN>
-__global__ void __launch_bounds__(256, 2)
+template <bool kQResident, bool kOneBlock, int KERN>
+__global__ void __launch_bounds__(kThreads, 3)
 kde_simt_f32_list_kernel(const float *__restrict__ xt, int64_t n, int64_t n_tiles, const float *__restrict__ qt,
                          int d_pad, float negc, const int *__restrict__ kept, int64_t kstride,
                          const int *__restrict__ kcount, const int *__restrict__ item_off,
                          const int *__restrict__ n_groups, int seg, int per, double *__restrict__ part_sum,
                          float *__restrict__ part_shift) {
-    __shared__ __align__(16) float sX[2][kSimtKC * kSimtTile];
-    // resident query tile: all d_pad coordinates (dynamic, d_pad x 64 floats); otherwise
-    // double-buffered chunks of the query tile
-    extern __shared__ __align__(16) float sQres[];
-    __shared__ __align__(16) float sQchunk[kQResident ? 1 : 2][kQResident ? 4 : kSimtKC * kSimtTile];
-    auto sQ = kQResident ? reinterpret_cast<float (*)[kSimtKC * kSimtTile]>(sQres)
-                         : reinterpret_cast<float (*)[kSimtKC * kSimtTile]>(&sQchunk[0][0]);
+    extern __shared__ __align__(16) float smem[];
     const int G = *n_groups;
     const int total = G > 0 ? item_off[G] : 0;
     for (int w = blockIdx.x; w < total; w += gridDim.x) {
@@ -316,15 +371,16 @@ kde_simt_f32_list_kernel(const float *__restrict__ xt, int64_t n, int64_t n_tile
         // be the list's last entry (the lists ascend), whose tail is enumerated last
         int64_t nt = (int64_t)(k1 - k0) * per;
         if (k1 > k0) nt -= max((int64_t)0, ((int64_t)list[k1 - k0 - 1] + 1) * per - n_tiles);
-        simt_item<kQResident, KERN>(
-            sX, sQ, xt, n, qt + (int64_t)g * d_pad * kSimtTile, d_pad, negc, nt,
+        simt_item<kQResident, kOneBlock, KERN>(
+            smem, xt, n, qt + (int64_t)g * d_pad * (2 * kSimtTile), d_pad, negc, nt,
             [list, per](int64_t i) { return (int64_t)list[i / per] * per + i % per; }, kSimtTile,
             part_sum + (int64_t)w * kSimtTile, part_shift + (int64_t)w * kSimtTile);
     }
 }
 
-// Row-major n x d -> tile-transposed [tile][d_pad][64], zero padded.
-template <typename T>
+// Row-major n x d -> tile-transposed [tile][d_pad][64], zero padded. kDup: every value
+// twice, [tile][d_pad][64][2] (queries).
+template <typename T, bool kDup>
 __global__ void to_tiles_kernel(const T *__restrict__ src, int64_t rows, int64_t d, int d_pad,
                                 int64_t n_tiles, float *__restrict__ dst) {
     const int64_t total = n_tiles * d_pad * kSimtTile;
@@ -337,7 +393,10 @@ __global__ void to_tiles_kernel(const T *__restrict__ src, int64_t rows, int64_t
         const int64_t row = t * kSimtTile + r;
         float v = 0.f;
         if (row < rows && k < d) v = (float)src[row * d + k];
-        dst[idx] = v;
+        if (kDup)
+            reinterpret_cast<float2 *>(dst)[idx] = make_float2(v, v);
+        else
+            dst[idx] = v;
     }
 }
 
@@ -354,7 +413,7 @@ __global__ void check_finite_kernel(const T *__restrict__ p, int64_t count, int 
 }
 
 // Rows idx[0 .. *count) of the row-major Q, in that order, into the tile-transposed
-// layout (rows past *count are zero).
+// query layout (every value twice; rows past *count are zero).
 __global__ void gather_rows_tiles_kernel(const float *__restrict__ Q, int64_t d, int d_pad,
                                          const int *__restrict__ idx, const int *__restrict__ count, int64_t m_cap,
                                          float *__restrict__ qt) {
@@ -365,7 +424,8 @@ __global__ void gather_rows_tiles_kernel(const float *__restrict__ Q, int64_t d,
         const int64_t rest = e / kSimtTile;
         const int k = (int)(rest % d_pad);
         const int64_t j = (rest / d_pad) * kSimtTile + r;
-        qt[e] = (j < cnt && k < d) ? Q[(int64_t)idx[j] * d + k] : 0.f;
+        const float v = (j < cnt && k < d) ? Q[(int64_t)idx[j] * d + k] : 0.f;
+        reinterpret_cast<float2 *>(qt)[e] = make_float2(v, v);
     }
 }
 
@@ -420,23 +480,46 @@ int simt_prepare_points(stag_kde *h, const float *dX) {
     const int64_t total = h->n_tiles * h->d_pad * kSimtTile;
     STAG_CUDA_TRY(dev_malloc(&h->xt, total * sizeof(float)));
     count_launch();
-    to_tiles_kernel<float><<<grid_for(total, 256), 256, 0, h->stream>>>(dX, h->n, h->d, h->d_pad,
+    to_tiles_kernel<float, false><<<grid_for(total, 256), 256, 0, h->stream>>>(dX, h->n, h->d, h->d_pad,
                                                                         h->n_tiles, h->xt);
     STAG_CUDA_TRY(cudaGetLastError());
     return 0;
 }
 
-// Launches the FP32 kernel instance for the handle's operand width and kernel function.
-template <int KERN>
-void launch_simt_kern(const stag_kde *h, dim3 grid, cudaStream_t s, int64_t m, float negc, int64_t tps) {
-    if (h->d_pad <= kSimtResidentMaxD)
-        kde_simt_f32_kernel<true, KERN><<<grid, 256, simt_resident_bytes(h->d_pad), s>>>(h->xt, h->n, h->n_tiles, h->qt, m, h->d_pad, negc, tps,
-                                                             h->part.sum, h->part.shift);
-    else
-        kde_simt_f32_kernel<false, KERN><<<grid, 256, 0, s>>>(h->xt, h->n, h->n_tiles, h->qt, m, h->d_pad, negc, tps,
-                                                              h->part.sum, h->part.shift);
+// Dynamic shared memory of simt_item: the ring of point chunks, and the queries (the whole
+// duplicated tile, or a ring of chunks).
+constexpr int kChunkBytes = kSimtKC * kSimtTile * 4;
+size_t simt_smem(int d_pad) {
+    return d_pad <= kSimtResidentMaxD ? kStages * kChunkBytes + (size_t)d_pad * kSimtTile * 8
+                                      : (size_t)kStages * 3 * kChunkBytes;
 }
-void launch_simt(const stag_kde *h, dim3 grid, cudaStream_t s, int64_t m, int64_t tps) {
+
+template <typename F>
+cudaError_t allow_smem(F *kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                std::max<int>(kStages * 3 * kChunkBytes,
+                                              kStages * kChunkBytes + kSimtResidentMaxD * kSimtTile * 8));
+}
+
+// Launches the FP32 kernel instance for the handle's operand width and kernel function:
+// up to 16 coordinates a pair's squared distance is one chain (no second set of totals).
+template <bool kQResident, bool kOneBlock, int KERN>
+int launch_simt_inst(const stag_kde *h, dim3 grid, cudaStream_t s, int64_t m, float negc, int64_t tps) {
+    auto kern = kde_simt_f32_kernel<kQResident, kOneBlock, KERN>;
+    // set once per instantiation (before any stream capture can be in progress)
+    static const cudaError_t attr = allow_smem(kern);
+    STAG_CUDA_TRY(attr);
+    kern<<<grid, kThreads, simt_smem(h->d_pad), s>>>(h->xt, h->n, h->n_tiles, h->qt, m, h->d_pad, negc, tps,
+                                                     h->part.sum, h->part.shift);
+    return 0;
+}
+template <int KERN>
+int launch_simt_kern(const stag_kde *h, dim3 grid, cudaStream_t s, int64_t m, float negc, int64_t tps) {
+    if (h->d_pad <= kSumBlock) return launch_simt_inst<true, true, KERN>(h, grid, s, m, negc, tps);
+    if (h->d_pad <= kSimtResidentMaxD) return launch_simt_inst<true, false, KERN>(h, grid, s, m, negc, tps);
+    return launch_simt_inst<false, false, KERN>(h, grid, s, m, negc, tps);
+}
+int launch_simt(const stag_kde *h, dim3 grid, cudaStream_t s, int64_t m, int64_t tps) {
     const float negc = (float)(-h->a * 1.4426950408889634);  // -a log2(e)
     switch (h->kernel) {
         case STAG_KDE_KERNEL_EXPONENTIAL:
@@ -461,11 +544,11 @@ static int64_t choose_tiles_per_split(const stag_kde *h, int64_t q_tiles) {
 int simt_query_f32(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaStream_t s,
                    int *dflag) {
     const int64_t q_tiles = ceil_div(m, kSimtTile);
-    int rc = ensure_qt(h, q_tiles * h->d_pad * kSimtTile);
+    int rc = ensure_qt(h, q_tiles * h->d_pad * kSimtTile * 2);
     if (rc) return rc;
     const int64_t total = q_tiles * h->d_pad * kSimtTile;
     count_launch();
-    to_tiles_kernel<float><<<grid_for(total, 256), 256, 0, s>>>(dQ, m, h->d, h->d_pad, q_tiles, h->qt);
+    to_tiles_kernel<float, true><<<grid_for(total, 256), 256, 0, s>>>(dQ, m, h->d, h->d_pad, q_tiles, h->qt);
     STAG_CUDA_TRY(cudaGetLastError());
     if (dflag) {
         rc = launch_check_finite_f32(dQ, m * h->d, dflag, s);
@@ -479,8 +562,9 @@ int simt_query_f32(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaSt
     dim3 grid((unsigned)q_tiles, (unsigned)splits);
     count_launch();
     prof_start(h, s);
-    launch_simt(h, grid, s, m, tps);
+    rc = launch_simt(h, grid, s, m, tps);
     prof_stop(h, s, (double)m * (double)h->n);
+    if (rc) return rc;
     STAG_CUDA_TRY(cudaGetLastError());
     return launch_combine(h->part.sum, h->part.shift, m, (int)splits, h->normalise ? 1.0 / (double)h->n : 1.0,
                           dOut, s);
@@ -488,7 +572,7 @@ int simt_query_f32(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaSt
 
 int simt_reserve(stag_kde *h, int64_t m) {
     const int64_t q_tiles = ceil_div(m, kSimtTile);
-    int rc = ensure_qt(h, q_tiles * h->d_pad * kSimtTile);
+    int rc = ensure_qt(h, q_tiles * h->d_pad * kSimtTile * 2);
     if (rc) return rc;
     const int64_t tps = choose_tiles_per_split(h, q_tiles);
     return ensure_partials(h, ceil_div(h->n_tiles, tps) * m);
@@ -522,22 +606,33 @@ int launch_subtract(double *v, int64_t count, double one, cudaStream_t s) {
     return 0;
 }
 
+template <bool kQResident, bool kOneBlock>
+static int list_launch_inst(const stag_kde *h, const float *xt, const float *qt, const int *kept, int64_t kstride,
+                            const int *kcount, const int *item_off, const int *n_groups, int seg, int per,
+                            double *part_sum, float *part_shift, cudaStream_t s) {
+    auto kern = kde_simt_f32_list_kernel<kQResident, kOneBlock, STAG_KDE_KERNEL_GAUSSIAN>;
+    static const cudaError_t attr = allow_smem(kern);
+    STAG_CUDA_TRY(attr);
+    const float negc = (float)(-h->a * 1.4426950408889634);  // -a log2(e)
+    count_launch();
+    kern<<<(unsigned)(h->sm_count * 3), kThreads, simt_smem(h->d_pad), s>>>(
+        xt, h->n, h->n_tiles, qt, h->d_pad, negc, kept, kstride, kcount, item_off, n_groups, seg, per, part_sum,
+        part_shift);
+    STAG_CUDA_TRY(cudaGetLastError());
+    return 0;
+}
+
 int simt_list_launch(const stag_kde *h, const float *xt, const float *qt, const int *kept, int64_t kstride,
                      const int *kcount, const int *item_off, const int *n_groups, int seg, int per, double *part_sum,
                      float *part_shift, cudaStream_t s) {
-    const float negc = (float)(-h->a * 1.4426950408889634);  // -a log2(e)
-    const dim3 grid((unsigned)(h->sm_count * 2));
-    count_launch();
+    if (h->d_pad <= kSumBlock)
+        return list_launch_inst<true, true>(h, xt, qt, kept, kstride, kcount, item_off, n_groups, seg, per, part_sum,
+                                            part_shift, s);
     if (h->d_pad <= kSimtResidentMaxD)
-        kde_simt_f32_list_kernel<true, STAG_KDE_KERNEL_GAUSSIAN><<<grid, 256, simt_resident_bytes(h->d_pad), s>>>(
-            xt, h->n, h->n_tiles, qt, h->d_pad, negc, kept, kstride, kcount, item_off, n_groups, seg, per, part_sum,
-            part_shift);
-    else
-        kde_simt_f32_list_kernel<false, STAG_KDE_KERNEL_GAUSSIAN><<<grid, 256, 0, s>>>(
-            xt, h->n, h->n_tiles, qt, h->d_pad, negc, kept, kstride, kcount, item_off, n_groups, seg, per, part_sum,
-            part_shift);
-    STAG_CUDA_TRY(cudaGetLastError());
-    return 0;
+        return list_launch_inst<true, false>(h, xt, qt, kept, kstride, kcount, item_off, n_groups, seg, per,
+                                             part_sum, part_shift, s);
+    return list_launch_inst<false, false>(h, xt, qt, kept, kstride, kcount, item_off, n_groups, seg, per, part_sum,
+                                          part_shift, s);
 }
 
 int simt_gather_rows(const stag_kde *h, const float *dQ, const int *idx, const int *count, int64_t m_cap, float *qt,
@@ -552,7 +647,7 @@ int simt_gather_rows(const stag_kde *h, const float *dQ, const int *idx, const i
 int simt_tiles_from_rows(const stag_kde *h, const float *rows, float *out, cudaStream_t s) {
     const int64_t total = h->n_tiles * h->d_pad * kSimtTile;
     count_launch();
-    to_tiles_kernel<float><<<grid_for(total, 256), 256, 0, s>>>(rows, h->n, h->d, h->d_pad, h->n_tiles, out);
+    to_tiles_kernel<float, false><<<grid_for(total, 256), 256, 0, s>>>(rows, h->n, h->d, h->d_pad, h->n_tiles, out);
     STAG_CUDA_TRY(cudaGetLastError());
     return 0;
 }

@@ -1838,7 +1838,7 @@ int tc_reserve(stag_kde *h, int64_t m, int tiles_per_unit) {
             STAG_CUDA_TRY(dev_malloc(&tc->gbuf, group_scratch_bytes(m, tc->T, tc->BN, nullptr, nullptr)));
             tc->gbuf_m = m;
         }
-        rc = ensure_qt(h, ceil_div(m, kSimtTile) * h->d_pad * kSimtTile);
+        rc = ensure_qt(h, ceil_div(m, kSimtTile) * h->d_pad * kSimtTile * 2);
     }
     if (!rc) rc = ensure_partials(h, sp * m);
     if (rc) return rc;

@@ -7,6 +7,7 @@
 // (the logistic form in the bounded variable t equals the definition and cannot
 // overflow). d2 is the squared distance, r = sqrt(d2).
 #pragma once
+#include "f32x2.cuh"
 #include "stag_kde.h"
 
 namespace stagkde {
@@ -41,6 +42,23 @@ __device__ __forceinline__ float term(float negc, float d2, float shift) {
             const float den = (1.f + t) * (1.f + t);
             return __fdividef(4.f * ts, den);
         }
+    }
+}
+
+// term for a packed pair of squared distances (the Gaussian's multiply-add is packed too;
+// each half's result is that of term).
+template <int KERN>
+__device__ __forceinline__ void term2(float negc, uint64_t negc2, uint64_t d2, float shift, float &e0, float &e1) {
+    if constexpr (KERN == STAG_KDE_KERNEL_GAUSSIAN) {
+        float a0, a1;
+        f2::unpack(f2::fma(negc2, d2, f2::pack(-shift, -shift)), a0, a1);
+        e0 = ex2_approx(a0);
+        e1 = ex2_approx(a1);
+    } else {
+        float a0, a1;
+        f2::unpack(d2, a0, a1);
+        e0 = term<KERN>(negc, a0, shift);
+        e1 = term<KERN>(negc, a1, shift);
     }
 }
 
