@@ -109,7 +109,7 @@ struct stag_kde {
     double *out_dev = nullptr;
     int64_t out_cap = 0;  // bytes
     stagkde::Partials part;
-    float *xrow = nullptr;    // row-major FP32 point set for gathers (subset sums), built on first use
+    float *xrow = nullptr;    // row-major FP32 point set, rows of d_pad, for gathers (subset sums), built on first use
     void *sub_dev = nullptr;  // host subset call: device copies of offsets, indices, weights
     int64_t sub_dev_cap = 0;  // bytes
     int *flag_dev = nullptr;  // input-validation flag
@@ -137,8 +137,9 @@ int simt_prepare_points(stag_kde *h, const float *dX);  // dX: device row-major 
 int simt_query_f32(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaStream_t s,
                    int *dflag);
 int ensure_partials(stag_kde *h, int64_t entries);
-// The point set in its original order, row-major (from the plain form's tiled copy).
-int simt_points_rows(stag_kde *h, float *out, cudaStream_t s);
+// The point set in its original order, row-major with rows of `stride` (d or d_pad)
+// coordinates (from the plain form's tiled copy).
+int simt_points_rows(stag_kde *h, float *out, int64_t stride, cudaStream_t s);
 int launch_subtract(double *v, int64_t count, double one, cudaStream_t s);
 // Sizes the plain form's scratch (tiled queries, partials) for queries of up to m rows.
 int simt_reserve(stag_kde *h, int64_t m);

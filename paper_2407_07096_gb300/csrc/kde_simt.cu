@@ -578,11 +578,13 @@ int simt_reserve(stag_kde *h, int64_t m) {
     return ensure_partials(h, ceil_div(h->n_tiles, tps) * m);
 }
 
-// Tile-transposed [tile][d_pad][64] back to row-major n x d.
-__global__ void tiles_to_rows_kernel(const float *__restrict__ xt, int64_t n, int64_t d, int d_pad,
+// Tile-transposed [tile][d_pad][64] back to row-major rows of `stride` coordinates (d, or
+// d_pad with the padding).
+__global__ void tiles_to_rows_kernel(const float *__restrict__ xt, int64_t n, int64_t stride, int d_pad,
                                      float *__restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * d; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = i / d, k = i % d;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * stride;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t row = i / stride, k = i % stride;
         out[i] = xt[((row / kSimtTile) * d_pad + k) * kSimtTile + row % kSimtTile];
     }
 }
@@ -592,9 +594,9 @@ __global__ void subtract_one_kernel(double *__restrict__ v, int64_t count, doubl
         v[i] -= one;
 }
 
-int simt_points_rows(stag_kde *h, float *out, cudaStream_t s) {
+int simt_points_rows(stag_kde *h, float *out, int64_t stride, cudaStream_t s) {
     count_launch();
-    tiles_to_rows_kernel<<<grid_for(h->n * h->d, 256), 256, 0, s>>>(h->xt, h->n, h->d, h->d_pad, out);
+    tiles_to_rows_kernel<<<grid_for(h->n * stride, 256), 256, 0, s>>>(h->xt, h->n, stride, h->d_pad, out);
     STAG_CUDA_TRY(cudaGetLastError());
     return 0;
 }

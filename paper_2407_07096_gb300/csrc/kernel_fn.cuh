@@ -28,6 +28,14 @@ __device__ __forceinline__ float sqrt_approx(float x) {
     return y;
 }
 
+// v 2^de for de in [-4000, 0] on the integer pipe (ldexp's FP64 multiplications hold the
+// FP64 pipe, two lanes per SM and clock, for 16 clocks each). Results below 2^-1022 are 0.
+__device__ __forceinline__ double scale_down(double v, int de) {
+    const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
+    if (e == 0x7ff) return v;
+    return e + de > 0 ? __hiloint2double(hi + (de << 20), __double2loint(v)) : 0.0;
+}
+
 template <int KERN>
 __device__ __forceinline__ float term(float negc, float d2, float shift) {
     if constexpr (KERN == STAG_KDE_KERNEL_GAUSSIAN) {

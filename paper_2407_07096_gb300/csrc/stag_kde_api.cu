@@ -530,7 +530,7 @@ int stag_kde_degrees(stag_kde_t *h, int exclude_self, double *dOut, void *stream
     // the point set in original order, as a query batch against itself
     int rc = ensure_bytes(&h->q_dev, &h->q_dev_cap, h->n * h->d * (int64_t)sizeof(float));
     if (rc) return rc;
-    rc = simt_points_rows(h, (float *)h->q_dev, s);
+    rc = simt_points_rows(h, (float *)h->q_dev, h->d, s);
     if (rc) return rc;
     rc = run_query(h, h->q_dev, h->n, dOut, s, nullptr);
     if (rc) return rc;

@@ -163,3 +163,25 @@ def test_benchmark_size_sampled_rows():
     want = oracle.kde_subset(X, Q[rows], 0.1, sub_off, sub_idx, np.full(len(sub_idx), n / L_))
     kap = _kappa(X, Q[rows], 0.1, sub_off, sub_idx, np.ones(len(sub_idx)), "gaussian")
     _check(got[rows], want, kap, 16)
+
+
+@pytest.mark.parametrize("d", [1, 4, 15, 16, 17, 30, 33, 100])
+@pytest.mark.parametrize("m,max_len", [(1, 33), (40, 3), (700, 70)])
+def test_staged_rows_edges(d, m, max_len):
+    # chunks of 16 coordinates (partial, padded, several), lists of less than a warp's 32
+    # entries and just above, runs of empty lists, indices out of range on the device
+    import torch
+    K = _kde_cls()
+    X, Q = mixture_inputs(d + m, 500, m, d)
+    a = 1.0 / d
+    off, idx, W = _ragged(d, m, 500, max_len, empty_every=2)
+    bad = idx.copy()
+    bad[::5] = 500
+    bad[3::11] = -1
+    keep = (bad >= 0) & (bad < 500)
+    want = oracle.kde_subset(X, Q, a, off, np.where(keep, bad, 0), np.where(keep, W, 0).astype(np.float32))
+    kap = _kappa(X, Q, a, off, np.where(keep, bad, 0), np.where(keep, W, 0), "gaussian")
+    with K(X, a, form="simt_f32") as kde:
+        got = kde.query_subset_dev(torch.from_numpy(Q).cuda(), torch.from_numpy(off).cuda(),
+                                   torch.from_numpy(bad).cuda(), torch.from_numpy(W).cuda()).cpu().numpy()
+    _check(got, want, np.nan_to_num(kap), d)
