@@ -20,10 +20,12 @@
 //
 // Query: hash the queries, binary-search each table for the query's key (one thread per
 // (query, table)), then remove repeats across tables so that every query gets its
-// distinct candidates in increasing index order. Up to 2^22 points, a block takes one
-// (query, slice of at most 1572864 points) at a time, sets a bit per bucket member in a
-// shared-memory bitmap of the slice and walks it in index order (a counting pass, a
-// prefix sum over the items, a writing pass). Beyond that, every bucket member is listed
+// distinct candidates in increasing index order. Up to 1572864 points, a block takes one
+// query at a time, sets a bit per bucket member in a shared-memory bitmap of the points and
+// walks it in index order, writing the list at an offset known from the bucket sizes (one
+// pass; the compact int64 lists are written when they are fetched). Up to 2^22 points, and
+// where those offsets would take too much memory, a block takes (query, slice) items in
+// two such walks (a counting pass, a prefix sum over the items, a writing pass). Beyond that, every bucket member is listed
 // (one warp per query) and repeats are removed by a radix sort of (query << 32 | index)
 // keys and a per-query unique pass.
 #include <stdint.h>
@@ -41,16 +43,27 @@ struct stag_lsh {
     int K = 0, L = 0;
     cudaStream_t stream = nullptr;
     float *A = nullptr, *B = nullptr;  // functions: L*K x d, L*K
+    float *At = nullptr;               // the functions as [K][d][L] (the lookup's lanes are tables)
     uint64_t *keys = nullptr;          // n*L sorted keys (table id in bits 58..63)
     uint32_t *ids = nullptr;           // n*L point indices in key order
     float *X = nullptr;                // n x d points (the lookup recomputes a member's K values)
+    uint32_t *dir = nullptr;           // per table, the first entry at or above each key prefix
+    int dir_bits = 0;                  // bits of a prefix (2^dir_bits + 1 entries per table)
     uint64_t salt = 0;                 // salt of the bucket keys
     int key_bits = 58;                 // bits of a bucket key
     // query scratch (grown on demand)
     void *scratch = nullptr;
     int64_t scratch_cap = 0;
-    void *cand = nullptr;  // the last query's deduplicated candidates (int64)
+    // The last query's distinct candidates: int64 lists in query order in cand, or (raw_lists)
+    // 32-bit lists in raw at the offsets raw_off, their compact offsets in own_off, and cand
+    // filled from them when somebody wants it (cand_ready).
+    void *cand = nullptr;
     int64_t cand_cap = 0;
+    void *raw = nullptr;
+    int64_t raw_cap = 0;
+    bool raw_lists = false, cand_ready = false;
+    const int64_t *raw_off = nullptr, *own_off = nullptr;  // (in scratch)
+    int64_t last_m = 0;
     void *host_q = nullptr;  // host API: device copies of Q and the offsets
     int64_t host_q_cap = 0;
     int64_t last_total = 0;  // size of the kept candidate lists (device query)
@@ -66,11 +79,8 @@ constexpr int kHashRows = 8;   // rows per block
 constexpr int kKeyShift = 58;  // table id above the 58-bit bucket key
 
 // h = floor((<x, a> + b) / 4) in FP32, fixed order, saturated to int32 (the conversion
-// with rounding toward -inf saturates). One function of one row, the same operations as
-// the tiled kernel below.
-__device__ __forceinline__ int32_t hash_one(const float *__restrict__ x, const float *__restrict__ a, float b, int d) {
-    float s = 0.f;
-    for (int k = 0; k < d; ++k) s = __fmaf_rn(x[k], a[k], s);
+// with rounding toward -inf saturates).
+__device__ __forceinline__ int32_t hash_of_dot(float s, float b) {
     return __float2int_rd(__fmul_rn(__fadd_rn(s, b), 0.25f));
 }
 
@@ -91,8 +101,7 @@ lsh_hash_kernel(const float *__restrict__ X, int64_t n, int d, const float *__re
     const float *x = X + i * d;
     float s = 0.f;
     for (int k = 0; k < d; ++k) s = __fmaf_rn(x[k], sa[k * kHashFns + lane], s);
-    const float v = __fmul_rn(__fadd_rn(s, B[f0 + lane]), 0.25f);
-    H[i * nf + f0 + lane] = __float2int_rd(v);
+    H[i * nf + f0 + lane] = hash_of_dot(s, B[f0 + lane]);
 }
 
 // key_bits-bit key (at most 58) of K hash values: a SplitMix64-style mix of each value
@@ -151,15 +160,43 @@ __device__ __forceinline__ int64_t lower_bound(const uint64_t *a, int64_t lo, in
 // The table view the lookup needs.
 struct LshTables {
     const uint64_t *keys;
-    const uint32_t *ids;
-    const float *X, *A, *B;  // points and functions (L*K x d), offsets
+    const uint32_t *ids, *dir;
+    const float *X, *At, *B;  // points; functions, coordinate-major [K][d][L]; offsets
     int64_t n;
-    int d, K, L, key_bits;
+    int d, K, L, key_bits, dir_bits;
     uint64_t salt;
 };
 
+// At[(k * d + c) * L + l] = A[(l * K + k) * d + c].
+__global__ void lsh_transpose_functions_kernel(const float *__restrict__ A, int d, int K, int L, float *__restrict__ At) {
+    const int64_t total = (int64_t)L * K * d;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t l = i % L, c = (i / L) % d, k = i / L / d;
+        At[i] = A[(l * K + k) * d + c];
+    }
+}
+
+// dir[l * (2^bits + 1) + t] = number of table l's entries whose key prefix is below t.
+__global__ void lsh_directory_kernel(const uint64_t *__restrict__ keys, int64_t n, int L, int key_bits, int bits,
+                                     uint32_t *__restrict__ dir) {
+    const int64_t total = n * L, stride = ((int64_t)1 << bits) + 1;
+    const uint64_t mask = (1ull << kKeyShift) - 1ull;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t l = e / n, i = e - l * n;
+        const int64_t t = (int64_t)((keys[e] & mask) >> (key_bits - bits));
+        const int64_t before = i ? (int64_t)((keys[e - 1] & mask) >> (key_bits - bits)) : -1;
+        uint32_t *d = dir + l * stride;
+        for (int64_t u = before + 1; u <= t; ++u) d[u] = (uint32_t)i;
+        if (i == n - 1)
+            for (int64_t u = t + 1; u < stride; ++u) d[u] = (uint32_t)n;
+    }
+}
+
 // Per (query, table): the bucket's range in the sorted arrays (empty unless the first
-// member's K values equal the query's: exact membership); per query: the total.
+// member's K values equal the query's: exact membership); per query: the total. Bound by the
+// its scattered loads: n = 1e6, L = 50, 1e4 queries: 469 us with two binary searches over the
+// whole table and the tuple check reading rows of A per lane, 311 with the key directory,
+// 130 with the functions coordinate-major (a warp's lanes are consecutive tables).
 __global__ void lsh_lookup_kernel(const int32_t *__restrict__ HQ, int64_t m, LshTables t, int64_t *__restrict__ range,
                                   unsigned long long *__restrict__ count) {
     const int K = t.K, L = t.L;
@@ -168,17 +205,34 @@ __global__ void lsh_lookup_kernel(const int32_t *__restrict__ HQ, int64_t m, Lsh
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = e / L, l = e % L;
         const int32_t *hq = HQ + j * (int64_t)K * L + l * K;
-        const uint64_t key = ((uint64_t)l << kKeyShift) | bucket_key(hq, K, t.salt, t.key_bits);
-        const int64_t lo = lower_bound(t.keys, l * n, (l + 1) * n, key);
-        int64_t hi = lower_bound(t.keys, lo, (l + 1) * n, key + 1);
+        const uint64_t bk = bucket_key(hq, K, t.salt, t.key_bits);
+        const uint64_t key = ((uint64_t)l << kKeyShift) | bk;
+        // the directory leaves the entries of one key prefix (about 16 of them, or one large
+        // bucket) to the binary searches
+        const uint32_t *dir = t.dir + l * (((int64_t)1 << t.dir_bits) + 1) + (bk >> (t.key_bits - t.dir_bits));
+        const int64_t d0 = l * n + dir[0], d1 = l * n + dir[1];
+        const int64_t lo = lower_bound(t.keys, d0, d1, key);
+        int64_t hi = lower_bound(t.keys, lo, d1, key + 1);
         if (hi > lo) {
+            // eight functions at a time, the point's coordinates read once for all of them (the
+            // operations of the hash kernel, in its order)
             const float *x = t.X + (int64_t)t.ids[lo] * t.d;
-            for (int k = 0; k < K; ++k) {
-                const int64_t f = l * K + k;
-                if (hash_one(x, t.A + f * t.d, t.B[f], t.d) != hq[k]) {
-                    hi = lo;  // another tuple with the same key: not this query's bucket
-                    break;
+            const int64_t plane = (int64_t)t.d * L;  // one function index's coordinates
+            for (int k0 = 0; k0 < K && hi > lo; k0 += 8) {
+                const int kn = min(8, K - k0);
+                const float *a = t.At + k0 * plane + l;
+                float acc[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) acc[u] = 0.f;
+                for (int c = 0; c < t.d; ++c, a += L) {
+                    const float xc = x[c];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (u < kn) acc[u] = __fmaf_rn(xc, a[u * plane], acc[u]);
                 }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)  // another tuple with the same key: not this query's bucket
+                    if (u < kn && hash_of_dot(acc[u], t.B[l * K + k0 + u]) != hq[k0 + u]) hi = lo;
             }
         }
         range[2 * e] = lo;
@@ -187,18 +241,21 @@ __global__ void lsh_lookup_kernel(const int32_t *__restrict__ HQ, int64_t m, Lsh
     }
 }
 
-// out[0] = 0, out[j + 1] = sum of in[0..j] (one block; m is modest: one entry per query)
-__global__ void scan_i64_kernel(const unsigned long long *__restrict__ in, int64_t m, int64_t *__restrict__ out) {
+// out[0] = 0, out[j + 1] = sum of min(in[0..j], most), and the same into out2 unless it is
+// NULL (one block; m is modest: one entry per query)
+__global__ void scan_i64_kernel(const unsigned long long *__restrict__ in, int64_t m, int64_t *__restrict__ out,
+                                int64_t *__restrict__ out2 = nullptr, unsigned long long most = ~0ull) {
     __shared__ long long s[1024];
     __shared__ long long carry;
     if (threadIdx.x == 0) {
         carry = 0;
         out[0] = 0;
+        if (out2) out2[0] = 0;
     }
     __syncthreads();
     for (int64_t base = 0; base < m; base += 1024) {
         const int64_t i = base + threadIdx.x;
-        long long v = i < m ? (long long)in[i] : 0;
+        long long v = i < m ? (long long)min(in[i], most) : 0;
         s[threadIdx.x] = v;
         __syncthreads();
         for (int off = 1; off < 1024; off <<= 1) {
@@ -207,7 +264,10 @@ __global__ void scan_i64_kernel(const unsigned long long *__restrict__ in, int64
             s[threadIdx.x] += t;
             __syncthreads();
         }
-        if (i < m) out[i + 1] = carry + s[threadIdx.x];
+        if (i < m) {
+            out[i + 1] = carry + s[threadIdx.x];
+            if (out2) out2[i + 1] = carry + s[threadIdx.x];
+        }
         __syncthreads();
         if (threadIdx.x == 1023) carry += s[1023];
         __syncthreads();
@@ -267,8 +327,9 @@ int64_t bitmap_slice_words(int64_t n) { return (bitmap_words(n) + bitmap_slices(
 bool bitmap_fits(int64_t n) { return n <= kBmMaxPoints; }
 
 // Exclusive prefix sum of c over the block's threads (thread order); *total gets the sum.
+template <int kThreads = kBmThreads>
 __device__ __forceinline__ int block_exclusive_scan(int c, int *warp_sums, int *total) {
-    constexpr int kWarps = kBmThreads >> 5;
+    constexpr int kWarps = kThreads >> 5;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int inc = c;
 #pragma unroll
@@ -360,6 +421,162 @@ lsh_bitmap_kernel(const int64_t *__restrict__ range, int64_t m, int L, const uin
     }
 }
 
+// The same in one pass for up to kMaxSliceWords * 32 points: the distinct candidates of
+// query j go, increasing, to raw[raw_off[j] ..] as 32-bit indices (raw_off from the bucket
+// sizes, an upper bound), their number to ucount[j]; lsh_expand_kernel later writes the
+// compact int64 lists. The two-pass kernel above builds every bitmap twice and reads all of
+// its words three times.
+// What bounds it is the chain of dependent steps per query (ranges, members, bits, walk),
+// so each step is short: the members of all tables are one flat list over the threads
+// (about seven each, all loads in flight; one warp per table left half of the warps with
+// two tables and the loads in turn), the next query's ranges are loaded meanwhile, and with
+// kSum a summary bitmap (one bit per word) lets the walk visit only the words that hold
+// something. kSum pays above 2^17 points (several blocks of 256 threads per SM without it).
+// Measured, n = 1e6, L = 50, 1e4 queries (7e7 members, 3.9e7 distinct): 431 us, and 109 to
+// expand, against 334 + 678 for the two passes and ~90 for the copy of their lists. Loading
+// the next query's members during the walk made no difference there (the walk and the bits
+// are bound by issue: about 10k of 13k clocks per query) and 24 % at n = 1e5.
+template <int kThreads, bool kSum>
+__global__ void __launch_bounds__(kThreads)
+lsh_bitmap1_kernel(const int64_t *__restrict__ range, int64_t m, int L, const uint32_t *__restrict__ ids, int words,
+                   const int64_t *__restrict__ raw_off, int64_t raw_stride, uint32_t *__restrict__ raw,
+                   unsigned long long *__restrict__ ucount) {
+    extern __shared__ uint32_t bm[];  // [words] bitmap, then (kSum) one bit per word
+    __shared__ int64_t slo[2][64];
+    __shared__ int pref[2][65];
+    __shared__ int warp_sums[kThreads / 32];
+    constexpr int U = 8;  // members per thread loaded ahead
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int nsum = kSum ? (words + 31) / 32 : 0;
+    uint32_t *sum = bm + words;
+    for (int w = tid; w < words + nsum; w += kThreads) bm[w] = 0u;
+    // warp 0: ranges of tables lane and lane + 32 of an item, and their exclusive prefix
+    int64_t a0 = 0, a1 = 0, b0 = 0, b1 = 0;
+    auto fetch = [&](int64_t j) {
+        a0 = a1 = b0 = b1 = 0;
+        if (j < m) {
+            const int64_t *r = range + 2 * j * L;
+            if (lane < L) {
+                a0 = r[2 * lane];
+                a1 = r[2 * lane + 1];
+            }
+            if (lane + 32 < L) {
+                b0 = r[2 * lane + 64];
+                b1 = r[2 * lane + 65];
+            }
+        }
+    };
+    auto publish = [&](int buf) {
+        const int ca = (int)(a1 - a0), cb = (int)(b1 - b0);
+        int ia = ca, ib = cb;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, ia, o), y = __shfl_up_sync(0xffffffffu, ib, o);
+            if (lane >= o) {
+                ia += x;
+                ib += y;
+            }
+        }
+        const int half = __shfl_sync(0xffffffffu, ia, 31);
+        slo[buf][lane] = a0;
+        slo[buf][lane + 32] = b0;
+        pref[buf][lane] = ia - ca;
+        pref[buf][lane + 32] = half + ib - cb;
+        if (lane == 31) pref[buf][64] = half + ib;
+    };
+    // member f of the item in buffer buf, all ones past its end (indices are below 2^32 - 1)
+    auto member = [&](int buf, int f) -> uint32_t {
+        if (f >= pref[buf][64]) return 0xffffffffu;
+        int t = 0;  // the last table whose members start at or before f
+#pragma unroll
+        for (int step = 32; step; step >>= 1)
+            if (pref[buf][t + step] <= f) t += step;
+        return ids[slo[buf][t] + (f - pref[buf][t])];
+    };
+    auto mark = [&](uint32_t i) {
+        if (i != 0xffffffffu) {
+            const uint32_t old = atomicOr(&bm[i >> 5], 1u << (i & 31));
+            if (kSum && old == 0u) atomicOr(&sum[i >> 10], 1u << ((i >> 5) & 31));
+        }
+    };
+    if (tid < 32) {
+        fetch(blockIdx.x);
+        publish(0);
+        fetch(blockIdx.x + (int64_t)gridDim.x);
+    }
+    __syncthreads();
+    uint32_t iv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) iv[u] = member(0, tid + u * kThreads);
+    int buf = 0;
+    for (int64_t j = blockIdx.x; j < m; j += gridDim.x, buf ^= 1) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) mark(iv[u]);
+        for (int f = tid + U * kThreads; f < pref[buf][64]; f += kThreads) mark(member(buf, f));
+        if (tid < 32) publish(buf ^ 1);
+        __syncthreads();
+        // the next item's first members are on their way while this one's words are walked
+        if (tid < 32) fetch(j + 2 * (int64_t)gridDim.x);
+#pragma unroll
+        for (int u = 0; u < U; ++u) iv[u] = member(buf ^ 1, tid + u * kThreads);
+        // this thread's words: all of [w0, w1), or those marked in its summary words
+        const int per = ((kSum ? nsum : words) + kThreads - 1) / kThreads;
+        const int w0 = min(kSum ? nsum : words, tid * per), w1 = min(kSum ? nsum : words, w0 + per);
+        int c = 0;
+        for (int w = w0; w < w1; ++w) {
+            if (kSum) {
+                for (uint32_t v = sum[w]; v; v &= v - 1u) c += __popc(bm[w * 32 + __ffs(v) - 1]);
+            } else {
+                c += __popc(bm[w]);
+            }
+        }
+        int total = 0;
+        const int before = block_exclusive_scan<kThreads>(c, warp_sums, &total);
+        uint32_t *dst = raw + (raw_off ? raw_off[j] : j * raw_stride) + before;
+        auto emit = [&](int w) {
+            for (uint32_t v = bm[w]; v; v &= v - 1u) *dst++ = (uint32_t)w * 32u + (uint32_t)(__ffs(v) - 1);
+            bm[w] = 0u;
+        };
+        for (int w = w0; w < w1; ++w) {
+            if (kSum) {
+                for (uint32_t v = sum[w]; v; v &= v - 1u) emit(w * 32 + __ffs(v) - 1);
+                sum[w] = 0u;
+            } else {
+                emit(w);
+            }
+        }
+        if (tid == 0) ucount[j] = (unsigned long long)total;
+        __syncthreads();  // cleared; this item's prefix and the scan scratch are free again
+    }
+}
+
+// out[off[j] + i] = raw[r(j) + i], r(j) = raw_off[j], or j * raw_stride: a warp takes 1024 consecutive outputs at a time,
+// finds their first query and walks on from there.
+__global__ void __launch_bounds__(256)
+lsh_expand_kernel(const uint32_t *__restrict__ raw, const int64_t *__restrict__ raw_off, int64_t raw_stride,
+                  const int64_t *__restrict__ off, int64_t m, int64_t total, int64_t *__restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t s = (blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5)) * 1024; s < total;
+         s += warps * 1024) {
+        const int64_t end = min(total, s + 1024);
+        int64_t lo = 0, hi = m - 1;  // the last query that starts at or before s
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (off[mid] <= s)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        for (int64_t p = s, j = lo; p < end; ++j) {
+            const int64_t q1 = min(end, off[j + 1]);
+            const uint32_t *src = raw + (raw_off ? raw_off[j] : j * raw_stride) - off[j];
+            for (int64_t i = p + lane; i < q1; i += 32) out[i] = (int64_t)src[i];
+            p = max(p, q1);
+        }
+    }
+}
+
 // dOff[j] = item_off[j * slices] for j = 0..m (a query's list starts at its first slice).
 __global__ void lsh_item_to_query_off_kernel(const int64_t *__restrict__ item_off, int64_t m, int64_t slices,
                                              int64_t *__restrict__ dOff) {
@@ -408,10 +625,99 @@ int bits_for(int64_t v) {
 }
 
 LshTables tables_of(const stag_lsh *h) {
-    return LshTables{h->keys, h->ids, h->X, h->A, h->B, h->n, (int)h->d, h->K, h->L, h->key_bits, h->salt};
+    return LshTables{h->keys, h->ids, h->dir, h->X, h->At, h->B, h->n, (int)h->d, h->K, h->L, h->key_bits, h->dir_bits, h->salt};
 }
 
-// The bitmap path of lsh_run: bucket ranges, distinct counts per (query, slice), their
+// One pass over the bitmaps: bucket ranges and sizes, their prefix sum, the 32-bit lists at
+// those offsets, the compact offsets. Taken while the upper bounds fit kMaxRawBytes (they
+// exceed the lists by the members that several tables share); *done says whether it was.
+// Synchronises the stream.
+constexpr int64_t kMaxRawBytes = (int64_t)4 << 30;
+constexpr int64_t kFixedRawBytes = (int64_t)64 << 20;
+constexpr int64_t kSumPoints = (int64_t)1 << 17;  // above: summary bitmap, wider blocks
+
+template <int kThreads, bool kSum>
+int launch_bitmap1(const stag_lsh *h, const int64_t *range, int64_t m, unsigned long long *ucount, int sms,
+                   cudaStream_t s) {
+    auto kern = lsh_bitmap1_kernel<kThreads, kSum>;
+    const int words = (int)bitmap_words(h->n);
+    const int smem = (words + (kSum ? (words + 31) / 32 : 0)) * 4;
+    constexpr int kMost = (int)((kSum ? kMaxSliceWords + (kMaxSliceWords + 31) / 32 : kSumPoints / 32) * 4);
+    static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+    STAG_CUDA_TRY(attr);
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(m, (int64_t)sms * (2048 / kThreads)));
+    count_launch();
+    kern<<<grid, kThreads, smem, s>>>(range, m, h->L, h->ids, words, h->raw_off, h->n, (uint32_t *)h->raw, ucount);
+    STAG_CUDA_TRY(cudaGetLastError());
+    return 0;
+}
+
+int lsh_run_bitmap1(stag_lsh *h, const int32_t *HQ, int64_t *range, unsigned long long *count, int64_t *raw_off,
+                    int64_t *own_off, int64_t m, int64_t *dOff, cudaStream_t s, int64_t *total, bool *done) {
+    *done = false;
+    // a small batch: n entries of room for every query, so that no sizes have to be known
+    const bool fixed = m * h->n * 4 <= kFixedRawBytes;
+    if (!fixed) STAG_CUDA_TRY(cudaMemsetAsync(count, 0, m * 8, s));
+    count_launch();
+    lsh_lookup_kernel<<<grid_for_elems(m * h->L, 256), 256, 0, s>>>(HQ, m, tables_of(h), range, fixed ? nullptr : count);
+    STAG_CUDA_TRY(cudaGetLastError());
+    int64_t R = m * h->n;
+    if (!fixed) {
+        count_launch();
+        scan_i64_kernel<<<1, 1024, 0, s>>>(count, m, raw_off, nullptr, (unsigned long long)h->n);
+        STAG_CUDA_TRY(cudaGetLastError());
+        STAG_CUDA_TRY(cudaMemcpyAsync(&R, raw_off + m, 8, cudaMemcpyDeviceToHost, s));
+        STAG_CUDA_TRY(cudaStreamSynchronize(s));
+        if (R * 4 > kMaxRawBytes) return 0;
+    }
+    int rc = grow(&h->raw, &h->raw_cap, std::max<int64_t>(R, 1) * 4);
+    if (rc) return rc;
+    int sms = 0;
+    STAG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    h->raw_off = fixed ? nullptr : raw_off;
+    if (h->n <= kSumPoints)
+        rc = launch_bitmap1<256, false>(h, range, m, count, sms, s);
+    else if (bitmap_words(h->n) <= 27648)  // two blocks' bitmaps fit one SM
+        rc = launch_bitmap1<512, true>(h, range, m, count, sms, s);
+    else
+        rc = launch_bitmap1<1024, true>(h, range, m, count, sms, s);
+    if (rc) return rc;
+    count_launch();
+    scan_i64_kernel<<<1, 1024, 0, s>>>(count, m, own_off, dOff);
+    STAG_CUDA_TRY(cudaGetLastError());
+    STAG_CUDA_TRY(cudaMemcpyAsync(total, own_off + m, 8, cudaMemcpyDeviceToHost, s));
+    STAG_CUDA_TRY(cudaStreamSynchronize(s));
+    h->own_off = own_off;
+    h->last_m = m;
+    h->raw_lists = true;
+    *done = true;
+    return 0;
+}
+
+// Writes the kept lists (int64, query order) to out (device) on stream s.
+int lsh_write_lists(stag_lsh *h, int64_t total, int64_t *out, cudaStream_t s) {
+    if (total == 0) return 0;
+    if (!h->raw_lists) {
+        STAG_CUDA_TRY(cudaMemcpyAsync(out, h->cand, total * 8, cudaMemcpyDeviceToDevice, s));
+        return 0;
+    }
+    count_launch();
+    lsh_expand_kernel<<<grid_for_elems(ceil_div(total, 1024) * 32, 256), 256, 0, s>>>(
+        (const uint32_t *)h->raw, h->raw_off, h->n, h->own_off, h->last_m, total, out);
+    STAG_CUDA_TRY(cudaGetLastError());
+    return 0;
+}
+
+// The kept lists in h->cand (for copies to the host).
+int lsh_need_cand(stag_lsh *h, int64_t total, cudaStream_t s) {
+    if (!h->raw_lists || h->cand_ready) return 0;
+    int rc = grow(&h->cand, &h->cand_cap, std::max<int64_t>(total, 1) * 8);
+    if (!rc) rc = lsh_write_lists(h, total, (int64_t *)h->cand, s);
+    if (!rc) h->cand_ready = true;
+    return rc;
+}
+
+// The two-pass bitmap path of lsh_run: bucket ranges, distinct counts per (query, slice), their
 // prefix sum, the lists, and the per-query offsets. Synchronises the stream.
 int lsh_run_bitmap(stag_lsh *h, const int32_t *HQ, int64_t *range, int64_t m, int64_t *dOff, cudaStream_t s,
                    int64_t *total) {
@@ -469,10 +775,12 @@ int lsh_run_bitmap(stag_lsh *h, const int32_t *HQ, int64_t *range, int64_t m, in
 int lsh_run(stag_lsh *h, const float *dQ, int64_t m, int64_t *dOff, cudaStream_t s, int64_t *total) {
     const int L = h->L, K = h->K;
     const int64_t nf = (int64_t)K * L;
-    // scratch: HQ (m * nf int32) | range (m * L * 2 int64) | count (m u64) | raw_off (m + 1 int64)
+    // scratch: HQ (m * nf int32) | range (m * L * 2 int64) | count (m u64) | raw_off, own_off
+    // (m + 1 int64 each)
     const int64_t b_hq = round_up(m * nf * 4, 256), b_rng = round_up(m * L * 16, 256);
     const int64_t b_cnt = round_up(m * 8, 256), b_off = round_up((m + 1) * 8, 256);
-    int rc = grow(&h->scratch, &h->scratch_cap, b_hq + b_rng + b_cnt + b_off);
+    int rc = grow(&h->scratch, &h->scratch_cap, b_hq + b_rng + b_cnt + 2 * b_off);
+    h->raw_lists = h->cand_ready = false;
     if (rc) return rc;
     char *base = (char *)h->scratch;
     int32_t *HQ = (int32_t *)base;
@@ -481,6 +789,12 @@ int lsh_run(stag_lsh *h, const float *dQ, int64_t m, int64_t *dOff, cudaStream_t
     int64_t *raw_off = (int64_t *)(base + b_hq + b_rng + b_cnt);
     rc = launch_hash(h, dQ, m, HQ, s);
     if (rc) return rc;
+    if (bitmap_slices(h->n) == 1) {
+        bool done = false;
+        rc = lsh_run_bitmap1(h, HQ, range, count, raw_off, (int64_t *)((char *)raw_off + b_off), m, dOff, s, total,
+                             &done);
+        if (rc || done) return rc;
+    }
     if (bitmap_fits(h->n)) return lsh_run_bitmap(h, HQ, range, m, dOff, s, total);
     STAG_CUDA_TRY(cudaMemsetAsync(count, 0, m * 8, s));
     count_launch(2);
@@ -559,6 +873,8 @@ void free_lsh(stag_lsh *h) {
     cudaFree(h->X);
     cudaFree(h->scratch);
     cudaFree(h->cand);
+    cudaFree(h->raw);
+    cudaFree(h->dir);
     cudaFree(h->sort_buf);
     cudaFree(h->host_q);
     if (h->stream) cudaStreamDestroy(h->stream);
@@ -616,7 +932,7 @@ stag_lsh_t *stag_lsh_create(const float *X, int64_t n, int64_t d, int K, int L, 
         cudaFree(dbad);
     };
     const int64_t nl = n * L;
-    if ((e = dev_malloc(&h->A, nf * d * 4)) != cudaSuccess || (e = dev_malloc(&h->B, nf * 4)) != cudaSuccess ||
+    if ((e = dev_malloc(&h->A, 2 * nf * d * 4)) != cudaSuccess || (e = dev_malloc(&h->B, nf * 4)) != cudaSuccess ||
         (e = dev_malloc(&h->keys, nl * 8)) != cudaSuccess || (e = dev_malloc(&h->ids, nl * 4)) != cudaSuccess ||
         (e = dev_malloc(&h->X, n * d * 4)) != cudaSuccess || (e = dev_malloc(&H, n * nf * 4)) != cudaSuccess ||
         (e = dev_malloc(&sortb, nl * 12 + radix_sort_hist_entries(nl) * 4)) != cudaSuccess ||
@@ -635,6 +951,9 @@ stag_lsh_t *stag_lsh_create(const float *X, int64_t n, int64_t d, int K, int L, 
         cleanup();
         return (cuda_fail(e, "cudaMemcpy (LSH inputs)"), bail(0));
     }
+    h->At = h->A + nf * d;
+    count_launch();
+    lsh_transpose_functions_kernel<<<grid_for_elems(nf * d, 256), 256, 0, s>>>(h->A, (int)d, K, L, h->At);
     int rc = launch_hash(h, dX, n, H, s);
     // keys, sort, and the check that no key is shared by two different K-tuples; on a
     // shared key the tables are rebuilt with the next salt
@@ -660,6 +979,19 @@ stag_lsh_t *stag_lsh_create(const float *X, int64_t n, int64_t d, int K, int L, 
             break;
         }
         clean = bad == 0;
+    }
+    if (!rc && clean) {
+        // prefixes of about 16 entries each, at most 2^16 of them
+        while (h->dir_bits < std::min(16, h->key_bits) && ((int64_t)16 << h->dir_bits) < n) ++h->dir_bits;
+        e = dev_malloc(&h->dir, L * (((int64_t)1 << h->dir_bits) + 1) * sizeof(uint32_t));
+        if (e == cudaSuccess) {
+            count_launch();
+            lsh_directory_kernel<<<grid_for_elems(nl, 256), 256, 0, s>>>(h->keys, n, L, h->key_bits, h->dir_bits,
+                                                                        h->dir);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) rc = cuda_fail(e, "LSH key directory");
     }
     if (!rc && !clean) rc = fail(STAG_KDE_EUNSUPPORTED, "LSH tables: every salt left two K-tuples sharing a key");
     cleanup();
@@ -691,9 +1023,7 @@ int stag_lsh_query_dev(stag_lsh_t *h, const float *dQ, int64_t m, int64_t *dOff,
     int rc = lsh_run(h, dQ, m, dOff, s, total);
     if (rc) return rc;
     h->last_total = *total;
-    if (dIdx && cap >= *total && *total > 0)
-        STAG_CUDA_TRY(cudaMemcpyAsync(dIdx, h->cand, *total * 8, cudaMemcpyDeviceToDevice, s));
-    return 0;
+    return dIdx && cap >= *total ? lsh_write_lists(h, *total, dIdx, s) : 0;
 }
 
 int stag_lsh_fetch_dev(stag_lsh_t *h, int64_t *dIdx, int64_t cap, void *stream) {
@@ -702,8 +1032,7 @@ int stag_lsh_fetch_dev(stag_lsh_t *h, int64_t *dIdx, int64_t cap, void *stream) 
     if (!dIdx || cap < h->last_total) return fail(STAG_KDE_EINVAL, "dIdx is NULL or cap is below the list size");
     Guard g(h->device);
     if (!g.ok) return fail(STAG_KDE_ECUDA, "cudaSetDevice failed");
-    STAG_CUDA_TRY(cudaMemcpyAsync(dIdx, h->cand, h->last_total * 8, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
-    return 0;
+    return lsh_write_lists(h, h->last_total, dIdx, (cudaStream_t)stream);
 }
 
 int stag_lsh_query(stag_lsh_t *h, const float *Q, int64_t m, int64_t *off, int64_t *idx, int64_t cap,
@@ -729,6 +1058,10 @@ int stag_lsh_query(stag_lsh_t *h, const float *Q, int64_t m, int64_t *off, int64
     if (rc) return rc;
     h->last_total = *total;
     STAG_CUDA_TRY(cudaMemcpyAsync(off, dOff, (m + 1) * 8, cudaMemcpyDeviceToHost, s));
+    if (idx && cap >= *total && *total > 0 && (rc = lsh_need_cand(h, *total, s))) {
+        cudaStreamSynchronize(s);
+        return rc;
+    }
     if (idx && cap >= *total && *total > 0)
         STAG_CUDA_TRY(cudaMemcpyAsync(idx, h->cand, *total * 8, cudaMemcpyDeviceToHost, s));
     STAG_CUDA_TRY(cudaStreamSynchronize(s));
@@ -741,6 +1074,8 @@ int stag_lsh_fetch(stag_lsh_t *h, int64_t *idx, int64_t cap) {
     if (!idx || cap < h->last_total) return fail(STAG_KDE_EINVAL, "idx is NULL or cap is below the list size");
     Guard g(h->device);
     if (!g.ok) return fail(STAG_KDE_ECUDA, "cudaSetDevice failed");
+    int rc = lsh_need_cand(h, h->last_total, h->stream);
+    if (rc) return rc;
     STAG_CUDA_TRY(cudaMemcpyAsync(idx, h->cand, h->last_total * 8, cudaMemcpyDeviceToHost, h->stream));
     STAG_CUDA_TRY(cudaStreamSynchronize(h->stream));
     return 0;

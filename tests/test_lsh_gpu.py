@@ -199,3 +199,19 @@ def test_membership_is_exact_when_keys_collide(monkeypatch):
     # would have matched a bucket (distinct tuples per table vs 4096 keys)
     tuples = sum(len({tuple(r) for r in HX[:, l * 3:(l + 1) * 3]}) for l in range(8))
     assert tuples * len(far) / 4096 > 100
+
+
+@pytest.mark.parametrize("n,m", [(5, 3), (17, 40), (131072, 2), (131073, 200), (884000, 2), (890000, 30)])
+def test_one_pass_lists_at_their_limits(n, m):
+    # key directories of 0 and more bits; with and without the summary bitmap, every block
+    # size, lists at fixed and at measured offsets; both ways to fetch them
+    import torch
+    r = np.random.default_rng(n)
+    X = (r.standard_normal((n, 3)) * 6).astype(np.float32)
+    Q = np.concatenate([X[r.integers(0, n, m - 1)] + np.float32(0.1), np.full((1, 3), 1e6, np.float32)])
+    with _cls()(X, 3, 7, seed=2) as lsh:
+        woff, widx = oracle.lsh_candidates(oracle.lsh_hash(X, lsh.A, lsh.B), oracle.lsh_hash(Q, lsh.A, lsh.B), 3, 7)
+        off, idx = lsh.query_dev(torch.from_numpy(Q).cuda())
+        hoff, hidx = lsh.query(Q)
+    assert np.array_equal(off.cpu().numpy(), woff) and np.array_equal(idx.cpu().numpy(), widx)
+    assert np.array_equal(hoff, woff) and np.array_equal(hidx, widx)
