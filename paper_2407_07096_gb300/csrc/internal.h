@@ -144,15 +144,7 @@ int launch_subtract(double *v, int64_t count, double one, cudaStream_t s);
 // Sizes the plain form's scratch (tiled queries, partials) for queries of up to m rows.
 int simt_reserve(stag_kde *h, int64_t m);
 int ensure_qt(stag_kde *h, int64_t floats);
-// Grouped pruned recompute (tensor-core form, d > 16): the plain form's register-tiled
-// kernel over lists of kept point tiles per query group (see kde_simt.cu), the gather of
-// rows idx[0 .. *count) into tile-transposed query tiles, and a tile-transposed copy of
-// row-major points (the k-d ordered set).
-int simt_list_launch(const stag_kde *h, const float *xt, const float *qt, const int *kept, int64_t kstride,
-                     const int *kcount, const int *item_off, const int *n_groups, int seg, int per, double *part_sum,
-                     float *part_shift, cudaStream_t s);
-int simt_gather_rows(const stag_kde *h, const float *dQ, const int *idx, const int *count, int64_t m_cap, float *qt,
-                     cudaStream_t s);
+// A tile-transposed copy of row-major points (the k-d ordered set).
 int simt_tiles_from_rows(const stag_kde *h, const float *rows, float *out, cudaStream_t s);
 int launch_check_finite_f32(const float *p, int64_t count, int *dflag, cudaStream_t s, int bit = 1);
 int launch_check_finite_f64(const double *p, int64_t count, int *dflag, cudaStream_t s);
@@ -180,10 +172,8 @@ int launch_combine(const double *part_sum, const float *part_shift, int64_t m, i
 // Stable LSD radix sort of (64-bit key, 32-bit value) pairs by key bits [0, bits); the
 // result ends in (keys, vals); hist holds radix_sort_hist_entries(n) entries (the digit
 // histogram, 256 per block of 4096 keys, and the totals of its scan chunks).
-// With dcount (device memory) only the first min(n, *dcount) entries are sorted (the
-// buffers are still sized for n; the rest is left as it is).
 int radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *ktmp, uint32_t *vtmp, uint32_t *hist, int64_t n,
-                     int bits, cudaStream_t s, const int *dcount = nullptr);
+                     int bits, cudaStream_t s);
 inline int64_t radix_sort_blocks(int64_t n) { return ceil_div(n, 4096); }
 inline int64_t radix_sort_hist_entries(int64_t n) {
     const int64_t e = 256 * radix_sort_blocks(n);
@@ -206,7 +196,15 @@ int tc_make_view(const stag_kde *base, stag_kde *view);
 int tc_operand_width(const stag_kde *h);
 int tc_epilogue_groups();
 size_t tc_inst_size();
-int tc_prep_public(stag_kde *h, const float *dQ, int64_t m, cudaStream_t s);
+// The row-term kernel over a device table of instances of one operand width (tc_fill_rt
+// fills an entry of tc_rt_size() bytes and returns its number of blocks).
+size_t tc_rt_size();
+int64_t tc_fill_rt(const stag_kde *h, const float *dQ, int64_t m, int64_t block_begin, void *inst);
+int tc_launch_rowterm(int Kp, const void *table, int n_inst, int64_t blocks, cudaStream_t s);
+// The finish kernels' instances (tc_finish.h).
+struct FinInst;
+void tc_fill_fin(const stag_kde *h, const float *dQ, int64_t m, int64_t splits, double *dOut, FinInst *f);
+int64_t tc_max_fix_items(const stag_kde *h, int64_t m);
 int64_t tc_fill_inst(const stag_kde *h, int64_t m, int tiles_per_unit, int64_t unit_begin, void *inst,
                      int64_t *splits);
 // One persistent launch for every operand width (16, 32, 64, 128 at index 0..3): table c
@@ -214,7 +212,6 @@ int64_t tc_fill_inst(const stag_kde *h, int64_t m, int tiles_per_unit, int64_t u
 // width) sizes the width's share of the CTAs.
 int tc_launch_multi(int eg, const void *const tables[4], const int n_inst[4], const int64_t units[4],
                     const double work[4], int *err, int sm_count, uint64_t wait_ns, cudaStream_t s);
-int tc_finish_public(stag_kde *h, const float *dQ, int64_t m, int64_t splits, double *dOut, cudaStream_t s);
 // kde_batch.cu
 void batch_forget_handle(stag_kde *h);
 

@@ -2,13 +2,17 @@
 //
 // Many independent instances (each a handle with its own point set, d and a, and a query
 // batch of its own size) are evaluated together:
-//   * query-side preparation of every instance;
+//   * query-side preparation: one launch per operand width over a table of instances;
 //   * ONE persistent tensor-core launch for every operand width (16/32/64/128): its CTAs
 //     are split into one range per width, sized by the width's share of the work, and each
 //     range walks the units (query tile, range of point tiles) of every instance of its
 //     width, read from a device table of instances (kde_tc.cu, TcInst, TcMulti);
-//   * per instance: FP64 combine with the error estimate and the FP32 recompute of flagged
-//     queries; instances on the plain forms run their usual path.
+//   * the FP64 combine with the error estimate, and the FP32 recompute of flagged queries,
+//     one launch each for every instance (tc_finish.cu); instances on the plain forms run
+//     their usual path on side streams.
+// (One chain of preparation, combine and twelve recompute kernels per instance made 3613
+// launches of 256 instances, and their sum the batch's time: 18.8 ms against 5 ms of
+// tensor-core work.)
 // The whole sequence is captured once into a CUDA graph and replayed on later calls with
 // the same handles, pointers and sizes. Before the first capture the autotuner times the
 // candidate (epilogue warp groups, tiles per unit) settings on the batch itself.
@@ -24,6 +28,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "tc_finish.h"
 
 namespace stagkde {
 namespace {
@@ -34,6 +39,8 @@ struct ClassLaunch {
     int64_t total_units = 0;
     double work = 0.0;        // SM time of the width's pairs, in units of one ex2 per pair
     void *d_table = nullptr;  // device copy of the instance table
+    void *d_rt = nullptr;     // the row-term kernel's table
+    int64_t rt_blocks = 0;
 };
 
 // Relative SM time of one pair at operand width Kp: the slower of one ex2 (32 per SM per
@@ -50,15 +57,21 @@ struct BatchPlan {
     std::vector<uint64_t> epochs;
     std::vector<int64_t> splits;  // tensor-core instances: splits of their work
     std::vector<ClassLaunch> classes;
+    // the finish kernels' table over all tensor-core instances, and their counters
+    void *d_fin = nullptr;
+    FinCtl *fin_ctl = nullptr;
+    int n_fin = 0, cblocks = 0, qblocks = 0, max_passes = 0, max_d_pad = 0;
+    int64_t max_items = 0;
+    bool recompute = false;
     int eg = 4;
     int tiles_per_unit = 32;
     int *d_err = nullptr;
     int *h_err = nullptr;  // pinned copy written at the end of every replay
     cudaStream_t cap = nullptr;
-    // side streams: the instances' preparation and finish chains are spread over them so
-    // that the small kernels of different instances overlap on the device (in the graph
-    // they become parallel branches between a fork and a join event)
-    static constexpr int kSide = 32;
+    // side streams: one per operand width for the row terms, the rest for instances on the
+    // plain forms (in the graph they become parallel branches between fork and join events)
+    static constexpr int kSide = 16;
+    static constexpr int kPrep = 4;  // side streams of the row terms
     cudaStream_t side[kSide] = {};
     cudaEvent_t fork = nullptr, joined[kSide] = {};
     cudaGraph_t graph = nullptr;
@@ -74,6 +87,16 @@ constexpr size_t kMaxPlans = 16;
 // reuses them, so the work split (and hence every result bit) stays the same
 std::map<std::vector<uintptr_t>, std::pair<int, int>> g_tuned;
 
+void free_tables(BatchPlan *p) {
+    for (auto &c : p->classes) {
+        cudaFree(c.d_table);
+        cudaFree(c.d_rt);
+    }
+    p->classes.clear();
+    cudaFree(p->d_fin);
+    p->d_fin = nullptr;
+}
+
 void free_plan(BatchPlan *p) {
     if (!p) return;
     int prev = -1;
@@ -82,7 +105,8 @@ void free_plan(BatchPlan *p) {
     if (p->cap) cudaStreamSynchronize(p->cap);
     if (p->exec) cudaGraphExecDestroy(p->exec);
     if (p->graph) cudaGraphDestroy(p->graph);
-    for (auto &c : p->classes) cudaFree(c.d_table);
+    free_tables(p);
+    cudaFree(p->fin_ctl);
     cudaFree(p->d_err);
     if (p->h_err) cudaFreeHost(p->h_err);
     if (p->cap) cudaStreamDestroy(p->cap);
@@ -115,59 +139,89 @@ int reserve_all(BatchPlan *p) {
 
 // Instance tables per operand width (device copies), from the current scratch.
 int build_tables(BatchPlan *p) {
-    for (auto &c : p->classes) cudaFree(c.d_table);
-    p->classes.clear();
+    free_tables(p);
     p->splits.assign(p->hs.size(), 0);
-    const size_t isz = tc_inst_size();
+    const size_t isz = tc_inst_size(), rsz = tc_rt_size();
+    std::vector<FinInst> fin;
+    p->cblocks = p->qblocks = p->max_passes = p->max_d_pad = 0;
+    p->max_items = 0;
+    p->recompute = false;
     for (int Kp : {16, 32, 64, 128}) {
-        std::vector<unsigned char> host;
-        ClassLaunch cl;
+        std::vector<unsigned char> host, rt;
+        p->classes.emplace_back();
+        ClassLaunch &cl = p->classes.back();
         cl.Kp = Kp;
         for (size_t i = 0; i < p->hs.size(); ++i) {
             stag_kde *h = p->hs[i];
             if (!is_tc(h) || tc_operand_width(h) != Kp || p->ms[i] == 0) continue;
             host.resize(host.size() + isz);
+            rt.resize(rt.size() + rsz);
             const int64_t units = tc_fill_inst(h, p->ms[i], p->tiles_per_unit, cl.total_units,
                                                host.data() + host.size() - isz, &p->splits[i]);
             cl.total_units += units;
+            cl.rt_blocks += tc_fill_rt(h, (const float *)p->qs[i], p->ms[i], cl.rt_blocks, rt.data() + rt.size() - rsz);
             cl.work += (double)p->ms[i] * (double)h->n * pair_cost(Kp);
             ++cl.n_inst;
+            FinInst f;
+            int cb, qb;
+            tc_fill_fin(h, (const float *)p->qs[i], p->ms[i], p->splits[i], p->outs[i], &f);
+            fin_number(&f, h->sm_count, p->cblocks, p->qblocks, &cb, &qb);
+            p->cblocks += cb;
+            p->qblocks += qb;
+            p->max_passes = std::max(p->max_passes, f.passes);
+            p->max_d_pad = std::max(p->max_d_pad, h->d_pad);
+            p->max_items += tc_max_fix_items(h, p->ms[i]);
+            p->recompute |= f.qflag != nullptr;
+            fin.push_back(f);
         }
-        if (!cl.n_inst) continue;
+        if (!cl.n_inst) {
+            p->classes.pop_back();
+            continue;
+        }
         STAG_CUDA_TRY(dev_malloc(&cl.d_table, host.size()));
         STAG_CUDA_TRY(cudaMemcpy(cl.d_table, host.data(), host.size(), cudaMemcpyHostToDevice));
-        p->classes.push_back(cl);
+        STAG_CUDA_TRY(dev_malloc(&cl.d_rt, rt.size()));
+        STAG_CUDA_TRY(cudaMemcpy(cl.d_rt, rt.data(), rt.size(), cudaMemcpyHostToDevice));
+    }
+    p->n_fin = (int)fin.size();
+    if (p->n_fin) {
+        STAG_CUDA_TRY(dev_malloc(&p->d_fin, fin.size() * sizeof(FinInst)));
+        STAG_CUDA_TRY(cudaMemcpy(p->d_fin, fin.data(), fin.size() * sizeof(FinInst), cudaMemcpyHostToDevice));
+        if (!p->fin_ctl) STAG_CUDA_TRY(dev_malloc(&p->fin_ctl, fin_ctl_bytes(p->n_fin)));
     }
     return 0;
 }
 
-// Queues the whole batch on stream s: the instances' query preparation spread over the
-// side streams, one persistent tensor-core launch for every operand width on s, then the
-// instances' combine and recompute chains spread over the side streams again; s waits
-// for every side stream at the end (fork/join with events, so the order holds both when
-// run directly and when captured into the graph).
+// Queues the whole batch on stream s: the row terms of each operand width on a side stream
+// of its own, the instances on the plain forms on the others, one persistent tensor-core
+// launch for every operand width on s once the row terms are there, then the combine and
+// the recompute; s waits for every side stream (fork/join with events, so the order holds
+// both when run directly and when captured into the graph).
 int enqueue(BatchPlan *p, cudaStream_t s) {
     int rc = 0;
-    auto fork = [&]() -> int {
-        STAG_CUDA_TRY(cudaEventRecord(p->fork, s));
-        for (int k = 0; k < BatchPlan::kSide; ++k) STAG_CUDA_TRY(cudaStreamWaitEvent(p->side[k], p->fork, 0));
-        return 0;
-    };
-    auto join = [&]() -> int {
-        for (int k = 0; k < BatchPlan::kSide; ++k) {
+    auto join = [&](int k0, int k1) -> int {
+        for (int k = k0; k < k1; ++k) {
             STAG_CUDA_TRY(cudaEventRecord(p->joined[k], p->side[k]));
             STAG_CUDA_TRY(cudaStreamWaitEvent(s, p->joined[k], 0));
         }
         return 0;
     };
-    auto side_of = [&](size_t i) { return p->side[i % BatchPlan::kSide]; };
-    rc = fork();
+    STAG_CUDA_TRY(cudaEventRecord(p->fork, s));
+    for (int k = 0; k < BatchPlan::kSide; ++k) STAG_CUDA_TRY(cudaStreamWaitEvent(p->side[k], p->fork, 0));
+    for (size_t c = 0; c < p->classes.size() && !rc; ++c)
+        rc = tc_launch_rowterm(p->classes[c].Kp, p->classes[c].d_rt, p->classes[c].n_inst, p->classes[c].rt_blocks,
+                               p->side[c % BatchPlan::kPrep]);
+    int next = BatchPlan::kPrep;
     for (size_t i = 0; i < p->hs.size() && !rc; ++i) {
         stag_kde *h = p->hs[i];
-        if (p->ms[i] == 0) continue;
-        if (is_tc(h)) rc = tc_prep_public(h, (const float *)p->qs[i], p->ms[i], side_of(i));
+        if (p->ms[i] == 0 || is_tc(h)) continue;
+        cudaStream_t si = p->side[next];
+        next = next + 1 < BatchPlan::kSide ? next + 1 : BatchPlan::kPrep;
+        rc = h->form == STAG_KDE_FORM_SIMT_F32
+                 ? simt_query_f32(h, (const float *)p->qs[i], p->ms[i], p->outs[i], si, nullptr)
+                 : f64_query(h, (const double *)p->qs[i], p->ms[i], p->outs[i], si, nullptr);
     }
-    if (!rc) rc = join();
+    if (!rc) rc = join(0, BatchPlan::kPrep);
     if (!rc && !p->classes.empty()) {
         // one persistent launch for every width: each width's CTAs serve its table
         const void *tables[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -182,20 +236,12 @@ int enqueue(BatchPlan *p, cudaStream_t s) {
             work[w] = c.work;
         }
         rc = tc_launch_multi(p->eg, tables, n_inst, units, work, p->d_err, p->hs[0]->sm_count, p->wait_ns, s);
+        if (!rc)
+            rc = fin_launch(FinInst{}, (const FinInst *)p->d_fin, p->n_fin, p->cblocks, p->qblocks, p->max_passes,
+                            p->max_d_pad, p->max_items, p->recompute, p->fin_ctl, p->d_err, p->hs[0]->sm_count,
+                            p->wait_ns, s);
     }
-    if (!rc) rc = fork();
-    for (size_t i = 0; i < p->hs.size() && !rc; ++i) {
-        stag_kde *h = p->hs[i];
-        if (p->ms[i] == 0) continue;
-        cudaStream_t si = side_of(i);
-        if (is_tc(h))
-            rc = tc_finish_public(h, (const float *)p->qs[i], p->ms[i], p->splits[i], p->outs[i], si);
-        else if (h->form == STAG_KDE_FORM_SIMT_F32)
-            rc = simt_query_f32(h, (const float *)p->qs[i], p->ms[i], p->outs[i], si, nullptr);
-        else
-            rc = f64_query(h, (const double *)p->qs[i], p->ms[i], p->outs[i], si, nullptr);
-    }
-    if (!rc) rc = join();
+    if (!rc) rc = join(BatchPlan::kPrep, BatchPlan::kSide);
     return rc;
 }
 

@@ -38,7 +38,7 @@
 //               columns of every tile, so an accumulator is drained by all warps at once.
 // A work unit is (query tile of 128 rows, contiguous range of point tiles); the partial
 // sums per (range, query) are combined in FP64, together with a per-query error
-// estimate, by tc_combine_kernel; queries whose estimate is too large are recomputed by
+// estimate, by fin_combine_kernel (tc_finish.cu); queries whose estimate is too large are recomputed by
 // the plain FP32 form.
 // Every mbarrier wait is bounded (%globaltimer); on expiry the kernel records an error
 // code, makes the other roles stop, waits for its own copies and MMAs, frees TMEM and
@@ -58,6 +58,7 @@
 #include "internal.h"
 #include "kernel_fn.cuh"
 #include "sm100_ptx.cuh"
+#include "tc_finish.h"
 
 namespace stagkde {
 
@@ -98,10 +99,10 @@ struct TcData {
     int64_t part_w_cap = 0;
     float *xkt = nullptr;      // k-d ordered points in the plain form's tile-transposed layout
                                // (the recompute of flagged queries)
-    void *gbuf = nullptr;      // grouped-recompute scratch (GroupScratch), sized for gbuf_m rows
+    void *gbuf = nullptr;      // recompute scratch (fin_scratch_bytes), sized for gbuf_m rows
     int64_t gbuf_m = 0;
-    int *fix_idx = nullptr;    // [m_cap]: queries handed to the plain form
-    int *fix_count = nullptr;  // device counter
+    int *fix_count = nullptr;  // device: number of queries handed to the plain form
+    FinCtl *fin_ctl = nullptr; // device: the recompute's phase counters
     int *err = nullptr;        // device error code (timeouts)
     int *err_host = nullptr;   // pinned mirror
 };
@@ -110,10 +111,6 @@ namespace {
 
 constexpr int kErrTimeout = 1;
 constexpr int BM = 128;  // queries per tile (MMA M, TMEM lanes)
-// Queries whose estimated tensor-core error exceeds this are recomputed with the plain
-// FP32 form; the estimate bounds the measured error from above (ratio <= ~0.96), so the
-// queries kept stay below ~7.2e-5 against the 1e-4 tolerance.
-constexpr double kTcErrThreshold = 7.5e-5;
 }  // namespace
 
 // Epilogue warps per TMEM lane quadrant (2 or 4); STAG_KDE_TC_EG overrides the default.
@@ -157,7 +154,7 @@ struct Cfg {
     static constexpr int OFF_B = OFF_A + AB * A_BYTES;
     static constexpr int OFF_META = OFF_B + SB * B_BYTES;
     static constexpr int OFF_MERGE = OFF_META + SMETA * META_STRIDE;
-    static constexpr int OFF_BAR = OFF_MERGE + BM * 24 * (EG - 1);
+    static constexpr int OFF_BAR = OFF_MERGE + BM * 16 * (EG - 1);
     static constexpr int NBAR = 2 * SB + 2 * SMETA + 2 * AB + 2 * 4 + 3;  // 4: accumulators, at most
     static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
     static constexpr int BYTES = OFF_MISC + 64;
@@ -555,11 +552,14 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
         constexpr int STEP = C::RING ? EG / 2 : 1;
         constexpr int WCOLS = C::WCOLS;
         constexpr int NCH = WCOLS / 32;
+        // Columns whose terms share one FP32 sum: half a tile (RING) or a quarter of one,
+        // whatever EG, so that the launch settings do not change a result's bits.
+        constexpr int SUBCH = (C::RING ? BN / 2 : BN / 4) / 32;
+        static_assert(SUBCH >= 1 && NCH % SUBCH == 0, "whole sums per visit");
         const int col0 = C::RING ? half * WCOLS : grp * WCOLS;   // first point column of the visit
         static_assert(WCOLS % 32 == 0 && (EG == 2 || EG == 4), "whole 32-column chunks");
         double *msum = reinterpret_cast<double *>(smem + C::OFF_MERGE);   // [EG-1][BM]
         double *mw = msum + (EG - 1) * BM;                                 // [EG-1][BM]
-        float *mshift = reinterpret_cast<float *>(mw + (EG - 1) * BM);     // [EG-1][BM]
         uint32_t tcount = 0, ucount = 0;  // point tiles and units this CTA has passed
         bool ok = true;
         RowState st{0.f, 0.f, 0.f, 0.f};
@@ -589,6 +589,14 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
             const uint32_t taddr =
                 tmem_base + ((uint32_t)(quad * 32) << 16) + acc * C::ACC_COLS + (C::RING ? 0 : grp * WCOLS);
             uint64_t acc_a = 0, acc_b = 0;  // {0.f, 0.f}
+            auto fold = [&]() {
+                float s0, s1, s2, s3;
+                unpack2(acc_a, s0, s1);
+                unpack2(acc_b, s2, s3);
+                const float ts = (s0 + s1) + (s2 + s3);
+                kahan_add(st.ksum, st.kc, ts);
+                st.w32 = fmaf(ts, vw, st.w32);
+            };
             auto release_acc = [&]() {
                 // every TMEM column of this accumulator has been read: hand it back
                 ptx::tc_fence_before();
@@ -605,6 +613,10 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
                     ptx::reg_fence32(Da);
                     if (c + 1 == NCH) release_acc();
                     epi_chunk<kMasked>(acc_a, acc_b, Da, kk2, nb2, vcols - c * 32);
+                    if ((c + 1) % SUBCH == 0 && c + 1 < NCH) {
+                        fold();
+                        acc_a = acc_b = 0;
+                    }
                 }
             } else {
                 // software pipeline: the TMEM load of chunk c+1 is in flight while chunk c
@@ -627,6 +639,10 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
                         epi_chunk<kMasked>(acc_a, acc_b, Db, kk2, nb2, vcols - c * 32);
                     else
                         epi_chunk<kMasked>(acc_a, acc_b, Da, kk2, nb2, vcols - c * 32);
+                    if ((c + 1) % SUBCH == 0 && c + 1 < NCH) {
+                        fold();
+                        acc_a = acc_b = 0;
+                    }
                     if (c + 1 < NCH) {
                         ptx::tmem_ld_wait();
                         if (c & 1)
@@ -638,12 +654,7 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
             }
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&empty_m[ms]);
-            float s0, s1, s2, s3;
-            unpack2(acc_a, s0, s1);
-            unpack2(acc_b, s2, s3);
-            const float ts = (s0 + s1) + (s2 + s3);
-            kahan_add(st.ksum, st.kc, ts);
-            st.w32 = fmaf(ts, vw, st.w32);
+            fold();
             return true;
         };
         for (int64_t u = cta; u < total_units && ok; u += ncta) {
@@ -688,7 +699,6 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
                 }
                 msum[(grp - 1) * BM + row] = acc64;
                 mw[(grp - 1) * BM + row] = w64;
-                mshift[(grp - 1) * BM + row] = st.shift;
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(merge_full);
             } else {
@@ -697,30 +707,24 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
                     timed_out();
                     break;
                 }
-                float os[EG - 1];
                 double oa[EG - 1], ow[EG - 1];
-                float sm = st.shift;
 #pragma unroll
                 for (int g = 0; g < EG - 1; ++g) {
                     oa[g] = msum[g * BM + row];
                     ow[g] = mw[g * BM + row];
-                    os[g] = mshift[g * BM + row];
-                    sm = fmaxf(sm, os[g]);
                 }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(merge_empty);
-                const int e0 = cexp(st.shift - sm);
-                double tot = ldexp(acc64, e0), wt = ldexp(w64, e0);
+                double tot = acc64, wt = w64;  // (every group has the row's shift)
 #pragma unroll
                 for (int g = 0; g < EG - 1; ++g) {
-                    const int e = cexp(os[g] - sm);
-                    tot += ldexp(oa[g], e);
-                    wt += ldexp(ow[g], e);
+                    tot += oa[g];
+                    wt += ow[g];
                 }
                 const int64_t q = qt * BM + row;
                 if (q < I.m) {
                     I.part_sum[split * I.m + q] = tot;
-                    I.part_shift[split * I.m + q] = sm;
+                    I.part_shift[split * I.m + q] = st.shift;
                     I.part_w[split * I.m + q] = wt;
                 }
             }
@@ -969,32 +973,65 @@ struct RowTermGeo {
     static constexpr int smem_bytes(int kp) { return kp * QS * 4; }
 };
 
-template <int KP>
+// One instance of the row-term kernel (a launch serves a table of them, or one).
+struct RtInst {
+    const float *Q, *centT, *cg, *tinfo, *scales;
+    float *R, *unorm;
+    unsigned *ub;
+    __half *ahi, *alo;
+    int *qbad, *fix_count, *flag;  // flag (or NULL): bit 0 is set if a query is not finite or beyond 1e15
+    int64_t m, m_pad, T;
+    int d, tiles_per_block, qblocks, block_begin;  // qblocks = m_pad / 128
+    float c;
+};
+
+// (kTable is a template parameter because a single instance's fields are then read where
+// they are used, from constant memory, and cost no registers)
+template <int KP, bool kTable>
 __global__ void __launch_bounds__(RowTermGeo::THREADS, KP <= 16 ? 3 : 2)
-tc_rowterm_kernel(const float *__restrict__ Q, int64_t m, int64_t d, int64_t m_pad, const float *__restrict__ cent,
-                  int64_t T, int tiles_per_block, float c, float *__restrict__ R, const float *__restrict__ cg,
-                  float *__restrict__ unorm, const float *__restrict__ tinfo, unsigned *__restrict__ ub,
-                  const float *__restrict__ scales, __half *__restrict__ ahi, __half *__restrict__ alo,
-                  int *__restrict__ qbad, const float *__restrict__ centT) {
+tc_rowterm_kernel(const __grid_constant__ RtInst inst0, const RtInst *__restrict__ table, int n_inst) {
+    int which = 0;
+    if (kTable) {
+        int hi = n_inst - 1;
+        while (which < hi) {
+            const int mid = (which + hi + 1) >> 1;
+            if (table[mid].block_begin <= (int)blockIdx.x)
+                which = mid;
+            else
+                hi = mid - 1;
+        }
+    }
+    __shared__ RtInst sinst;
+    if (kTable) {
+        for (int i = threadIdx.x; i < (int)(sizeof(RtInst) / 4); i += RowTermGeo::THREADS)
+            reinterpret_cast<int *>(&sinst)[i] = reinterpret_cast<const int *>(table + which)[i];
+        __syncthreads();
+    }
+    const RtInst &I = kTable ? sinst : inst0;
+    const int64_t m = I.m, d = I.d, m_pad = I.m_pad, T = I.T;
+    const int tiles_per_block = I.tiles_per_block;
+    const float c = I.c;
+    const int block = (int)blockIdx.x - I.block_begin, by = block / I.qblocks;  // tile range
     using RG = RowTermGeo;
     constexpr int TG = RG::TG, KC = RG::KC, QS = RG::QS;
     extern __shared__ __align__(16) float sq[];              // [KP][QS]: the block's queries
     __shared__ __align__(16) uint64_t sc[KC * TG];           // [k][tile slot]: (c, c)
     __shared__ float srad[TG];
-    const int64_t q0 = (int64_t)blockIdx.x * 128;
+    const int64_t q0 = (int64_t)(block - by * I.qblocks) * 128;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (blockIdx.y == 0) {
+    if (block == 0 && tid == 0) *I.fix_count = 0;
+    if (by == 0) {
         // ||q - c_g|| and the A operand: FP16 hi/lo splits of u, zero for padding rows and
         // coordinates, stored eight coordinates (16 bytes) at a time; two threads per query
         const int r = tid >> 1, part = tid & 1;
         const int64_t q = q0 + r;
         const bool real = q < m;
         const int k0 = part * (KP / 2);
-        const double su = scales[1];
+        const double su = I.scales[1];
         float s2 = 0.f;
-        int bad = 0;
-        uint4 *dh = reinterpret_cast<uint4 *>(ahi + q * KP + k0);
-        uint4 *dl = reinterpret_cast<uint4 *>(alo + q * KP + k0);
+        int bad = 0, refused = 0;
+        uint4 *dh = reinterpret_cast<uint4 *>(I.ahi + q * KP + k0);
+        uint4 *dl = reinterpret_cast<uint4 *>(I.alo + q * KP + k0);
 #pragma unroll 1
         for (int k8 = 0; k8 < KP / 16; ++k8) {
             __align__(16) __half hv[8], lv[8];
@@ -1003,10 +1040,11 @@ tc_rowterm_kernel(const float *__restrict__ Q, int64_t m, int64_t d, int64_t m_p
                 const int k = k0 + k8 * 8 + j;
                 __half hh = __float2half_rn(0.f), ll = __float2half_rn(0.f);
                 if (real && k < d) {
-                    const float qk = Q[q * d + k];
-                    const float df = qk - cg[k];
+                    const float qk = I.Q[q * d + k];
+                    refused |= !(fabs((double)qk) <= 1e15);
+                    const float df = qk - I.cg[k];
                     s2 = fmaf(df, df, s2);
-                    const double u = ((double)qk - (double)cg[k]) * su;
+                    const double u = ((double)qk - (double)I.cg[k]) * su;
                     if (fabs(u) < 0x1p15) {
                         hh = __float2half_rn((float)u);
                         ll = __float2half_rn((float)(u - (double)__half2float(hh)));
@@ -1023,16 +1061,17 @@ tc_rowterm_kernel(const float *__restrict__ Q, int64_t m, int64_t d, int64_t m_p
         s2 += __shfl_xor_sync(0xffffffffu, s2, 1);
         bad |= __shfl_xor_sync(0xffffffffu, bad, 1);
         if (part == 0) {
-            unorm[q] = real ? sqrtf(s2) : 0.f;
-            if (bad) qbad[q] = 1;
+            I.unorm[q] = real ? sqrtf(s2) : 0.f;
+            I.qbad[q] = bad;
         }
+        if (refused && I.flag) atomicOr(I.flag, 1);
     }
     const int wq = warp & 3, wt = warp >> 2, lq = lane & 3, lt = lane >> 2;
     const int qo = wq * 32 + lq * 8;  // first of the thread's 8 queries (block-relative)
     const int to = wt * 32 + lt * 4;  // first of its 4 tiles (chunk-relative)
     // centre slots: the pairs (to, to+1) of a warp's lanes side by side, then (to+2, to+3)
     const int cs0 = wt * 32 + lt * 2, cs1 = cs0 + 16;
-    const int64_t ta = (int64_t)blockIdx.y * tiles_per_block;
+    const int64_t ta = (int64_t)by * tiles_per_block;
     const int64_t tb = min(T, ta + tiles_per_block);
     // upper bound on the exponent -c ||q - x||^2 over the tiles of this block: every x of
     // tile t lies within the tile's max radius rho_t of c_t, so
@@ -1045,7 +1084,7 @@ tc_rowterm_kernel(const float *__restrict__ Q, int64_t m, int64_t d, int64_t m_p
     for (int e = tid; e < KP * 128; e += RG::THREADS) {
         const int r = e / KP, k = e % KP;
         const int64_t q = q0 + r;
-        sq[k * QS + r] = (q < m && k < d) ? Q[q * d + k] : 0.f;
+        sq[k * QS + r] = (q < m && k < d) ? I.Q[q * d + k] : 0.f;
     }
     // Stages: (chunk of 64 tiles, block of 16 coordinates). The centres (and, at a chunk's
     // first block, the tiles' radii) of the next stage are loaded into registers while the
@@ -1061,9 +1100,9 @@ tc_rowterm_kernel(const float *__restrict__ Q, int64_t m, int64_t d, int64_t m_p
         for (int i = 0; i < PER; ++i) {
             const int e = tid + i * RG::THREADS;
             const int j = e % TG, k = e / TG;  // tile j of the chunk, coordinate kb + k
-            pv[i] = j < gn ? centT[(int64_t)(kb + k) * T + g0 + j] : 0.f;
+            pv[i] = j < gn ? I.centT[(int64_t)(kb + k) * T + g0 + j] : 0.f;
         }
-        prad = (kb == 0 && tid < gn) ? tinfo[(g0 + tid) * 4 + 1] : 0.f;
+        prad = (kb == 0 && tid < gn) ? I.tinfo[(g0 + tid) * 4 + 1] : 0.f;
     };
     if (nstages > 0) load_stage(0);
     uint64_t tot[4][4];  // [tile][query pair], packed (query 2p, 2p+1)
@@ -1128,7 +1167,7 @@ tc_rowterm_kernel(const float *__restrict__ Q, int64_t m, int64_t d, int64_t m_p
                 const float g = fmaxf(0.f, ptx::sqrt_approx(rv[i]) * (1.f - 1e-5f) - rr);
                 ubest[i] = fmaxf(ubest[i], -g * g);
             }
-            float4 *dst = reinterpret_cast<float4 *>(R + (g0 + jt) * m_pad + q0 + qo);
+            float4 *dst = reinterpret_cast<float4 *>(I.R + (g0 + jt) * m_pad + q0 + qo);
             dst[0] = make_float4(rv[0], rv[1], rv[2], rv[3]);
             dst[1] = make_float4(rv[4], rv[5], rv[6], rv[7]);
         }
@@ -1144,277 +1183,9 @@ tc_rowterm_kernel(const float *__restrict__ Q, int64_t m, int64_t d, int64_t m_p
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int64_t q = q0 + qo + i;
-            atomicMax(ub + q, float_order_bits(q < m ? ubest[i] : 0.f));
+            atomicMax(I.ub + q, float_order_bits(q < m ? ubest[i] : 0.f));
         }
     }
-}
-
-// FP32 recompute of the queries the tensor-core estimate flags, over the tiles that can
-// matter only. Per query, from the row terms R_t = c ||q - c_t||^2 and the tiles' max
-// radii rho_t (c = a log2 e, exponents in log2 units):
-//     ub_t = -(max(0, sqrt(R_t) - sqrt(c) rho_t))^2  >= every exponent -c ||q - x||^2 in tile t
-//     lb_t = -(sqrt(R_t) + sqrt(c) rho_t)^2          <= the largest exponent in tile t
-// (with a 1e-5 relative slack on sqrt(R_t) for rounding), so LB = max_t lb_t bounds the
-// row's largest term from below, and a tile with ub_t < LB - 64 holds only terms below
-// 2^-64 of it: all of them together change the sum by less than n 2^-64 relative, and
-// the tile is skipped. The others are evaluated like the plain FP32 form.
-constexpr float kPruneLog2 = 64.f;
-
-// ---------------------------------------------------------------- grouped recompute
-// The flagged queries are recomputed in groups of 64 so that every point load serves 64
-// queries (the plain form's register-tiled kernel), while the tiles that cannot matter
-// are still skipped:
-//   (1) the combine kernel flags queries and counts them per block; a scan and an ordered
-//       compaction list the flagged queries in query order, each with the bound LB of its
-//       largest exponent, its threshold LB - 64 and, as sort key, the tile holding LB;
-//   (2) a stable sort by that tile (k-d order: queries near the same points become
-//       neighbours; stable on an ordered input, so the groups are deterministic; it visits
-//       only the flagged entries) and the gather of the sorted queries, 64 per group;
-//   (3) per group, the union of its members' kept tiles (ub_t >= threshold for at least
-//       one member);
-//   (4) the list kernel (kde_simt.cu) over each group's kept tiles, in segments of `seg`
-//       tiles;
-//   (5) per query, the FP64 combine of its group's segments.
-// A member evaluates the other members' tiles too: more terms than its own bound needs,
-// never fewer.
-// Exclusive prefix sum (one block): off[0..n] from in[0..n), n = *n_dev if given, else
-// the flagged queries' group count ceil(*cnt_dev / 64) if given, else n_host; the total
-// also goes to *total_out if given.
-__global__ void __launch_bounds__(1024)
-tc_scan_kernel(const int *__restrict__ in, const int *__restrict__ cnt_dev, int n_host, int *__restrict__ off,
-               int *__restrict__ total_out) {
-    __shared__ int sdata[1024];
-    __shared__ int carry;
-    const int n = cnt_dev ? (*cnt_dev + 63) / 64 : n_host;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < n; base += 1024) {
-        const int i = base + threadIdx.x;
-        sdata[threadIdx.x] = i < n ? in[i] : 0;
-        __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {
-            const int v = threadIdx.x >= o ? sdata[threadIdx.x - o] : 0;
-            __syncthreads();
-            sdata[threadIdx.x] += v;
-            __syncthreads();
-        }
-        if (i < n) off[i + 1] = carry + sdata[threadIdx.x];
-        __syncthreads();
-        if (threadIdx.x == 1023) carry += sdata[1023];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        off[0] = 0;
-        if (total_out) *total_out = carry;
-    }
-}
-
-// The flagged queries in query order (block b's flagged queries start at boff[b]; inside
-// a block, by warp, then lane), each with the tile holding the lower bound LB of its
-// largest exponent as sort key, and its threshold LB - 64.
-__global__ void __launch_bounds__(256)
-tc_flag_compact_kernel(const int *__restrict__ qflag, const int *__restrict__ boff, int64_t m, int64_t m_pad,
-                       const float *__restrict__ R, const float *__restrict__ tinfo, int64_t T, float c,
-                       int *__restrict__ fix_idx, uint64_t *__restrict__ key, uint32_t *__restrict__ val,
-                       float *__restrict__ thr) {
-    __shared__ int wcnt[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool flag = j < m && qflag[j];
-    const unsigned mask = __ballot_sync(0xffffffffu, flag);
-    if (lane == 0) wcnt[warp] = __popc(mask);
-    __syncthreads();
-    if (!mask) return;
-    int w0 = boff[blockIdx.x];
-    for (int k = 0; k < warp; ++k) w0 += wcnt[k];
-    const float sqc = sqrtf(c);
-    if (__popc(mask) >= 8) {
-        // many flagged queries in the warp: each lane walks the tiles of its own query
-        // (eight row terms in flight; the loads of the warp's queries coalesce)
-        if (flag) {
-            float best = -INFINITY;
-            int bt = 0;
-            constexpr int U = 8;
-            for (int t0 = 0; t0 < (int)T; t0 += U) {
-                float rv[U], rho[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int t = min(t0 + u, (int)T - 1);
-                    rv[u] = R[(int64_t)t * m_pad + j];
-                    rho[u] = tinfo[(int64_t)t * 4 + 1];
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const float h2 = sqrtf(rv[u]) * (1.f + 1e-5f) + sqc * rho[u];
-                    const float lb = -h2 * h2;
-                    if (t0 + u < (int)T && lb > best) {  // ties keep the smaller tile
-                        best = lb;
-                        bt = t0 + u;
-                    }
-                }
-            }
-            const int w = w0 + __popc(mask & ((1u << lane) - 1u));
-            fix_idx[w] = (int)j;
-            key[w] = (uint64_t)bt;
-            val[w] = (uint32_t)j;
-            thr[j] = best - kPruneLog2;
-        }
-        return;
-    }
-    // few: the warp takes its flagged queries one at a time, its lanes striding over the
-    // tiles (four row terms in flight per lane), then a warp arg-max (ties keep the
-    // smaller tile)
-    unsigned rem = mask;
-    while (rem) {
-        const int src = __ffs(rem) - 1;
-        rem &= rem - 1u;
-        const int64_t jq = blockIdx.x * (int64_t)blockDim.x + warp * 32 + src;
-        float best = -INFINITY;
-        int bt = INT_MAX;
-        for (int t0 = lane; t0 < (int)T; t0 += 4 * 32) {
-            float rv[4], rho[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int t = min(t0 + 32 * u, (int)T - 1);
-                rv[u] = R[(int64_t)t * m_pad + jq];
-                rho[u] = tinfo[(int64_t)t * 4 + 1];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float h2 = sqrtf(rv[u]) * (1.f + 1e-5f) + sqc * rho[u];
-                const float lb = -h2 * h2;
-                if (t0 + 32 * u < (int)T && lb > best) {  // a lane's tiles ascend
-                    best = lb;
-                    bt = t0 + 32 * u;
-                }
-            }
-        }
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-            const float ob = __shfl_xor_sync(0xffffffffu, best, off);
-            const int ot = __shfl_xor_sync(0xffffffffu, bt, off);
-            if (ob > best || (ob == best && ot < bt)) {
-                best = ob;
-                bt = ot;
-            }
-        }
-        if (lane == src) {
-            const int w = w0 + __popc(mask & ((1u << src) - 1u));
-            fix_idx[w] = (int)jq;
-            key[w] = (uint64_t)bt;
-            val[w] = (uint32_t)jq;
-            thr[jq] = best - kPruneLog2;
-        }
-    }
-}
-
-// Per group (one block of 256 threads, grid-stride): the tiles some member may need, in
-// increasing order, into kept[g * T ..]; their number and the group's segment count.
-__global__ void __launch_bounds__(256)
-tc_group_keep_kernel(const uint32_t *__restrict__ order, const float *__restrict__ thr,
-                     const int *__restrict__ fix_count, int *__restrict__ n_groups, int64_t m_pad,
-                     const float *__restrict__ R, const float *__restrict__ tinfo, int64_t T, float c, int seg,
-                     int *__restrict__ kept, int *__restrict__ kcount, int *__restrict__ items) {
-    __shared__ int sq[64];
-    __shared__ float sthr[64];
-    __shared__ int wcnt[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cnt = *fix_count, G = (cnt + 63) / 64;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *n_groups = G;
-    const float sqc = sqrtf(c);
-    for (int g = blockIdx.x; g < G; g += gridDim.x) {
-        const int rows = min(64, cnt - g * 64);
-        __syncthreads();
-        if (threadIdx.x < rows) {
-            const int q = (int)order[g * 64 + threadIdx.x];
-            sq[threadIdx.x] = q;
-            sthr[threadIdx.x] = thr[q];
-        }
-        __syncthreads();
-        int base = 0;
-        for (int64_t t0 = 0; t0 < T; t0 += 256) {
-            const int64_t t = t0 + threadIdx.x;
-            bool keep = false;
-            if (t < T) {
-                const float rho = sqc * tinfo[t * 4 + 1];
-                // eight members' row terms in flight at a time
-                for (int r0 = 0; r0 < rows && !keep; r0 += 8) {
-                    float rv[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) rv[u] = R[t * m_pad + sq[min(r0 + u, rows - 1)]];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const float gap = fmaxf(0.f, sqrtf(rv[u]) * (1.f - 1e-5f) - rho);
-                        keep = keep || (r0 + u < rows && -gap * gap >= sthr[r0 + u]);
-                    }
-                }
-            }
-            const unsigned mask = __ballot_sync(0xffffffffu, keep);
-            if (lane == 0) wcnt[warp] = __popc(mask);
-            __syncthreads();
-            int off = base;
-            for (int w = 0; w < warp; ++w) off += wcnt[w];
-            if (keep) kept[(int64_t)g * T + off + __popc(mask & ((1u << lane) - 1u))] = (int)t;
-            for (int w = 0; w < 8; ++w) base += wcnt[w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            kcount[g] = base;
-            items[g] = (base + seg - 1) / seg;
-        }
-    }
-}
-
-// Per flagged query (sorted position j): the FP64 sum of its group's segment partials.
-__global__ void tc_group_combine_kernel(const double *__restrict__ part_sum, const float *__restrict__ part_shift,
-                                        const int *__restrict__ item_off, const uint32_t *__restrict__ order,
-                                        const int *__restrict__ fix_count, double scale, double *__restrict__ out) {
-    const int cnt = *fix_count;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < cnt; j += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t g = j / 64, r = j % 64;
-        const int w0 = item_off[g], w1 = item_off[g + 1];
-        float smax = -INFINITY;
-        for (int w = w0; w < w1; ++w) smax = fmaxf(smax, part_shift[(int64_t)w * 64 + r]);
-        double tot = 0.0;
-        for (int w = w0; w < w1; ++w) tot += ldexp(part_sum[(int64_t)w * 64 + r], cexp(part_shift[(int64_t)w * 64 + r] - smax));
-        out[order[j]] = w1 > w0 ? ldexp(tot, cexp(smax)) * scale : 0.0;
-    }
-}
-
-// FP64 combine of the per-split partials (as kde_combine.cu) plus the per-query error
-// estimate of the tensor-core form,
-//     est = a * (sum_t S_t w_t) / (sum_t S_t),   w_t = max(2^-21 ||q - c_g|| r_t, beta rho_t^2),
-// S_t the query's sum over tile t, r_t that tile's RMS radius, rho_t its largest radius
-// and beta = 2^-23 sqrt(MMA steps). The first term (the split products' error grows with
-// ||q - c_g|| |x - c_t|) was calibrated on the whole arithmetic over spatially coherent
-// tiles, so it covers their FP32 accumulation error too; the second takes over where the
-// accumulation error of a tile's outlying points (it grows with ||x - c_t||^2; see
-// tc_tile_radius) exceeds it. The epilogue accumulates sum_t S_t w_t. Queries with
-// est > thr (or an empty sum) are appended to fix_idx for the plain FP32 form.
-__global__ void __launch_bounds__(256)
-tc_combine_kernel(const double *__restrict__ part_sum, const float *__restrict__ part_shift,
-                  const double *__restrict__ part_w, int64_t m, int splits, double scale, const int *__restrict__ qbad,
-                  double a, double thr, double *__restrict__ out, int *__restrict__ qflag, int *__restrict__ bcnt) {
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // one query per thread
-    bool flag = false;
-    if (j < m) {
-        float smax = -INFINITY;
-        for (int k = 0; k < splits; ++k) smax = fmaxf(smax, part_shift[(int64_t)k * m + j]);
-        double tot = 0.0, wt = 0.0;
-        for (int k = 0; k < splits; ++k) {
-            const int e = cexp(part_shift[(int64_t)k * m + j] - smax);
-            tot += ldexp(part_sum[(int64_t)k * m + j], e);
-            wt += ldexp(part_w[(int64_t)k * m + j], e);
-        }
-        out[j] = ldexp(tot, cexp(smax)) * scale;
-        // tot is in units of 2^smax, a bound on every term: below 2^-40 the bound was too
-        // loose for the fixed shift (terms under 2^-126 of it were flushed)
-        const double est = (tot >= 0x1p-40 && !qbad[j]) ? a * (wt / tot) : INFINITY;
-        flag = est > thr && qflag;
-        if (qflag) qflag[j] = flag ? 1 : 0;
-    }
-    const int c = __syncthreads_count(flag);
-    if (bcnt && threadIdx.x == 0) bcnt[blockIdx.x] = c;
 }
 
 // ------------------------------------------------------------------ host helpers
@@ -1611,9 +1382,9 @@ void tc_free(stag_kde *h) {
     cudaFree(tc->qbad);
     cudaFree(tc->ub);
     cudaFree(tc->part_w);
-    cudaFree(tc->fix_idx);
     cudaFree(tc->gbuf);
     cudaFree(tc->fix_count);
+    cudaFree(tc->fin_ctl);
     cudaFree(tc->err);
     if (tc->err_host) cudaFreeHost(tc->err_host);
     delete tc;
@@ -1712,52 +1483,6 @@ int tc_prepare_points(stag_kde *h, const float *dX) {
     return rc;
 }
 
-// Carving of the grouped-recompute scratch for up to m query rows.
-struct GroupScratch {
-    uint64_t *key, *ktmp;
-    uint32_t *val, *vtmp, *hist;
-    float *thr;
-    int *qflag, *bcnt, *boff, *kept, *kcount, *items, *item_off, *n_groups;
-    double *psum;
-    float *pshift;
-};
-
-// Kept point tiles per work item: at least eight 64-point tiles (the per-item set-up is
-// then amortised), and at most 64 items per group.
-static int group_seg(int64_t T, int BN) { return (int)std::max<int64_t>(8 * 64 / BN, ceil_div(T, 64)); }
-
-static int64_t group_scratch_bytes(int64_t m, int64_t T, int BN, GroupScratch *gs, void *base) {
-    const int64_t G = ceil_div(std::max<int64_t>(m, 1), 64);
-    const int64_t B = ceil_div(std::max<int64_t>(m, 1), 256);  // blocks of the combine kernel
-    const int64_t items = G * ceil_div(T, group_seg(T, BN));  // at most 64 segments per group
-    int64_t off = 0;
-    auto take = [&](int64_t bytes) {
-        const int64_t o = off;
-        off += round_up(bytes, 256);
-        return static_cast<char *>(base) + o;
-    };
-    const int64_t mm = std::max<int64_t>(m, 1);
-    GroupScratch g;
-    g.key = (uint64_t *)take(mm * 8);
-    g.ktmp = (uint64_t *)take(mm * 8);
-    g.val = (uint32_t *)take(mm * 4);
-    g.vtmp = (uint32_t *)take(mm * 4);
-    g.hist = (uint32_t *)take(radix_sort_hist_entries(mm) * 4);
-    g.thr = (float *)take(mm * 4);
-    g.qflag = (int *)take(mm * 4);
-    g.bcnt = (int *)take(B * 4);
-    g.boff = (int *)take((B + 1) * 4);
-    g.kept = (int *)take(G * T * 4);
-    g.kcount = (int *)take(G * 4);
-    g.items = (int *)take(G * 4);
-    g.item_off = (int *)take((G + 1) * 4);
-    g.n_groups = (int *)take(4);
-    g.psum = (double *)take(items * 64 * 8);
-    g.pshift = (float *)take(items * 64 * 4);
-    if (gs) *gs = g;
-    return off;
-}
-
 static int ensure_query_scratch(stag_kde *h, int64_t m_pad) {
     TcData *tc = h->tc;
     const int Kp = tc->Kp;
@@ -1778,19 +1503,20 @@ static int ensure_query_scratch(stag_kde *h, int64_t m_pad) {
         cudaFree(tc->unorm);
         cudaFree(tc->qbad);
         cudaFree(tc->ub);
-        cudaFree(tc->fix_idx);
         tc->unorm = nullptr;
         tc->qbad = nullptr;
         tc->ub = nullptr;
-        tc->fix_idx = nullptr;
         tc->unorm_cap = 0;
         STAG_CUDA_TRY(dev_malloc(&tc->unorm, m_pad * sizeof(float)));
         STAG_CUDA_TRY(dev_malloc(&tc->qbad, m_pad * sizeof(int)));
         STAG_CUDA_TRY(dev_malloc(&tc->ub, m_pad * sizeof(unsigned)));
-        STAG_CUDA_TRY(dev_malloc(&tc->fix_idx, m_pad * sizeof(int)));
+        // (zero between calls: the row-term kernel raises them, the combine puts them back)
+        STAG_CUDA_TRY(cudaMemset(tc->ub, 0, m_pad * sizeof(unsigned)));
+        STAG_CUDA_TRY(cudaStreamSynchronize(nullptr));  // (the query's stream may not wait for this one)
         tc->unorm_cap = m_pad;
     }
     if (!tc->fix_count) STAG_CUDA_TRY(dev_malloc(&tc->fix_count, sizeof(int)));
+    if (!tc->fin_ctl) STAG_CUDA_TRY(dev_malloc(&tc->fin_ctl, fin_ctl_bytes(1)));
     const int64_t need = tc->T * m_pad;
     if (tc->rt_cap < need) {
         cudaFree(tc->rowterm);
@@ -1835,7 +1561,7 @@ int tc_reserve(stag_kde *h, int64_t m, int tiles_per_unit) {
             cudaFree(tc->gbuf);
             tc->gbuf = nullptr;
             tc->gbuf_m = 0;
-            STAG_CUDA_TRY(dev_malloc(&tc->gbuf, group_scratch_bytes(m, tc->T, tc->BN, nullptr, nullptr)));
+            STAG_CUDA_TRY(dev_malloc(&tc->gbuf, fin_scratch_bytes(m, tc->T, tc->BN, nullptr, nullptr)));
             tc->gbuf_m = m;
         }
         rc = ensure_qt(h, ceil_div(m, kSimtTile) * h->d_pad * kSimtTile * 2);
@@ -1853,30 +1579,51 @@ int tc_reserve(stag_kde *h, int64_t m, int tiles_per_unit) {
     return 0;
 }
 
-// Query-side preparation: FP16 splits of the queries, the row terms and bounds (one launch).
-static int tc_prep(stag_kde *h, const float *dQ, int64_t m, cudaStream_t s) {
-    TcData *tc = h->tc;
-    const int Kp = tc->Kp;
-    const int64_t m_pad = round_up(m, BM);
-    const double c = h->a * 1.4426950408889634;
-    STAG_CUDA_TRY(cudaMemsetAsync(tc->qbad, 0, m_pad * sizeof(int), s));
-    STAG_CUDA_TRY(cudaMemsetAsync(tc->ub, 0, m_pad * sizeof(unsigned), s));
+// The row-term kernel's view of one instance; returns its number of blocks.
+static int64_t fill_rt(const stag_kde *h, const float *dQ, int64_t m, int tiles_per_block, int block_begin, int *dflag,
+                       RtInst *r) {
+    const TcData *tc = h->tc;
+    *r = RtInst{};
+    r->Q = dQ;
+    r->centT = tc->centT;
+    r->cg = tc->cg;
+    r->tinfo = tc->tinfo;
+    r->scales = tc->scales;
+    r->R = tc->rowterm;
+    r->unorm = tc->unorm;
+    r->ub = tc->ub;
+    r->ahi = tc->a_hi;
+    r->alo = tc->a_lo;
+    r->qbad = tc->qbad;
+    r->fix_count = tc->fix_count;
+    r->flag = dflag;
+    r->m = m;
+    r->m_pad = round_up(m, BM);
+    r->T = tc->T;
+    r->d = (int)h->d;
+    r->tiles_per_block = tiles_per_block;
+    r->qblocks = (int)(r->m_pad / BM);
+    r->block_begin = block_begin;
+    r->c = (float)(h->a * 1.4426950408889634);
+    return r->qblocks * ceil_div(tc->T, tiles_per_block);
+}
+
+static int launch_rowterm(int Kp, const RtInst &r0, const RtInst *table, int n_inst, int64_t blocks, cudaStream_t s) {
+    if (blocks > 0x7fffffff) return fail(STAG_KDE_EINVAL, "query batch too large");
     count_launch(1);
-    // tiles per block: 256, fewer when that leaves under ~4 blocks per SM (small batches)
-    int tpb = 256;
-    while (tpb > RowTermGeo::TG && (m_pad / BM) * ceil_div(tc->T, tpb) < 4 * (int64_t)h->sm_count) tpb /= 2;
-    dim3 grid((unsigned)(m_pad / BM), (unsigned)ceil_div(tc->T, tpb));
     switch (Kp) {
 #define STAG_ROWTERM(KPV)                                                                                          \
     case KPV: {                                                                                                    \
         /* set once per instantiation (before any stream capture can be in progress) */                           \
-        static cudaError_t attr = cudaFuncSetAttribute(tc_rowterm_kernel<KPV>,                                    \
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,               \
-                                                       RowTermGeo::smem_bytes(KPV));                              \
-        STAG_CUDA_TRY(attr);                                                                                       \
-        tc_rowterm_kernel<KPV><<<grid, RowTermGeo::THREADS, RowTermGeo::smem_bytes(KPV), s>>>(                     \
-            dQ, m, h->d, m_pad, tc->cent, tc->T, tpb, (float)c, tc->rowterm, tc->cg, tc->unorm, tc->tinfo, tc->ub,  \
-            tc->scales, tc->a_hi, tc->a_lo, tc->qbad, tc->centT);                                                  \
+        auto kern = table ? tc_rowterm_kernel<KPV, true> : tc_rowterm_kernel<KPV, false>;                         \
+        constexpr int smem = RowTermGeo::smem_bytes(KPV);                                                          \
+        static cudaError_t attr0 = cudaFuncSetAttribute(tc_rowterm_kernel<KPV, false>,                            \
+                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);       \
+        static cudaError_t attr1 = cudaFuncSetAttribute(tc_rowterm_kernel<KPV, true>,                             \
+                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);       \
+        STAG_CUDA_TRY(attr0);                                                                                      \
+        STAG_CUDA_TRY(attr1);                                                                                      \
+        kern<<<(unsigned)blocks, RowTermGeo::THREADS, smem, s>>>(r0, table, n_inst);                              \
         break;                                                                                                     \
     }
         STAG_ROWTERM(16)
@@ -1887,6 +1634,19 @@ static int tc_prep(stag_kde *h, const float *dQ, int64_t m, cudaStream_t s) {
     }
     STAG_CUDA_TRY(cudaGetLastError());
     return 0;
+}
+
+// Query-side preparation: FP16 splits of the queries, the row terms and bounds, and the
+// input check if dflag is given (one launch).
+static int tc_prep(stag_kde *h, const float *dQ, int64_t m, int *dflag, cudaStream_t s) {
+    TcData *tc = h->tc;
+    const int64_t m_pad = round_up(m, BM);
+    // tiles per block: 256, fewer when that leaves under ~4 blocks per SM (small batches)
+    int tpb = 256;
+    while (tpb > RowTermGeo::TG && (m_pad / BM) * ceil_div(tc->T, tpb) < 4 * (int64_t)h->sm_count) tpb /= 2;
+    RtInst r;
+    const int64_t blocks = fill_rt(h, dQ, m, tpb, 0, dflag, &r);
+    return launch_rowterm(tc->Kp, r, nullptr, 1, blocks, s);
 }
 
 // Fills the kernel's view of one instance (units numbered from unit_begin).
@@ -1917,70 +1677,55 @@ static void fill_inst(const stag_kde *h, int64_t m, int64_t q_tiles, int64_t spl
     I->units = q_tiles * splits;
 }
 
-// Grouped recompute of the flagged queries, all on stream s (after tc_combine_kernel has
-// written the per-query flags and per-block counts into the scratch).
-static int tc_fixup_grouped(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaStream_t s) {
+// The finish kernels' view of one instance (tc_finish.h).
+static void fill_fin(const stag_kde *h, const float *dQ, int64_t m, int64_t splits, double *dOut, FinInst *f) {
     TcData *tc = h->tc;
-    GroupScratch g;
-    group_scratch_bytes(m, tc->T, tc->BN, &g, tc->gbuf);
-    const int64_t m_pad = round_up(m, BM);
-    const int64_t B = ceil_div(m, 256);
-    const float c = (float)(h->a * 1.4426950408889634);
-    const int seg = group_seg(tc->T, tc->BN);
-    const int per = tc->BN / kSimtTile;
-    count_launch(2);
-    // the flagged queries in query order (their count into fix_count), with sort keys
-    tc_scan_kernel<<<1, 1024, 0, s>>>(g.bcnt, nullptr, (int)B, g.boff, tc->fix_count);
-    tc_flag_compact_kernel<<<(unsigned)B, 256, 0, s>>>(g.qflag, g.boff, m, m_pad, tc->rowterm, tc->tinfo, tc->T, c,
-                                                       tc->fix_idx, g.key, g.val, g.thr);
-    STAG_CUDA_TRY(cudaGetLastError());
-    // stable sort by leading tile of the flagged entries only (device count): the input
-    // is in query order, so the groups are deterministic
-    int bits = 1;
-    while (((int64_t)1 << bits) < tc->T) ++bits;
-    int rc = radix_sort_pairs(g.key, g.val, g.ktmp, g.vtmp, g.hist, m, bits, s, tc->fix_count);
-    if (rc) return rc;
-    rc = simt_gather_rows(h, dQ, reinterpret_cast<const int *>(g.val), tc->fix_count, m, h->qt, s);
-    if (rc) return rc;
-    count_launch(2);
-    tc_group_keep_kernel<<<(unsigned)(h->sm_count * 4), 256, 0, s>>>(g.val, g.thr, tc->fix_count, g.n_groups, m_pad,
-                                                                      tc->rowterm, tc->tinfo, tc->T, c, seg, g.kept,
-                                                                      g.kcount, g.items);
-    tc_scan_kernel<<<1, 1024, 0, s>>>(g.items, tc->fix_count, 0, g.item_off, nullptr);
-    STAG_CUDA_TRY(cudaGetLastError());
-    rc = simt_list_launch(h, tc->xkt, h->qt, g.kept, tc->T, g.kcount, g.item_off, g.n_groups, seg, per, g.psum,
-                          g.pshift, s);
-    if (rc) return rc;
-    count_launch();
-    tc_group_combine_kernel<<<(unsigned)std::min<int64_t>(ceil_div(m, 256), 1024), 256, 0, s>>>(
-        g.psum, g.pshift, g.item_off, g.val, tc->fix_count, h->normalise ? 1.0 / (double)h->n : 1.0, dOut);
-    STAG_CUDA_TRY(cudaGetLastError());
-    return 0;
+    *f = FinInst{};
+    if (h->tc_check) fin_scratch_bytes(m, tc->T, tc->BN, f, tc->gbuf);
+    f->part_sum = h->part.sum;
+    f->part_shift = h->part.shift;
+    f->part_w = tc->part_w;
+    f->qbad = tc->qbad;
+    f->ub = tc->ub;
+    f->out = dOut;
+    f->fix_count = tc->fix_count;
+    f->m = m;
+    f->m_pad = round_up(m, BM);
+    f->splits = (int)splits;
+    f->scale = h->normalise ? 1.0 / (double)h->n : 1.0;
+    f->a = h->a;
+    f->Q = dQ;
+    f->R = tc->rowterm;
+    f->tinfo = tc->tinfo;
+    f->xkt = tc->xkt;
+    f->n = h->n;
+    f->n_tiles = h->n_tiles;
+    f->T = tc->T;
+    f->d = (int)h->d;
+    f->d_pad = h->d_pad;
+    f->c = (float)(h->a * 1.4426950408889634);
+    f->negc = (float)(-h->a * 1.4426950408889634);
+    f->qt = h->qt;
 }
 
+// Work items the recompute of m queries can have at most (bounds its grid).
+static int64_t max_fix_items(int64_t m, int64_t T) { return ceil_div(m, 64) * std::min<int64_t>(64, T); }
+
 // FP64 combine with the per-query error estimate, then the FP32 recompute of the flagged
-// queries over the tiles that can matter (tc_fixup_grouped).
+// queries over the tiles that can matter (tc_finish.cu).
 static int tc_finish(stag_kde *h, const float *dQ, int64_t m, int64_t splits, double *dOut, cudaStream_t s) {
     TcData *tc = h->tc;
-    const bool check = h->tc_check;
-    GroupScratch g{};
-    if (check) group_scratch_bytes(m, tc->T, tc->BN, &g, tc->gbuf);
-    count_launch();
-    tc_combine_kernel<<<(unsigned)ceil_div(m, 256), 256, 0, s>>>(
-        h->part.sum, h->part.shift, tc->part_w, m, (int)splits, h->normalise ? 1.0 / (double)h->n : 1.0, tc->qbad,
-        h->a, kTcErrThreshold, dOut, check ? g.qflag : nullptr, check ? g.bcnt : nullptr);
-    STAG_CUDA_TRY(cudaGetLastError());
-    if (!check) return 0;
-    // groups of 64 flagged queries share every point load (a per-query pass would re-read
-    // its kept tiles once per query)
-    return tc_fixup_grouped(h, dQ, m, dOut, s);
+    FinInst f;
+    fill_fin(h, dQ, m, splits, dOut, &f);
+    int cblocks, qblocks;
+    fin_number(&f, h->sm_count, 0, 0, &cblocks, &qblocks);
+    return fin_launch(f, nullptr, 1, cblocks, qblocks, f.passes, h->d_pad, max_fix_items(m, tc->T), h->tc_check,
+                      tc->fin_ctl, tc->err, h->sm_count, h->wait_ns, s);
 }
 
 int tc_operand_width(const stag_kde *h) { return h->tc ? h->tc->Kp : 0; }
 
 size_t tc_inst_size() { return sizeof(TcInst); }
-
-int tc_prep_public(stag_kde *h, const float *dQ, int64_t m, cudaStream_t s) { return tc_prep(h, dQ, m, s); }
 
 int64_t tc_fill_inst(const stag_kde *h, int64_t m, int tiles_per_unit, int64_t unit_begin, void *inst,
                      int64_t *splits) {
@@ -1991,19 +1736,27 @@ int64_t tc_fill_inst(const stag_kde *h, int64_t m, int tiles_per_unit, int64_t u
     return I->units;
 }
 
-int tc_finish_public(stag_kde *h, const float *dQ, int64_t m, int64_t splits, double *dOut, cudaStream_t s) {
-    return tc_finish(h, dQ, m, splits, dOut, s);
+size_t tc_rt_size() { return sizeof(RtInst); }
+
+int64_t tc_fill_rt(const stag_kde *h, const float *dQ, int64_t m, int64_t block_begin, void *inst) {
+    return fill_rt(h, dQ, m, 256, (int)block_begin, nullptr, reinterpret_cast<RtInst *>(inst));
 }
+
+int tc_launch_rowterm(int Kp, const void *table, int n_inst, int64_t blocks, cudaStream_t s) {
+    return launch_rowterm(Kp, RtInst{}, reinterpret_cast<const RtInst *>(table), n_inst, blocks, s);
+}
+
+void tc_fill_fin(const stag_kde *h, const float *dQ, int64_t m, int64_t splits, double *dOut, FinInst *f) {
+    fill_fin(h, dQ, m, splits, dOut, f);
+}
+
+int64_t tc_max_fix_items(const stag_kde *h, int64_t m) { return max_fix_items(m, h->tc->T); }
 
 int tc_query(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaStream_t s, int *dflag) {
     TcData *tc = h->tc;
     int rc = tc_reserve(h, m, h->tune_tiles_per_unit);
     if (rc) return rc;
-    if (dflag) {
-        rc = launch_check_finite_f32(dQ, m * h->d, dflag, s);
-        if (rc) return rc;
-    }
-    rc = tc_prep(h, dQ, m, s);
+    rc = tc_prep(h, dQ, m, dflag, s);
     if (rc) return rc;
     int64_t q_tiles, splits, tps;
     plan_units(h, m, h->tune_tiles_per_unit, &q_tiles, &splits, &tps);

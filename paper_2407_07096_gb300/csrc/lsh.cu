@@ -633,7 +633,7 @@ LshTables tables_of(const stag_lsh *h) {
 // exceed the lists by the members that several tables share); *done says whether it was.
 // Synchronises the stream.
 constexpr int64_t kMaxRawBytes = (int64_t)4 << 30;
-constexpr int64_t kFixedRawBytes = (int64_t)64 << 20;
+constexpr int64_t kFixedRawBytes = (int64_t)256 << 20;
 constexpr int64_t kSumPoints = (int64_t)1 << 17;  // above: summary bitmap, wider blocks
 
 template <int kThreads, bool kSum>
