@@ -951,7 +951,7 @@ __global__ void tc_tile_radius_kernel(const float *__restrict__ X, int64_t n, in
 // R[t][q] = c * ||q - c_t||^2 by direct differences in FP32 (padding queries: 0), the
 // per-query upper bound on every exponent, and ||q - c_g||. The first column of blocks
 // also writes the query's scaled, centred coordinates u = (q - c_g) * scale_u as FP16
-// hi/lo pairs (the MMA's A operand; the difference and scale in FP64, u_lo = u - u_hi)
+// hi/lo pairs (the MMA's A operand, split_query)
 // and flags, in qbad, a query farther from the data than that range (its row is zeroed and
 // the combine hands it to the plain FP32 form).
 // Register tiling: a block takes 128 queries and walks its range of point tiles 64 at a
@@ -972,6 +972,25 @@ struct RowTermGeo {
     static constexpr int QS = 128 + 4;  // row stride of the transposed queries (floats)
     static constexpr int smem_bytes(int kp) { return kp * QS * 4; }
 };
+
+// The FP16 hi/lo split of u = (q - c) su, su a power of two, df = fl(q - c): hi = half(fl(u)),
+// lo = half(fl(u - hi)), as if u were formed without rounding; bad = 1 (and zeros) where |u|
+// reaches 2^15. The difference's rounding error comes from Knuth's two-sum, so everything
+// stays in FP32: fl(u) is df su, df su - hi is exact (24 and 11 bits with a common leading
+// part) and one addition rounds u - hi. The same values as in double precision, whose
+// conversions and products held the FP64 pipe (16 clocks an instruction) for 28 us per 128
+// queries at K = 128, the longest chain of a small call.
+__device__ __forceinline__ void split_query(float q, float c, float df, float su, __half &hi, __half &lo, int &bad) {
+    const float bb = df - q;                     // -c as it was subtracted
+    const float er = (q - (df - bb)) - (c + bb);  // q - c = df + er exactly
+    const float u = __fmul_rn(df, su), eu = __fmul_rn(er, su);
+    if (fabsf(u) < 0x1p15f || (fabsf(u) == 0x1p15f && copysignf(1.f, u) * eu < 0.f)) {
+        hi = __float2half_rn(u);
+        lo = __float2half_rn((u - __half2float(hi)) + eu);
+    } else {
+        bad = 1;
+    }
+}
 
 // One instance of the row-term kernel (a launch serves a table of them, or one).
 struct RtInst {
@@ -1027,7 +1046,7 @@ tc_rowterm_kernel(const __grid_constant__ RtInst inst0, const RtInst *__restrict
         const int64_t q = q0 + r;
         const bool real = q < m;
         const int k0 = part * (KP / 2);
-        const double su = I.scales[1];
+        const float su = I.scales[1];
         float s2 = 0.f;
         int bad = 0, refused = 0;
         uint4 *dh = reinterpret_cast<uint4 *>(I.ahi + q * KP + k0);
@@ -1040,17 +1059,11 @@ tc_rowterm_kernel(const __grid_constant__ RtInst inst0, const RtInst *__restrict
                 const int k = k0 + k8 * 8 + j;
                 __half hh = __float2half_rn(0.f), ll = __float2half_rn(0.f);
                 if (real && k < d) {
-                    const float qk = I.Q[q * d + k];
-                    refused |= !(fabs((double)qk) <= 1e15);
-                    const float df = qk - I.cg[k];
+                    const float qk = I.Q[q * d + k], ck = I.cg[k];
+                    refused |= !(fabsf(qk) <= 1e15f);
+                    const float df = qk - ck;
                     s2 = fmaf(df, df, s2);
-                    const double u = ((double)qk - (double)I.cg[k]) * su;
-                    if (fabs(u) < 0x1p15) {
-                        hh = __float2half_rn((float)u);
-                        ll = __float2half_rn((float)(u - (double)__half2float(hh)));
-                    } else {
-                        bad = 1;
-                    }
+                    split_query(qk, ck, df, su, hh, ll, bad);
                 }
                 hv[j] = hh;
                 lv[j] = ll;
