@@ -68,6 +68,13 @@ struct Partials {
 
 struct TcData;  // tensor-core form data (kde_tc.cu)
 
+// A host query of up to kStageRows rows copies its results beside the status into pinned
+// memory and waits once; larger ones check the status first and then copy straight to the
+// caller (whose buffer stays untouched on failure either way).
+constexpr int64_t kStageRows = 8192;
+constexpr size_t kStageOffset = 64;
+constexpr size_t kStageBytes = kStageOffset + kStageRows * sizeof(double);
+
 }  // namespace stagkde
 
 struct stag_kde {
@@ -112,10 +119,13 @@ struct stag_kde {
     float *xrow = nullptr;    // row-major FP32 point set, rows of d_pad, for gathers (subset sums), built on first use
     void *sub_dev = nullptr;  // host subset call: device copies of offsets, indices, weights
     int64_t sub_dev_cap = 0;  // bytes
-    int *flag_dev = nullptr;  // input-validation flag
+    // status of the host calls: [0] input-validation flag, [1] the tensor-core kernel's error
+    // code. Zero between calls; status_dirty: a call ended before it had read them.
+    int *flag_dev = nullptr;
+    bool status_dirty = false;
     cudaStream_t copy_stream[2] = {nullptr, nullptr};  // host subset call: extra streams for the list copies
     cudaEvent_t copy_done[2] = {nullptr, nullptr};
-    int *flag_host = nullptr; // pinned mirror
+    int *flag_host = nullptr; // pinned: the status, then (from kStageOffset) small results
     int sm_count = 0;
 
     // main-kernel timing (stag_kde_profile_begin/end)
@@ -146,8 +156,7 @@ int simt_reserve(stag_kde *h, int64_t m);
 int ensure_qt(stag_kde *h, int64_t floats);
 // A tile-transposed copy of row-major points (the k-d ordered set).
 int simt_tiles_from_rows(const stag_kde *h, const float *rows, float *out, cudaStream_t s);
-int launch_check_finite_f32(const float *p, int64_t count, int *dflag, cudaStream_t s, int bit = 1);
-int launch_check_finite_f64(const double *p, int64_t count, int *dflag, cudaStream_t s);
+int launch_check_finite_f32(const float *p, int64_t count, int *dflag, cudaStream_t s, int bit);
 
 // kde_subset.cu: weighted subset sums over per-query (index, weight) lists. `entries`
 // (the list entries, if known on the host) only feeds the profiling counters.
@@ -186,10 +195,6 @@ int tc_tile_points(int64_t d);
 int tc_prepare_points(stag_kde *h, const float *dX);
 int tc_query(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaStream_t s, int *dflag);
 void tc_free(stag_kde *h);
-// The kernel's error code (a bounded wait that expired): tc_error_enqueue queues its copy
-// to the host on s; after s has been synchronised, tc_error_take reports and clears it.
-int tc_error_enqueue(stag_kde *h, cudaStream_t s);
-int tc_error_take(stag_kde *h, cudaStream_t s);
 int tc_reserve(stag_kde *h, int64_t m, int tiles_per_unit);
 int tc_make_view(const stag_kde *base, stag_kde *view);
 // Pieces of a tensor-core query for the batched path (kde_tc.cu).

@@ -92,7 +92,7 @@ template <int KERN, int R>
 __global__ void __launch_bounds__(kThreads)
 kde_f64_kernel(const double *__restrict__ X, int64_t n, const double *__restrict__ Q, int64_t m, int d, double a,
                double scale, int qlog, int64_t tiles_per_split, double *part, unsigned *ticket,
-               double *__restrict__ out) {
+               double *__restrict__ out, int *flag) {
     __shared__ double sx[2][kMaxPts * kXS];
     __shared__ double sq[2][kKC * kMaxQl];
     __shared__ double tab[kTab];
@@ -103,6 +103,12 @@ kde_f64_kernel(const double *__restrict__ X, int64_t n, const double *__restrict
     const int64_t q0 = (int64_t)blockIdx.x * ql;
     const int rows = (int)min((int64_t)ql, m - q0);
     if (tid < kTab) tab[tid] = exp2((double)tid / kTab);
+    if (flag && blockIdx.y == 0) {
+        // the input check: bit 0 if a query is not finite or beyond 1e15
+        int bad = 0;
+        for (int64_t e = tid; e < (int64_t)rows * d; e += kThreads) bad |= !(fabs(Q[q0 * d + e]) <= 1e15);
+        if (bad) atomicOr(flag, 1);
+    }
     const int64_t tiles = (n + pts - 1) / pts;
     const int64_t t0 = blockIdx.y * tiles_per_split, t1 = min(tiles, t0 + tiles_per_split);
     const int nch = (d + kKC - 1) / kKC;
@@ -212,15 +218,16 @@ Split64 split64(const stag_kde *h, int64_t m) {
 }
 
 template <int KERN>
-void launch64(const stag_kde *h, const Split64 &sp, const double *dQ, int64_t m, double *dOut, cudaStream_t s) {
+void launch64(const stag_kde *h, const Split64 &sp, const double *dQ, int64_t m, double *dOut, int *dflag,
+              cudaStream_t s) {
     const dim3 grid((unsigned)sp.q_tiles, (unsigned)sp.splits);
     const double scale = h->normalise ? 1.0 / (double)h->n : 1.0;
     if (sp.r == 4)
         kde_f64_kernel<KERN, 4><<<grid, kThreads, 0, s>>>(h->x64, h->n, dQ, m, (int)h->d, h->a, scale, sp.qlog, sp.tps,
-                                                          h->f64_part, h->tickets, dOut);
+                                                          h->f64_part, h->tickets, dOut, dflag);
     else
         kde_f64_kernel<KERN, 1><<<grid, kThreads, 0, s>>>(h->x64, h->n, dQ, m, (int)h->d, h->a, scale, sp.qlog, sp.tps,
-                                                          h->f64_part, h->tickets, dOut);
+                                                          h->f64_part, h->tickets, dOut, dflag);
 }
 
 }  // namespace
@@ -242,10 +249,6 @@ int f64_set_scratch(stag_kde *h, void *p) {
 }
 
 int f64_query(stag_kde *h, const double *dQ, int64_t m, double *dOut, cudaStream_t s, int *dflag) {
-    if (dflag) {
-        int rc = launch_check_finite_f64(dQ, m * h->d, dflag, s);
-        if (rc) return rc;
-    }
     if (h->d > kF64MaxD) return fail(STAG_KDE_EUNSUPPORTED, "FP64 form: d too large");
     const Split64 sp = split64(h, m);
     if (sp.q_tiles > 0x7fffffff) return fail(STAG_KDE_EINVAL, "query batch too large");
@@ -253,13 +256,13 @@ int f64_query(stag_kde *h, const double *dQ, int64_t m, double *dOut, cudaStream
     prof_start(h, s);
     switch (h->kernel) {
         case STAG_KDE_KERNEL_EXPONENTIAL:
-            launch64<STAG_KDE_KERNEL_EXPONENTIAL>(h, sp, dQ, m, dOut, s);
+            launch64<STAG_KDE_KERNEL_EXPONENTIAL>(h, sp, dQ, m, dOut, dflag, s);
             break;
         case STAG_KDE_KERNEL_LOGISTIC:
-            launch64<STAG_KDE_KERNEL_LOGISTIC>(h, sp, dQ, m, dOut, s);
+            launch64<STAG_KDE_KERNEL_LOGISTIC>(h, sp, dQ, m, dOut, dflag, s);
             break;
         default:
-            launch64<STAG_KDE_KERNEL_GAUSSIAN>(h, sp, dQ, m, dOut, s);
+            launch64<STAG_KDE_KERNEL_GAUSSIAN>(h, sp, dQ, m, dOut, dflag, s);
     }
     prof_stop(h, s, (double)m * (double)h->n);
     STAG_CUDA_TRY(cudaGetLastError());

@@ -55,11 +55,13 @@ kde_simt_f32_kernel(const float *__restrict__ xt, int64_t n, int64_t n_tiles, co
 }
 
 // Row-major n x d -> tile-transposed [tile][d_pad][64], zero padded. kDup: every value
-// twice, [tile][d_pad][64][2] (queries).
+// twice, [tile][d_pad][64][2] (queries). Sets bit 0 of *flag (or NULL) if a value is not
+// finite or exceeds 1e15 in magnitude.
 template <typename T, bool kDup>
 __global__ void to_tiles_kernel(const T *__restrict__ src, int64_t rows, int64_t d, int d_pad,
-                                int64_t n_tiles, float *__restrict__ dst) {
+                                int64_t n_tiles, float *__restrict__ dst, int *flag = nullptr) {
     const int64_t total = n_tiles * d_pad * kSimtTile;
+    int bad = 0;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
          idx += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(idx % kSimtTile);
@@ -69,16 +71,17 @@ __global__ void to_tiles_kernel(const T *__restrict__ src, int64_t rows, int64_t
         const int64_t row = t * kSimtTile + r;
         float v = 0.f;
         if (row < rows && k < d) v = (float)src[row * d + k];
+        bad |= !(fabsf(v) <= 1e15f);  // (FP32 values: the same as <= 1e15)
         if (kDup)
             reinterpret_cast<float2 *>(dst)[idx] = make_float2(v, v);
         else
             dst[idx] = v;
     }
+    if (flag && bad) atomicOr(flag, 1);
 }
 
 // ORs `bit` into *flag when a value is not finite or exceeds 1e15 in magnitude.
-template <typename T>
-__global__ void check_finite_kernel(const T *__restrict__ p, int64_t count, int *flag, int bit) {
+__global__ void check_finite_kernel(const float *__restrict__ p, int64_t count, int *flag, int bit) {
     int bad = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -120,15 +123,7 @@ int ensure_qt(stag_kde *h, int64_t floats) {
 int launch_check_finite_f32(const float *p, int64_t count, int *dflag, cudaStream_t s, int bit) {
     if (count <= 0) return 0;
     count_launch();
-    check_finite_kernel<float><<<grid_for(count, 256), 256, 0, s>>>(p, count, dflag, bit);
-    STAG_CUDA_TRY(cudaGetLastError());
-    return 0;
-}
-
-int launch_check_finite_f64(const double *p, int64_t count, int *dflag, cudaStream_t s) {
-    if (count <= 0) return 0;
-    count_launch();
-    check_finite_kernel<double><<<grid_for(count, 256), 256, 0, s>>>(p, count, dflag, 1);
+    check_finite_kernel<<<grid_for(count, 256), 256, 0, s>>>(p, count, dflag, bit);
     STAG_CUDA_TRY(cudaGetLastError());
     return 0;
 }
@@ -192,12 +187,8 @@ int simt_query_f32(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaSt
     if (rc) return rc;
     const int64_t total = q_tiles * h->d_pad * kSimtTile;
     count_launch();
-    to_tiles_kernel<float, true><<<grid_for(total, 256), 256, 0, s>>>(dQ, m, h->d, h->d_pad, q_tiles, h->qt);
+    to_tiles_kernel<float, true><<<grid_for(total, 256), 256, 0, s>>>(dQ, m, h->d, h->d_pad, q_tiles, h->qt, dflag);
     STAG_CUDA_TRY(cudaGetLastError());
-    if (dflag) {
-        rc = launch_check_finite_f32(dQ, m * h->d, dflag, s);
-        if (rc) return rc;
-    }
     const int64_t tps = choose_tiles_per_split(h, q_tiles);
     const int64_t splits = ceil_div(h->n_tiles, tps);
     rc = ensure_partials(h, splits * m);

@@ -103,8 +103,7 @@ struct TcData {
     int64_t gbuf_m = 0;
     int *fix_count = nullptr;  // device: number of queries handed to the plain form
     FinCtl *fin_ctl = nullptr; // device: the recompute's phase counters
-    int *err = nullptr;        // device error code (timeouts)
-    int *err_host = nullptr;   // pinned mirror
+    int *err = nullptr;        // device error code (timeouts): the handle's flag_dev + 1
 };
 
 namespace {
@@ -1398,8 +1397,6 @@ void tc_free(stag_kde *h) {
     cudaFree(tc->gbuf);
     cudaFree(tc->fix_count);
     cudaFree(tc->fin_ctl);
-    cudaFree(tc->err);
-    if (tc->err_host) cudaFreeHost(tc->err_host);
     delete tc;
     h->tc = nullptr;
 }
@@ -1433,9 +1430,7 @@ int tc_make_view(const stag_kde *base, stag_kde *view) {
     tc->map_blo = b->map_blo;
     tc->map_baug = b->map_baug;
     tc->map_aaug = b->map_aaug;
-    STAG_CUDA_TRY(dev_malloc(&tc->err, sizeof(int)));
-    STAG_CUDA_TRY(cudaMemset(tc->err, 0, sizeof(int)));
-    STAG_CUDA_TRY(cudaMallocHost(&tc->err_host, sizeof(int)));
+    tc->err = view->flag_dev + 1;
     return 0;
 }
 
@@ -1468,9 +1463,7 @@ int tc_prepare_points(stag_kde *h, const float *dX) {
     STAG_CUDA_TRY(dev_malloc(&tc->vmax_bits, sizeof(unsigned)));
     STAG_CUDA_TRY(dev_malloc(&tc->xmax_bits, sizeof(unsigned)));
     STAG_CUDA_TRY(dev_malloc(&tc->scales, 4 * sizeof(float)));
-    STAG_CUDA_TRY(dev_malloc(&tc->err, sizeof(int)));
-    STAG_CUDA_TRY(cudaMallocHost(&tc->err_host, sizeof(int)));
-    STAG_CUDA_TRY(cudaMemsetAsync(tc->err, 0, sizeof(int), s));
+    tc->err = h->flag_dev + 1;
     STAG_CUDA_TRY(cudaMemsetAsync(tc->vmax_bits, 0, sizeof(unsigned), s));
     STAG_CUDA_TRY(cudaMemsetAsync(tc->xmax_bits, 0, sizeof(unsigned), s));
 
@@ -1788,23 +1781,6 @@ int tc_fixed_rows(stag_kde *h, int64_t *count) {
     int v = 0;
     if (tc && tc->fix_count && h->tc_check) STAG_CUDA_TRY(cudaMemcpy(&v, tc->fix_count, sizeof(int), cudaMemcpyDeviceToHost));
     *count = v;
-    return 0;
-}
-
-int tc_error_enqueue(stag_kde *h, cudaStream_t s) {
-    TcData *tc = h->tc;
-    if (!tc) return 0;
-    STAG_CUDA_TRY(cudaMemcpyAsync(tc->err_host, tc->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    return 0;
-}
-
-int tc_error_take(stag_kde *h, cudaStream_t s) {
-    TcData *tc = h->tc;
-    if (!tc) return 0;
-    if (*tc->err_host) {
-        STAG_CUDA_TRY(cudaMemsetAsync(tc->err, 0, sizeof(int), s));
-        return fail(STAG_KDE_ETIMEDOUT, "tensor-core kernel: a bounded wait expired");
-    }
     return 0;
 }
 

@@ -184,8 +184,10 @@ stag_kde *make_view(stag_kde *base) {
     v->sm_count = base->sm_count;
     cudaError_t e;
     if ((e = cudaStreamCreateWithFlags(&v->stream, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = dev_malloc(&v->flag_dev, sizeof(int))) != cudaSuccess ||
-        (e = cudaMallocHost(&v->flag_host, sizeof(int))) != cudaSuccess) {
+        (e = dev_malloc(&v->flag_dev, 2 * sizeof(int))) != cudaSuccess ||
+        (e = cudaMemsetAsync(v->flag_dev, 0, 2 * sizeof(int), v->stream)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(v->stream)) != cudaSuccess ||
+        (e = cudaMallocHost(&v->flag_host, kStageBytes)) != cudaSuccess) {
         cuda_fail(e, "view set-up");
         free_handle(v);
         return nullptr;
@@ -264,6 +266,15 @@ int run_query(stag_kde *h, const void *dQ, int64_t m, double *dOut, cudaStream_t
     return fail(STAG_KDE_EINVAL, "handle has an unknown form");
 }
 
+// The status words are zero when a host call begins (a call that ended early left them
+// unread) and again once it has read them.
+int status_begin(stag_kde *h) {
+    if (h->status_dirty) STAG_CUDA_TRY(cudaMemsetAsync(h->flag_dev, 0, 2 * sizeof(int), h->stream));
+    h->status_dirty = true;
+    return 0;
+}
+void status_end(stag_kde *h, bool set) { h->status_dirty = set; }
+
 size_t elem_size(int dtype) { return dtype == STAG_KDE_F64 ? sizeof(double) : sizeof(float); }
 
 }  // namespace
@@ -330,8 +341,10 @@ stag_kde_t *stag_kde_create_ex(const void *X, int dtype, int64_t n, int64_t d, d
         return bail("cudaDeviceGetAttribute", e);
     if ((e = cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking)) != cudaSuccess)
         return bail("cudaStreamCreate", e);
-    if ((e = dev_malloc(&h->flag_dev, sizeof(int))) != cudaSuccess) return bail("dev_malloc(flag)", e);
-    if ((e = cudaMallocHost(&h->flag_host, sizeof(int))) != cudaSuccess) return bail("cudaMallocHost", e);
+    if ((e = dev_malloc(&h->flag_dev, 2 * sizeof(int))) != cudaSuccess) return bail("dev_malloc(flag)", e);
+    if ((e = cudaMemsetAsync(h->flag_dev, 0, 2 * sizeof(int), h->stream)) != cudaSuccess)
+        return bail("cudaMemset(flag)", e);
+    if ((e = cudaMallocHost(&h->flag_host, kStageBytes)) != cudaSuccess) return bail("cudaMallocHost", e);
 
     const size_t bytes = (size_t)(n * d) * elem_size(dtype);
     if (dtype == STAG_KDE_F64) {
@@ -399,27 +412,27 @@ int stag_kde_query(stag_kde_t *h, const void *Q, int64_t m, double *out) {
     if (rc) return rc;
     rc = ensure_bytes((void **)&h->out_dev, &h->out_cap, m * 8);
     if (rc) return rc;
-    STAG_CUDA_TRY(cudaMemsetAsync(h->flag_dev, 0, sizeof(int), h->stream));
+    rc = status_begin(h);
+    if (rc) return rc;
     STAG_CUDA_TRY(cudaMemcpyAsync(h->q_dev, Q, qbytes, cudaMemcpyHostToDevice, h->stream));
     rc = run_query(h, h->q_dev, m, h->out_dev, h->stream, h->flag_dev);
     if (rc) {
         cudaStreamSynchronize(h->stream);
         return rc;
     }
-    // one synchronisation for both checks: the input flag and the kernel's error code
-    STAG_CUDA_TRY(cudaMemcpyAsync(h->flag_host, h->flag_dev, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    if (h->form == STAG_KDE_FORM_TC) {
-        rc = tc_error_enqueue(h, h->stream);
-        if (rc) {
-            cudaStreamSynchronize(h->stream);
-            return rc;
-        }
-    }
+    const bool staged = m <= kStageRows;
+    char *stage = reinterpret_cast<char *>(h->flag_host) + kStageOffset;
+    STAG_CUDA_TRY(cudaMemcpyAsync(h->flag_host, h->flag_dev, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if (staged) STAG_CUDA_TRY(cudaMemcpyAsync(stage, h->out_dev, m * 8, cudaMemcpyDeviceToHost, h->stream));
     STAG_CUDA_TRY(cudaStreamSynchronize(h->stream));
-    // (a set error code is cleared either way; the input error is the one reported)
-    const int terr = h->form == STAG_KDE_FORM_TC ? tc_error_take(h, h->stream) : 0;
-    if (*h->flag_host) return fail(STAG_KDE_EINVAL, "Q has a non-finite value or |q| > 1e15");
-    if (terr) return terr;
+    const int flag = h->flag_host[0], err = h->flag_host[1];
+    status_end(h, flag || err);
+    if (flag) return fail(STAG_KDE_EINVAL, "Q has a non-finite value or |q| > 1e15");
+    if (err) return fail(STAG_KDE_ETIMEDOUT, "tensor-core kernel: a bounded wait expired");
+    if (staged) {
+        memcpy(out, stage, m * 8);
+        return 0;
+    }
     STAG_CUDA_TRY(cudaMemcpyAsync(out, h->out_dev, m * 8, cudaMemcpyDeviceToHost, h->stream));
     STAG_CUDA_TRY(cudaStreamSynchronize(h->stream));
     return 0;
@@ -494,8 +507,9 @@ int stag_kde_query_subset(stag_kde_t *h, const float *Q, int64_t m, const int64_
         STAG_CUDA_TRY(cudaMemcpyAsync(dOff, off, (m + 1) * 8, cudaMemcpyHostToDevice, s));
         if (W && nnz > 0) STAG_CUDA_TRY(cudaMemcpyAsync(dW, W, nnz * 4, cudaMemcpyHostToDevice, s));
         STAG_CUDA_TRY(cudaMemcpyAsync(dQ, Q, m * h->d * 4, cudaMemcpyHostToDevice, s));
-        STAG_CUDA_TRY(cudaMemsetAsync(h->flag_dev, 0, sizeof(int), s));
-        int r = launch_check_finite_f32(dQ, m * h->d, h->flag_dev, s, 4);
+        int r = status_begin(h);
+        if (r) return r;
+        r = launch_check_finite_f32(dQ, m * h->d, h->flag_dev, s, 4);
         if (r) return r;
         for (int i = 0; i < 2; ++i) STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->copy_done[i], 0));
         r = subset_check_entries(dIdx, W ? dW : nullptr, nnz, h->n, h->flag_dev, s);
@@ -513,6 +527,7 @@ int stag_kde_query_subset(stag_kde_t *h, const float *Q, int64_t m, const int64_
         return rc;
     }
     STAG_CUDA_TRY(cudaStreamSynchronize(s));
+    status_end(h, *h->flag_host != 0);
     if (*h->flag_host & 4) return fail(STAG_KDE_EINVAL, "Q has a non-finite value or |q| > 1e15");
     if (*h->flag_host & 1) return fail(STAG_KDE_EINVAL, "an index is outside [0, n)");
     if (*h->flag_host & 2) return fail(STAG_KDE_EINVAL, "weights must be finite and >= 0");
