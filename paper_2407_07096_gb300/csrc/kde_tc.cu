@@ -26,7 +26,7 @@
 //               constant column), per point tile the B planes (v_hi, v_lo, -g pieces)
 //               and a metadata block (R of the unit's 128 queries, the tile's
 //               radius) into rings of stages;
-//   warp 1      allocates TMEM; one thread issues 3 * K/16 + 1 MMAs per accumulator
+//   warp 1      allocates TMEM; one thread issues 3 * ceil(d/16) + 1 MMAs per accumulator
 //               and commits. K = 16 ("ring"): four accumulators of 128 lanes x BN/2
 //               FP32 columns, half tile k into accumulator k mod 4; K >= 32: two
 //               accumulators of BN columns, tile t into accumulator t mod 2;
@@ -192,6 +192,7 @@ struct TcInst {
     float *part_shift;
     double *part_w;
     int64_t m, m_pad, n, T, q_tiles, tiles_per_split, unit_begin, units;
+    int ksteps;  // ceil(d / 16): the MMA K-steps that hold coordinates (the rest of Kp is zero)
 };
 
 // The instance owning global unit u (binary search over unit_begin).
@@ -465,72 +466,95 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
                 const uint32_t abase = a0 + ab * C::A_BYTES;
                 const uint32_t alo = ptx::smem_desc_lo(abase, 16);
                 const uint32_t alo_aug = ptx::smem_desc_lo(abase + 2 * C::A_PLANE, 16);
-                for (int64_t t = t0; t < t1 && ok; ++t, ++tcount) {
-                    const int sb = tcount % SB;
-                    if (!ptx::mbar_wait_bounded(&full_b[sb], (tcount / SB) & 1, wait_ns, abort_flag)) {
-                        timed_out();
-                        ok = false;
-                        break;
-                    }
-                    ptx::tc_fence_after();
-                    const uint32_t bbase = b0 + sb * C::B_BYTES;
-                    // 3 * K/16 + 1 MMAs: the split products, then the point term. Each operand's
-                    // descriptor is the stage's base low word plus a compile-time constant and a
-                    // constant high word, so the single issuing thread (which shares its
-                    // scheduler with epilogue warps) spends one add per operand: at K = 16 the
-                    // MMAs of a half tile are short and issue cost decides the pipe's rate.
-                    const uint32_t blo = ptx::smem_desc_lo(bbase, 16);
-                    const uint32_t blo_aug = ptx::smem_desc_lo(bbase + 2 * C::B_PLANE, 16);
-                    constexpr uint32_t HI = ptx::smem_desc_hi(G::SBO, G::SW);
-                    constexpr uint32_t HI_AUG = ptx::smem_desc_hi(256, ptx::kSw32);
-                    auto issue = [&](uint32_t d_tmem, uint32_t row0) {
-                        uint32_t accumulate = 0;
-#pragma unroll
-                        for (int prod = 0; prod < 3; ++prod) {
-                            // (u_hi, v_hi), (u_hi, v_lo), (u_lo, v_hi); B rows row0..
-#pragma unroll
-                            for (int s = 0; s < KP / 16; ++s) {
-                                const uint32_t aoff = (prod == 2 ? C::A_PLANE : 0) + G::koff(s, BM);
-                                const uint32_t boff =
-                                    (prod == 1 ? C::B_PLANE : 0) + row0 * G::CW * 2 + G::koff(s, BN);
-                                ptx::mma_f16_w(d_tmem, alo + (aoff >> 4), HI, blo + (boff >> 4), HI, C::IDESC,
-                                               accumulate);
-                                accumulate = 1;
-                            }
+                // The tile loop for KS K-steps: those that hold coordinates, ceil(d/16) of them (a
+                // K-step of padding adds zeros: d = 100 spends 22 MMAs per tile instead of 25,
+                // d = 43 spends 10 instead of 13). A constant, since a bound read in the loop
+                // costs the issuing thread a branch per MMA (d = 128: 2909 -> 3243 us).
+                auto run_tiles = [&](auto ks_c) {
+                    constexpr int KS = decltype(ks_c)::value;
+                    for (int64_t t = t0; t < t1 && ok; ++t, ++tcount) {
+                        const int sb = tcount % SB;
+                        if (!ptx::mbar_wait_bounded(&full_b[sb], (tcount / SB) & 1, wait_ns, abort_flag)) {
+                            timed_out();
+                            ok = false;
+                            break;
                         }
-                        // constant A column x (-g/2) pieces, one K = 16 step
-                        ptx::mma_f16_w(d_tmem, alo_aug, HI_AUG, blo_aug + ((row0 * 32) >> 4), HI_AUG, C::IDESC, 1);
-                    };
-                    if constexpr (C::RING) {
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const uint32_t k = 2 * tcount + h;  // half tile index, CTA-wide
-                            const int acc = k % C::NACC;
-                            if (!ptx::mbar_wait_bounded(&acc_empty[acc], ((k / C::NACC) & 1) ^ 1, wait_ns,
+                        ptx::tc_fence_after();
+                        const uint32_t bbase = b0 + sb * C::B_BYTES;
+                        // 3 * K/16 + 1 MMAs: the split products, then the point term. Each operand's
+                        // descriptor is the stage's base low word plus a compile-time constant and a
+                        // constant high word, so the single issuing thread (which shares its
+                        // scheduler with epilogue warps) spends one add per operand: at K = 16 the
+                        // MMAs of a half tile are short and issue cost decides the pipe's rate.
+                        const uint32_t blo = ptx::smem_desc_lo(bbase, 16);
+                        const uint32_t blo_aug = ptx::smem_desc_lo(bbase + 2 * C::B_PLANE, 16);
+                        constexpr uint32_t HI = ptx::smem_desc_hi(G::SBO, G::SW);
+                        constexpr uint32_t HI_AUG = ptx::smem_desc_hi(256, ptx::kSw32);
+                        auto issue = [&](uint32_t d_tmem, uint32_t row0) {
+                            uint32_t accumulate = 0;
+    #pragma unroll
+                            for (int prod = 0; prod < 3; ++prod) {
+                                // (u_hi, v_hi), (u_hi, v_lo), (u_lo, v_hi); B rows row0..
+    #pragma unroll
+                                for (int s = 0; s < KS; ++s) {
+                                    const uint32_t aoff = (prod == 2 ? C::A_PLANE : 0) + G::koff(s, BM);
+                                    const uint32_t boff =
+                                        (prod == 1 ? C::B_PLANE : 0) + row0 * G::CW * 2 + G::koff(s, BN);
+                                    ptx::mma_f16_w(d_tmem, alo + (aoff >> 4), HI, blo + (boff >> 4), HI, C::IDESC,
+                                                   accumulate);
+                                    accumulate = 1;
+                                }
+                            }
+                            // constant A column x (-g/2) pieces, one K = 16 step
+                            ptx::mma_f16_w(d_tmem, alo_aug, HI_AUG, blo_aug + ((row0 * 32) >> 4), HI_AUG, C::IDESC, 1);
+                        };
+                        if constexpr (C::RING) {
+    #pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const uint32_t k = 2 * tcount + h;  // half tile index, CTA-wide
+                                const int acc = k % C::NACC;
+                                if (!ptx::mbar_wait_bounded(&acc_empty[acc], ((k / C::NACC) & 1) ^ 1, wait_ns,
+                                                            abort_flag)) {
+                                    timed_out();
+                                    ok = false;
+                                    break;
+                                }
+                                ptx::tc_fence_after();
+                                issue(tmem_base + acc * C::ACC_COLS, h * C::ACC_COLS);
+                                ptx::mma_commit(&acc_full[acc]);
+                            }
+                        } else {
+                            const int acc = tcount % C::NACC;
+                            if (!ptx::mbar_wait_bounded(&acc_empty[acc], ((tcount / C::NACC) & 1) ^ 1, wait_ns,
                                                         abort_flag)) {
                                 timed_out();
                                 ok = false;
                                 break;
                             }
                             ptx::tc_fence_after();
-                            issue(tmem_base + acc * C::ACC_COLS, h * C::ACC_COLS);
+                            issue(tmem_base + acc * C::ACC_COLS, 0);
                             ptx::mma_commit(&acc_full[acc]);
                         }
-                    } else {
-                        const int acc = tcount % C::NACC;
-                        if (!ptx::mbar_wait_bounded(&acc_empty[acc], ((tcount / C::NACC) & 1) ^ 1, wait_ns,
-                                                    abort_flag)) {
-                            timed_out();
-                            ok = false;
-                            break;
-                        }
-                        ptx::tc_fence_after();
-                        issue(tmem_base + acc * C::ACC_COLS, 0);
-                        ptx::mma_commit(&acc_full[acc]);
+                        if (!ok) break;
+                        // the stage's operands are free once the tile's MMAs are done
+                        ptx::mma_commit(&empty_b[sb]);
                     }
-                    if (!ok) break;
-                    // the stage's operands are free once the tile's MMAs are done
-                    ptx::mma_commit(&empty_b[sb]);
+                };
+                using std::integral_constant;
+                if constexpr (KP == 128) {
+                    switch (I.ksteps) {
+                        case 5: run_tiles(integral_constant<int, 5>{}); break;
+                        case 6: run_tiles(integral_constant<int, 6>{}); break;
+                        case 7: run_tiles(integral_constant<int, 7>{}); break;
+                        default: run_tiles(integral_constant<int, 8>{}); break;
+                    }
+                } else if constexpr (KP == 64) {
+                    if (I.ksteps == 3)
+                        run_tiles(integral_constant<int, 3>{});
+                    else
+                        run_tiles(integral_constant<int, 4>{});
+                } else {
+                    run_tiles(integral_constant<int, KP / 16>{});
                 }
                 if (ok) ptx::mma_commit(&a_empty[ab]);
             }
@@ -552,7 +576,9 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
         constexpr int WCOLS = C::WCOLS;
         constexpr int NCH = WCOLS / 32;
         // Columns whose terms share one FP32 sum: half a tile (RING) or a quarter of one,
-        // whatever EG, so that the launch settings do not change a result's bits.
+        // whatever EG, so that the tuned setting does not change those sums. (The order in
+        // which a group meets its tiles still shows in the last bits: the compensated sum
+        // is exact to 2^-48 only where no term exceeds the sum before it.)
         constexpr int SUBCH = (C::RING ? BN / 2 : BN / 4) / 32;
         static_assert(SUBCH >= 1 && NCH % SUBCH == 0, "whole sums per visit");
         const int col0 = C::RING ? half * WCOLS : grp * WCOLS;   // first point column of the visit
@@ -1003,9 +1029,10 @@ struct RtInst {
     float c;
 };
 
+// KS: blocks of 16 coordinates that are summed, at least ceil(d / 16).
 // (kTable is a template parameter because a single instance's fields are then read where
 // they are used, from constant memory, and cost no registers)
-template <int KP, bool kTable>
+template <int KP, int KS, bool kTable>
 __global__ void __launch_bounds__(RowTermGeo::THREADS, KP <= 16 ? 3 : 2)
 tc_rowterm_kernel(const __grid_constant__ RtInst inst0, const RtInst *__restrict__ table, int n_inst) {
     int which = 0;
@@ -1101,7 +1128,8 @@ tc_rowterm_kernel(const __grid_constant__ RtInst inst0, const RtInst *__restrict
     // Stages: (chunk of 64 tiles, block of 16 coordinates). The centres (and, at a chunk's
     // first block, the tiles' radii) of the next stage are loaded into registers while the
     // current stage is computed, so the global-memory latency hides behind the math.
-    constexpr int NKB = KP / KC, PER = KC * TG / RG::THREADS;  // values a thread stages
+    // (KS blocks of 16 coordinates: those past d are zero on both sides)
+    constexpr int NKB = KS, PER = KC * TG / RG::THREADS;  // values a thread stages
     const int nstages = (int)ceil_div_dev(tb - ta, (int64_t)TG) * NKB;
     float pv[PER], prad = 0.f;
     auto load_stage = [&](int st) {
@@ -1161,7 +1189,7 @@ tc_rowterm_kernel(const __grid_constant__ RtInst inst0, const RtInst *__restrict
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int p = 0; p < 4; ++p) tot[j][p] = kb == 0 ? acc[j][p] : f2::add(tot[j][p], acc[j][p]);
-        if (kb + KC < KP) continue;
+        if (kb + KC < NKB * KC) continue;
         // the chunk's row terms (padding queries: 0) and the bounds
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -1618,24 +1646,30 @@ static int launch_rowterm(int Kp, const RtInst &r0, const RtInst *table, int n_i
     if (blocks > 0x7fffffff) return fail(STAG_KDE_EINVAL, "query batch too large");
     count_launch(1);
     switch (Kp) {
-#define STAG_ROWTERM(KPV)                                                                                          \
-    case KPV: {                                                                                                    \
-        /* set once per instantiation (before any stream capture can be in progress) */                           \
-        auto kern = table ? tc_rowterm_kernel<KPV, true> : tc_rowterm_kernel<KPV, false>;                         \
+#define STAG_ROWTERM(KPV, KSV)                                                                                     \
+    {                                                                                                              \
+        auto kern = table ? tc_rowterm_kernel<KPV, KPV / 16, true> : tc_rowterm_kernel<KPV, KSV, false>;          \
         constexpr int smem = RowTermGeo::smem_bytes(KPV);                                                          \
-        static cudaError_t attr0 = cudaFuncSetAttribute(tc_rowterm_kernel<KPV, false>,                            \
+        static cudaError_t attr0 = cudaFuncSetAttribute(tc_rowterm_kernel<KPV, KSV, false>,                       \
                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);       \
-        static cudaError_t attr1 = cudaFuncSetAttribute(tc_rowterm_kernel<KPV, true>,                             \
+        static cudaError_t attr1 = cudaFuncSetAttribute(tc_rowterm_kernel<KPV, KPV / 16, true>,                   \
                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);       \
         STAG_CUDA_TRY(attr0);                                                                                      \
         STAG_CUDA_TRY(attr1);                                                                                      \
         kern<<<(unsigned)blocks, RowTermGeo::THREADS, smem, s>>>(r0, table, n_inst);                              \
         break;                                                                                                     \
     }
-        STAG_ROWTERM(16)
-        STAG_ROWTERM(32)
-        STAG_ROWTERM(64)
-        STAG_ROWTERM(128)
+        // (a table's instances differ in d: every block of the width)
+        case 16: STAG_ROWTERM(16, 1)
+        case 32: STAG_ROWTERM(32, 2)
+        case 64:
+            if (!table && r0.d <= 48) STAG_ROWTERM(64, 3)
+            STAG_ROWTERM(64, 4)
+        case 128:
+            if (!table && r0.d <= 80) STAG_ROWTERM(128, 5)
+            if (!table && r0.d <= 96) STAG_ROWTERM(128, 6)
+            if (!table && r0.d <= 112) STAG_ROWTERM(128, 7)
+            STAG_ROWTERM(128, 8)
 #undef STAG_ROWTERM
     }
     STAG_CUDA_TRY(cudaGetLastError());
@@ -1681,6 +1715,7 @@ static void fill_inst(const stag_kde *h, int64_t m, int64_t q_tiles, int64_t spl
     I->tiles_per_split = tps;
     I->unit_begin = unit_begin;
     I->units = q_tiles * splits;
+    I->ksteps = (int)ceil_div(h->d, 16);
 }
 
 // The finish kernels' view of one instance (tc_finish.h).

@@ -60,15 +60,33 @@ def test_uneven_instances_in_one_launch():
     import torch
     from paper_2407_07096_gb300.kde import query_batch
     sizes = [(3317, 4200, 128, 1.0), (1500, 64, 8, 0.1), (70000, 300, 32, 3.0), (900, 1, 64, 0.5), (2500, 900, 128, 1.0)]
-    kdes, Qs, alone = [], [], []
-    for i, (n, m, d, a) in enumerate(sizes):
-        X, Q = _flagging(n, m, d, 50 + i)
-        kdes.append(_kde(X, a))
-        Qs.append(torch.from_numpy(Q).cuda())
-        alone.append(_kde(X, a).query(Q))
-    for _ in range(2):
-        outs = query_batch(kdes, Qs)
-        torch.cuda.synchronize()
-    for k, o, w in zip(kdes, outs, alone):
-        # the same bits: neither the launch settings nor the neighbours matter
-        np.testing.assert_allclose(o.cpu().numpy(), w, rtol=1e-12)
+    data = [_flagging(n, m, d, 50 + i) for i, (n, m, d, a) in enumerate(sizes)]
+    kdes = [_kde(X, s[3]) for (X, _), s in zip(data, sizes)]
+    Qs = [torch.from_numpy(Q).cuda() for _, Q in data]
+    outs = [o.clone() for o in query_batch(kdes, Qs)]
+    again = query_batch(kdes, Qs)
+    torch.cuda.synchronize()
+    for (X, Q), (n, m, d, a), o, o2 in zip(data, sizes, outs, again):
+        sel = np.unique(np.linspace(0, m - 1, 100).astype(int))
+        want = oracle.kde(X, Q[sel], a)
+        _, _, kappa = oracle.kde_log(X, Q[sel], a)
+        ok = want > 1e-290
+        assert np.all(oracle.rel_err(o.cpu().numpy()[sel], want)[ok] <= tol_tc(kappa, d)[ok])
+        assert torch.equal(o, o2)
+
+
+@pytest.mark.parametrize("d", [17, 32, 33, 48, 49, 64, 65, 80, 81, 96, 97, 112, 113, 128])
+def test_operand_steps(d):
+    # every number of 16-coordinate steps at both of its ends, alone and from a table
+    import torch
+    from paper_2407_07096_gb300.kde import query_batch
+    X, Q = _flagging(1300, 150, d, d)
+    a = 0.5 / d
+    want = oracle.kde(X, Q, a)
+    _, _, kappa = oracle.kde_log(X, Q, a)
+    with _kde(X, a) as kde, _kde(X[:700], a) as other:
+        got = kde.query(Q)
+        Qd = torch.from_numpy(Q).cuda()
+        batch = query_batch([other, kde], [Qd[:3], Qd])[1].cpu().numpy()
+    for v in (got, batch):
+        assert np.all(oracle.rel_err(v, want) <= tol_tc(kappa, d))
