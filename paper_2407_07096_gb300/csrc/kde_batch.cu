@@ -163,11 +163,7 @@ int build_tables(BatchPlan *p) {
             cl.work += (double)p->ms[i] * (double)h->n * pair_cost(Kp);
             ++cl.n_inst;
             FinInst f;
-            int cb, qb;
             tc_fill_fin(h, (const float *)p->qs[i], p->ms[i], p->splits[i], p->outs[i], &f);
-            fin_number(&f, h->sm_count, p->cblocks, p->qblocks, &cb, &qb);
-            p->cblocks += cb;
-            p->qblocks += qb;
             p->max_passes = std::max(p->max_passes, f.passes);
             p->max_d_pad = std::max(p->max_d_pad, h->d_pad);
             p->max_items += tc_max_fix_items(h, p->ms[i]);
@@ -182,6 +178,18 @@ int build_tables(BatchPlan *p) {
         STAG_CUDA_TRY(cudaMemcpy(cl.d_table, host.data(), host.size(), cudaMemcpyHostToDevice));
         STAG_CUDA_TRY(dev_malloc(&cl.d_rt, rt.size()));
         STAG_CUDA_TRY(cudaMemcpy(cl.d_rt, rt.data(), rt.size(), cudaMemcpyHostToDevice));
+    }
+    // the instances with the largest recompute items first (an item is `seg` tiles of up to
+    // 256 points against 64 queries: 0.7 ms of a block's time at d = 128, n = 2e5), so that
+    // the small ones fill the end of that phase
+    std::stable_sort(fin.begin(), fin.end(), [](const FinInst &a, const FinInst &b) {
+        return ((int64_t)a.seg << a.per_log) * a.d_pad > ((int64_t)b.seg << b.per_log) * b.d_pad;
+    });
+    for (FinInst &f : fin) {
+        int cb, qb;
+        fin_number(&f, p->hs[0]->sm_count, p->cblocks, p->qblocks, &cb, &qb);
+        p->cblocks += cb;
+        p->qblocks += qb;
     }
     p->n_fin = (int)fin.size();
     if (p->n_fin) {

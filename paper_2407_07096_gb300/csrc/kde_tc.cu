@@ -1163,7 +1163,9 @@ tc_rowterm_kernel(const __grid_constant__ RtInst inst0, const RtInst *__restrict
         if (kb == 0 && tid < TG) srad[tid] = prad;
         __syncthreads();
         if (st + 1 < nstages) load_stage(st + 1);
-        if (to >= gn) continue;  // all four of this thread's tiles lie past the range's end
+        // all four of this thread's tiles lie past the range's end, or all of its warp's
+        // queries are padding (a small batch; their row terms are never used)
+        if (to >= gn || q0 + wq * 32 >= m) continue;
         uint64_t acc[4][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j)

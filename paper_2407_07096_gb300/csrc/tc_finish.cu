@@ -3,10 +3,10 @@
 // over the tiles that can matter.
 //
 // Two launches, whatever the number of instances:
-//   fin_combine_kernel  one group of `lpq` lanes per query adds its ranges' partials (a
+//   fin_combine_kernel  a group of `lpq` lanes per query adds its ranges' partials (a
 //                       single thread per query walks them one latency at a time: 724 us
 //                       for 17 queries with 1200 ranges each; 32 lanes with eight loads in
-//                       flight each: 30 us);
+//                       flight each: 30 us, a block per query: 7);
 //   fin_fix_kernel      returns at once when no query is flagged. Otherwise its blocks
 //                       work through the phases below, taking work items from a counter
 //                       per phase and waiting for a phase's last item before the next.
@@ -121,9 +121,23 @@ fin_combine_kernel(const __grid_constant__ FinInst inst0, const FinInst *__restr
             wt += pw[(int64_t)k * m];
         }
     }
-    for (int o = lpq >> 1; o; o >>= 1) {
+    for (int o = min(lpq, 32) >> 1; o; o >>= 1) {
         tot += __shfl_xor_sync(0xffffffffu, tot, o);
         wt += __shfl_xor_sync(0xffffffffu, wt, o);
+    }
+    if (lpq == 256) {  // (one query per block: its eight warps)
+        __shared__ double part[2][8];
+        if ((tid & 31) == 0) {
+            part[0][tid >> 5] = tot;
+            part[1][tid >> 5] = wt;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < 8; ++w) {
+                tot += part[0][w];
+                wt += part[1][w];
+            }
+        }
     }
     if (j < m && sub == 0) {
         I.out[j] = ldexp(tot, cexp(I.part_shift[j])) * I.scale;
@@ -422,9 +436,8 @@ __device__ __forceinline__ void gather_group(const FinInst &I, int g, int F) {
     }
 }
 
-// Work item w of the instance: kept tiles [s * seg, min(kcount, (s + 1) * seg)) of its group.
-__device__ __forceinline__ void list_item(const FinInst &I, int G, int w, float *smem) {
-    const int g = find_owner(G, w, [&](int i) { return I.item_off[i]; });
+// Work item w of the instance: kept tiles [s * seg, min(kcount, (s + 1) * seg)) of its group g.
+__device__ __forceinline__ void list_item(const FinInst &I, int g, int w, float *smem) {
     const int k0 = (w - I.item_off[g]) * I.seg;
     const int k1 = min(I.kcount[g], k0 + I.seg);
     const int *list = I.kept + (int64_t)g * I.T + k0;
@@ -619,9 +632,18 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
                 },
                 item_begin, warp_sums);
     });
-    ok = ok && run(ok ? item_begin[n_inst] : 0, [&](int it) {
-        const int i = find_owner(n_inst, it, [&](int k) { return item_begin[k]; });
-        list_item(tab[i], group_begin[i + 1] - group_begin[i], it - item_begin[i], smem);
+    const int items = ok ? item_begin[n_inst] : 0;
+    int li = -1, lg = -1;  // instance and group of this block's last item
+    ok = ok && run(items, [&](int it) {
+        if (li < 0 || it < item_begin[li] || it >= item_begin[li + 1]) {
+            li = find_owner(n_inst, it, [&](int k) { return item_begin[k]; });
+            lg = -1;
+        }
+        const FinInst &I = tab[li];
+        const int w = it - item_begin[li];
+        if (lg < 0 || w < I.item_off[lg] || w >= I.item_off[lg + 1])
+            lg = find_owner(group_begin[li + 1] - group_begin[li], w, [&](int k) { return I.item_off[k]; });
+        list_item(I, lg, w, smem);
     });
     if (ok)
         run(groups, [&](int gg) {
@@ -690,6 +712,9 @@ void fin_number(FinInst *inst, int sm_count, int cblock, int qblock, int *cblock
     // do not fill the chip
     int lpq = 1;
     while (lpq < 32 && lpq * 8 <= inst->splits && inst->m * lpq < (int64_t)sm_count * 1024) lpq *= 2;
+    // few queries with hundreds of ranges each: a whole block per query (17 queries with 1200
+    // ranges: 30 -> 7 us)
+    if (lpq == 32 && inst->splits >= 256 && inst->m <= 2 * (int64_t)sm_count) lpq = 256;
     inst->lpq = lpq;
     inst->cblock_begin = cblock;
     inst->qblock_begin = qblock;

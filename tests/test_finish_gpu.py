@@ -90,3 +90,14 @@ def test_operand_steps(d):
         batch = query_batch([other, kde], [Qd[:3], Qd])[1].cpu().numpy()
     for v in (got, batch):
         assert np.all(oracle.rel_err(v, want) <= tol_tc(kappa, d))
+
+
+@pytest.mark.parametrize("n,m", [(70000, 31), (70000, 33), (300000, 97), (300000, 304), (300000, 305)])
+def test_few_queries_many_ranges(n, m):
+    # a whole block per query up to two queries per SM, warps of padding queries skipped
+    X, Q = _flagging(n, m, 20, n + m)
+    want = oracle.kde(X, Q, 0.02)
+    _, _, kappa = oracle.kde_log(X, Q, 0.02)
+    with _kde(X, 0.02) as kde:
+        got = kde.query(Q)
+    assert np.all(oracle.rel_err(got, want) <= tol_tc(kappa, 20))
