@@ -15,7 +15,7 @@
 // tensor-core work.)
 // The whole sequence is captured once into a CUDA graph and replayed on later calls with
 // the same handles, pointers and sizes. Before the first capture the autotuner times the
-// candidate (epilogue warp groups, tiles per unit) settings on the batch itself.
+// candidate numbers of point tiles per work unit on the batch itself.
 //
 // A query's result does not depend on the batch around it: every instance keeps its own
 // units, partials and combine, and a unit's arithmetic depends only on its own rows.
@@ -63,7 +63,6 @@ struct BatchPlan {
     int n_fin = 0, cblocks = 0, qblocks = 0, max_passes = 0, max_d_pad = 0;
     int64_t max_items = 0;
     bool recompute = false;
-    int eg = 4;
     int tiles_per_unit = 32;
     int *d_err = nullptr;
     int *h_err = nullptr;  // pinned copy written at the end of every replay
@@ -85,7 +84,7 @@ std::list<BatchPlan *> g_plans;  // most recently used first
 constexpr size_t kMaxPlans = 16;
 // settings chosen by the tuner per batch signature: a plan rebuilt after a scratch change
 // reuses them, so the work split (and hence every result bit) stays the same
-std::map<std::vector<uintptr_t>, std::pair<int, int>> g_tuned;
+std::map<std::vector<uintptr_t>, int> g_tuned;
 
 void free_tables(BatchPlan *p) {
     for (auto &c : p->classes) {
@@ -243,7 +242,7 @@ int enqueue(BatchPlan *p, cudaStream_t s) {
             units[w] = c.total_units;
             work[w] = c.work;
         }
-        rc = tc_launch_multi(p->eg, tables, n_inst, units, work, p->d_err, p->hs[0]->sm_count, p->wait_ns, s);
+        rc = tc_launch_multi(tables, n_inst, units, work, p->d_err, p->hs[0]->sm_count, p->wait_ns, s);
         if (!rc)
             rc = fin_launch(FinInst{}, (const FinInst *)p->d_fin, p->n_fin, p->cblocks, p->qblocks, p->max_passes,
                             p->max_d_pad, p->max_items, p->recompute, p->fin_ctl, p->d_err, p->hs[0]->sm_count,
@@ -253,47 +252,42 @@ int enqueue(BatchPlan *p, cudaStream_t s) {
     return rc;
 }
 
-// Times the candidate settings on the batch itself (uncaptured runs) and keeps the best.
+// Times the candidate unit sizes on the batch itself (uncaptured runs) and keeps the best.
+// (Epilogue groups: always four; two measured 2 to 5 % slower on every batch tried, 5 to 256
+// instances, and with one launch per width the difference is well above the timing noise.)
 int autotune(BatchPlan *p) {
     bool any_tc = false;
     for (auto *h : p->hs) any_tc |= is_tc(h);
     if (!any_tc) return 0;
-    const int egs[] = {2, 4};
     const int tpus[] = {16, 32, 64};
     cudaEvent_t e0, e1;
     STAG_CUDA_TRY(cudaEventCreate(&e0));
     STAG_CUDA_TRY(cudaEventCreate(&e1));
     float best = 1e30f;
-    int best_eg = 4, best_tpu = 32;
+    int best_tpu = 32;
     int rc = 0;
-    for (int eg : egs) {
-        for (int tpu : tpus) {
-            p->eg = eg;
-            p->tiles_per_unit = tpu;
-            if ((rc = reserve_all(p)) || (rc = build_tables(p))) break;
-            if ((rc = enqueue(p, p->cap))) break;  // warm-up
-            cudaEventRecord(e0, p->cap);
-            if ((rc = enqueue(p, p->cap))) break;
-            cudaEventRecord(e1, p->cap);
-            cudaError_t e = cudaEventSynchronize(e1);
-            if (e != cudaSuccess) {
-                rc = cuda_fail(e, "autotune");
-                break;
-            }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best) {
-                best = ms;
-                best_eg = eg;
-                best_tpu = tpu;
-            }
+    for (int tpu : tpus) {
+        p->tiles_per_unit = tpu;
+        if ((rc = reserve_all(p)) || (rc = build_tables(p))) break;
+        if ((rc = enqueue(p, p->cap))) break;  // warm-up
+        cudaEventRecord(e0, p->cap);
+        if ((rc = enqueue(p, p->cap))) break;
+        cudaEventRecord(e1, p->cap);
+        cudaError_t e = cudaEventSynchronize(e1);
+        if (e != cudaSuccess) {
+            rc = cuda_fail(e, "autotune");
+            break;
         }
-        if (rc) break;
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (ms < best) {
+            best = ms;
+            best_tpu = tpu;
+        }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) return rc;
-    p->eg = best_eg;
     p->tiles_per_unit = best_tpu;
     return 0;
 }
@@ -316,11 +310,10 @@ int build_plan(BatchPlan *p) {
     int rc = 0;
     auto tuned = g_tuned.find(p->key);
     if (tuned != g_tuned.end()) {
-        p->eg = tuned->second.first;
-        p->tiles_per_unit = tuned->second.second;
+        p->tiles_per_unit = tuned->second;
     } else {
         rc = autotune(p);
-        if (!rc) g_tuned[p->key] = {p->eg, p->tiles_per_unit};
+        if (!rc) g_tuned[p->key] = p->tiles_per_unit;
     }
     if (!rc) rc = reserve_all(p);
     if (!rc) rc = build_tables(p);

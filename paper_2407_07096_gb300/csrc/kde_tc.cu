@@ -1342,7 +1342,7 @@ int launch_multi_eg(const TcMulti &mp, int grid, int *err, uint64_t wait_ns, cud
 
 }  // namespace
 
-int tc_launch_multi(int eg, const void *const tables[4], const int n_inst[4], const int64_t units[4],
+int tc_launch_multi(const void *const tables[4], const int n_inst[4], const int64_t units[4],
                     const double work[4], int *err, int sm_count, uint64_t wait_ns, cudaStream_t s) {
     // CTAs per width in proportion to its work, at least one for a width with units and
     // never more than its units
@@ -1390,7 +1390,7 @@ int tc_launch_multi(int eg, const void *const tables[4], const int n_inst[4], co
         mp.cta_begin[c + 1] = mp.cta_begin[c] + cta[c];
     }
     if (total <= 0) return 0;
-    return eg == 2 ? launch_multi_eg<2>(mp, total, err, wait_ns, s) : launch_multi_eg<4>(mp, total, err, wait_ns, s);
+    return launch_multi_eg<4>(mp, total, err, wait_ns, s);
 }
 
 bool tc_supported(int64_t d) { return kp_for(d) != 0; }
@@ -1809,7 +1809,10 @@ int tc_query(stag_kde *h, const float *dQ, int64_t m, double *dOut, cudaStream_t
     rc = launch_tc_any(tc->Kp, h->tune_eg ? h->tune_eg : tc_epilogue_groups(), inst, nullptr, 1, inst.units,
                        tc->err, h->sm_count, h->wait_ns, s);
     prof_stop(h, s, (double)m * (double)h->n);
-    if (rc) return rc;
+    if (rc) {
+        cudaMemsetAsync(tc->ub, 0, round_up(m, BM) * sizeof(unsigned), s);  // (the combine will not)
+        return rc;
+    }
     return tc_finish(h, dQ, m, splits, dOut, s);
 }
 
