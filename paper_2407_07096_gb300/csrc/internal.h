@@ -104,6 +104,7 @@ struct stag_kde {
     double *f64_part = nullptr;
     unsigned *tickets = nullptr;
     void *view_scratch = nullptr;
+    cudaEvent_t f64_done = nullptr;  // the last FP64 query that used them (calls may come on several streams)
 
     // tensor-core form
     stagkde::TcData *tc = nullptr;

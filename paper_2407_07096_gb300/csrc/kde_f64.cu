@@ -245,6 +245,7 @@ int f64_set_scratch(stag_kde *h, void *p) {
     h->f64_part = static_cast<double *>(p);
     h->tickets = reinterpret_cast<unsigned *>(h->f64_part + f64_partials(h));
     STAG_CUDA_TRY(cudaMemsetAsync(h->tickets, 0, (size_t)h->sm_count * 8 * sizeof(unsigned), h->stream));
+    STAG_CUDA_TRY(cudaEventCreateWithFlags(&h->f64_done, cudaEventDisableTiming));
     return 0;
 }
 
@@ -252,6 +253,15 @@ int f64_query(stag_kde *h, const double *dQ, int64_t m, double *dOut, cudaStream
     if (h->d > kF64MaxD) return fail(STAG_KDE_EUNSUPPORTED, "FP64 form: d too large");
     const Split64 sp = split64(h, m);
     if (sp.q_tiles > 0x7fffffff) return fail(STAG_KDE_EINVAL, "query batch too large");
+    // Queries of one handle queued on several streams share the partial sums: each waits for
+    // the one before it (a captured query is ordered by its graph alone, like the other forms').
+    bool ordered = false;
+    if (sp.splits > 1) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        ordered = cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+        if (!ordered) cudaGetLastError();
+    }
+    if (ordered) STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->f64_done, 0));
     count_launch();
     prof_start(h, s);
     switch (h->kernel) {
@@ -266,6 +276,7 @@ int f64_query(stag_kde *h, const double *dQ, int64_t m, double *dOut, cudaStream
     }
     prof_stop(h, s, (double)m * (double)h->n);
     STAG_CUDA_TRY(cudaGetLastError());
+    if (ordered) STAG_CUDA_TRY(cudaEventRecord(h->f64_done, s));
     return 0;
 }
 

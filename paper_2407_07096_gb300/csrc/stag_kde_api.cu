@@ -146,6 +146,7 @@ void free_handle(stag_kde *h) {
     cudaFree(h->part.sum);
     cudaFree(h->part.shift);
     cudaFree(h->view_scratch);
+    if (h->f64_done) cudaEventDestroy(h->f64_done);
     cudaFree(h->flag_dev);
     if (h->flag_host) cudaFreeHost(h->flag_host);
     for (int i = 0; i < 2; ++i) {

@@ -51,3 +51,25 @@ def test_exponent_range():
     normal = want > 1e-307
     assert np.all(np.abs(got[normal] - want[normal]) <= 3 * 2.0 ** -53 * want[normal])
     assert np.all(np.abs(got[~normal] - want[~normal]) <= 2 * 5e-324 + 1e-15 * want[~normal])
+
+
+def test_queries_on_several_streams():
+    # queued on different streams without waiting: the handle's partial sums are shared
+    import torch
+    X, Q = mixture_inputs(11, 60000, 96, 5, dtype=np.float64)
+    with _kde(X, 0.2) as kde:
+        want = [kde.query(Q + 0.1 * i) for i in range(6)]
+        Qd = [torch.from_numpy(Q + 0.1 * i).cuda() for i in range(6)]
+        torch.cuda.synchronize()
+        streams = [torch.cuda.Stream() for _ in range(3)]
+        outs = [kde.query_dev(Qd[i], stream=streams[i % 3]) for i in range(6)]
+        torch.cuda.synchronize()
+        # and under capture (no allocation, no cross-stream wait)
+        g, out = torch.cuda.CUDAGraph(), torch.empty(96, dtype=torch.float64, device="cuda")
+        with torch.cuda.graph(g):
+            kde.query_dev(Qd[5], out)
+        g.replay()
+        torch.cuda.synchronize()
+    for o, w in zip(outs, want):
+        assert np.array_equal(o.cpu().numpy(), w)
+    assert np.array_equal(out.cpu().numpy(), want[5])
