@@ -19,8 +19,11 @@
 //    exp, below -745.2 the result is 0 in double.
 //  * the last block of a query tile to finish (an atomic ticket that wraps to zero by
 //    itself) adds the tile's partial sums in range order, so there is no combine launch.
-// Measured, n = m = 1000, d = 2, host call: 933 us before (902 us of it the kernel), 81 us
-// now.
+//  * a query under stream capture takes all ranges in one block per query tile (kOwn): its
+//    replays may overlap other queries of the handle, so it uses no shared partial sums.
+// Measured, n = m = 1000, d = 2: host call 933 us before (902 us of it the kernel), 70 us
+// now; on the device 901 -> 48 us, a replayed capture 900 -> 193 us. n = 1e5, m = 1, d = 8:
+// 124.8 ms -> 19 us, replayed 1.60 ms.
 // Sums: per thread in index order, then a fixed tree over the point lanes, then the ranges
 // in order: bitwise reproducible.
 #include <math.h>
@@ -87,8 +90,10 @@ __device__ __forceinline__ double reduce_lanes(double s, int ql, double *red) {
                             : 0.0;
 }
 
-// R points per thread and tile; ql = 1 << qlog.
-template <int KERN, int R>
+// R points per thread and tile; ql = 1 << qlog. kOwn: the block takes every range of points
+// of its queries in turn and combines them itself, in the order in which the last block of
+// the split form does (the same bits), without the handle's partial sums.
+template <int KERN, int R, bool kOwn>
 __global__ void __launch_bounds__(kThreads)
 kde_f64_kernel(const double *__restrict__ X, int64_t n, const double *__restrict__ Q, int64_t m, int d, double a,
                double scale, int qlog, int64_t tiles_per_split, double *part, unsigned *ticket,
@@ -97,6 +102,7 @@ kde_f64_kernel(const double *__restrict__ X, int64_t n, const double *__restrict
     __shared__ double sq[2][kKC * kMaxQl];
     __shared__ double tab[kTab];
     __shared__ double red[4 * kMaxQl];
+    __shared__ double own[kOwn ? kMaxQl : 1];
     __shared__ bool last;
     const int ql = 1 << qlog, pl = kThreads >> qlog, pts = pl * R;
     const int tid = threadIdx.x, j = tid & (ql - 1), p = tid >> qlog;
@@ -110,7 +116,7 @@ kde_f64_kernel(const double *__restrict__ X, int64_t n, const double *__restrict
         if (bad) atomicOr(flag, 1);
     }
     const int64_t tiles = (n + pts - 1) / pts;
-    const int64_t t0 = blockIdx.y * tiles_per_split, t1 = min(tiles, t0 + tiles_per_split);
+    const int64_t t0 = kOwn ? 0 : blockIdx.y * tiles_per_split, t1 = kOwn ? tiles : min(tiles, t0 + tiles_per_split);
     const int nch = (d + kKC - 1) / kKC;
 
     // chunk ch of point tile t, and (unless it is there already) of the queries
@@ -140,6 +146,8 @@ kde_f64_kernel(const double *__restrict__ X, int64_t n, const double *__restrict
     };
 
     double s = 0.0, d2[R];
+    double acc = 0.0;        // kOwn: the ranges whose number is p modulo pl
+    int64_t range = 0, in_range = 0;
 #pragma unroll
     for (int r = 0; r < R; ++r) d2[r] = 0.0;
     if (t0 < t1) load(0, t0, 0);
@@ -170,14 +178,25 @@ kde_f64_kernel(const double *__restrict__ X, int64_t n, const double *__restrict
                 if (p + r * pl < left && j < rows) s += term64<KERN>(a, d2[r], tab);
                 d2[r] = 0.0;
             }
+            if constexpr (kOwn) {
+                if (++in_range == tiles_per_split || t + 1 == t1) {
+                    const double v = reduce_lanes(s, ql, red);
+                    if (tid < ql) own[tid] = v;
+                    __syncthreads();
+                    if (p == (range & (pl - 1)) && j < rows) acc += own[j];
+                    s = 0.0;
+                    in_range = 0;
+                    ++range;
+                }
+            }
         }
         __syncthreads();  // the stage may be refilled
         st ^= 1;
         t = tn;
         ch = cn;
     }
-    s = reduce_lanes(s, ql, red);
-    if (gridDim.y == 1) {
+    s = reduce_lanes(kOwn ? acc : s, ql, red);
+    if (kOwn || gridDim.y == 1) {
         if (tid < rows) out[q0 + tid] = s * scale;
         return;
     }
@@ -217,17 +236,30 @@ Split64 split64(const stag_kde *h, int64_t m) {
     return s;
 }
 
-template <int KERN>
+template <int KERN, bool kOwn>
 void launch64(const stag_kde *h, const Split64 &sp, const double *dQ, int64_t m, double *dOut, int *dflag,
               cudaStream_t s) {
-    const dim3 grid((unsigned)sp.q_tiles, (unsigned)sp.splits);
+    const dim3 grid((unsigned)sp.q_tiles, kOwn ? 1u : (unsigned)sp.splits);
     const double scale = h->normalise ? 1.0 / (double)h->n : 1.0;
     if (sp.r == 4)
-        kde_f64_kernel<KERN, 4><<<grid, kThreads, 0, s>>>(h->x64, h->n, dQ, m, (int)h->d, h->a, scale, sp.qlog, sp.tps,
-                                                          h->f64_part, h->tickets, dOut, dflag);
+        kde_f64_kernel<KERN, 4, kOwn><<<grid, kThreads, 0, s>>>(h->x64, h->n, dQ, m, (int)h->d, h->a, scale, sp.qlog,
+                                                                sp.tps, h->f64_part, h->tickets, dOut, dflag);
     else
-        kde_f64_kernel<KERN, 1><<<grid, kThreads, 0, s>>>(h->x64, h->n, dQ, m, (int)h->d, h->a, scale, sp.qlog, sp.tps,
-                                                          h->f64_part, h->tickets, dOut, dflag);
+        kde_f64_kernel<KERN, 1, kOwn><<<grid, kThreads, 0, s>>>(h->x64, h->n, dQ, m, (int)h->d, h->a, scale, sp.qlog,
+                                                                sp.tps, h->f64_part, h->tickets, dOut, dflag);
+}
+
+template <bool kOwn>
+void launch64(const stag_kde *h, const Split64 &sp, const double *dQ, int64_t m, double *dOut, int *dflag,
+              cudaStream_t s) {
+    switch (h->kernel) {
+        case STAG_KDE_KERNEL_EXPONENTIAL:
+            return launch64<STAG_KDE_KERNEL_EXPONENTIAL, kOwn>(h, sp, dQ, m, dOut, dflag, s);
+        case STAG_KDE_KERNEL_LOGISTIC:
+            return launch64<STAG_KDE_KERNEL_LOGISTIC, kOwn>(h, sp, dQ, m, dOut, dflag, s);
+        default:
+            return launch64<STAG_KDE_KERNEL_GAUSSIAN, kOwn>(h, sp, dQ, m, dOut, dflag, s);
+    }
 }
 
 }  // namespace
@@ -254,26 +286,22 @@ int f64_query(stag_kde *h, const double *dQ, int64_t m, double *dOut, cudaStream
     const Split64 sp = split64(h, m);
     if (sp.q_tiles > 0x7fffffff) return fail(STAG_KDE_EINVAL, "query batch too large");
     // Queries of one handle queued on several streams share the partial sums: each waits for
-    // the one before it (a captured query is ordered by its graph alone, like the other forms').
-    bool ordered = false;
+    // the one before it. A captured query may be replayed beside any other and cannot wait
+    // for it: its blocks combine their own ranges.
+    bool own = false;
     if (sp.splits > 1) {
         cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-        ordered = cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
-        if (!ordered) cudaGetLastError();
+        STAG_CUDA_TRY(cudaStreamIsCapturing(s, &st));
+        own = st != cudaStreamCaptureStatusNone;
     }
+    const bool ordered = sp.splits > 1 && !own;
     if (ordered) STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->f64_done, 0));
     count_launch();
     prof_start(h, s);
-    switch (h->kernel) {
-        case STAG_KDE_KERNEL_EXPONENTIAL:
-            launch64<STAG_KDE_KERNEL_EXPONENTIAL>(h, sp, dQ, m, dOut, dflag, s);
-            break;
-        case STAG_KDE_KERNEL_LOGISTIC:
-            launch64<STAG_KDE_KERNEL_LOGISTIC>(h, sp, dQ, m, dOut, dflag, s);
-            break;
-        default:
-            launch64<STAG_KDE_KERNEL_GAUSSIAN>(h, sp, dQ, m, dOut, dflag, s);
-    }
+    if (own)
+        launch64<true>(h, sp, dQ, m, dOut, dflag, s);
+    else
+        launch64<false>(h, sp, dQ, m, dOut, dflag, s);
     prof_stop(h, s, (double)m * (double)h->n);
     STAG_CUDA_TRY(cudaGetLastError());
     if (ordered) STAG_CUDA_TRY(cudaEventRecord(h->f64_done, s));

@@ -64,12 +64,31 @@ def test_queries_on_several_streams():
         streams = [torch.cuda.Stream() for _ in range(3)]
         outs = [kde.query_dev(Qd[i], stream=streams[i % 3]) for i in range(6)]
         torch.cuda.synchronize()
-        # and under capture (no allocation, no cross-stream wait)
-        g, out = torch.cuda.CUDAGraph(), torch.empty(96, dtype=torch.float64, device="cuda")
-        with torch.cuda.graph(g):
-            kde.query_dev(Qd[5], out)
-        g.replay()
-        torch.cuda.synchronize()
     for o, w in zip(outs, want):
         assert np.array_equal(o.cpu().numpy(), w)
-    assert np.array_equal(out.cpu().numpy(), want[5])
+
+
+@pytest.mark.parametrize("kernel", ["gaussian", "exponential", "logistic"])
+@pytest.mark.parametrize("n,m,d", [(60000, 96, 5), (3001, 33, 9), (20000, 1, 3), (257, 6, 17)])
+def test_captured_queries_beside_others(n, m, d, kernel):
+    # replays on two streams and plain queries on a third: the same bits as one at a time
+    import torch
+    X, Q = mixture_inputs(12, n, m, d, dtype=np.float64)
+    with _kde(X, 0.2, kernel=kernel) as kde:
+        want = [kde.query(Q + 0.1 * i) for i in range(3)]
+        Qd = [torch.from_numpy(Q + 0.1 * i).cuda() for i in range(3)]
+        graphs = [torch.cuda.CUDAGraph() for _ in range(2)]
+        outs = [torch.empty(m, dtype=torch.float64, device="cuda") for _ in range(3)]
+        for i in range(2):
+            with torch.cuda.graph(graphs[i]):
+                kde.query_dev(Qd[i], outs[i])
+        torch.cuda.synchronize()
+        streams = [torch.cuda.Stream() for _ in range(3)]
+        for _ in range(4):
+            for i in range(2):
+                with torch.cuda.stream(streams[i]):
+                    graphs[i].replay()
+            kde.query_dev(Qd[2], outs[2], stream=streams[2])
+        torch.cuda.synchronize()
+        for o, w in zip(outs, want):
+            assert np.array_equal(o.cpu().numpy(), w)
