@@ -67,6 +67,9 @@ struct stag_lsh {
     void *host_q = nullptr;  // host API: device copies of Q and the offsets
     int64_t host_q_cap = 0;
     int64_t last_total = 0;  // size of the kept candidate lists (device query)
+    // after the last queued copy of the kept lists to the caller: the next query, whatever its
+    // stream, waits for it before it touches raw, scratch or cand
+    cudaEvent_t lists_read = nullptr;
     void *sort_buf = nullptr;  // raw candidate keys and radix-sort buffers (grown on demand)
     int64_t sort_cap = 0;
 };
@@ -558,7 +561,8 @@ lsh_bitmap1_kernel(const int64_t *__restrict__ range, int64_t m, int L, const ui
 // queries.)
 __global__ void __launch_bounds__(256)
 lsh_expand_kernel(const uint32_t *__restrict__ raw, const int64_t *__restrict__ raw_off, int64_t raw_stride,
-                  const int64_t *__restrict__ off, int64_t m, int64_t total, int span, int64_t *__restrict__ out) {
+                  int64_t raw_entries, const int64_t *__restrict__ off, int64_t m, int64_t total, int span,
+                  int64_t *__restrict__ out) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     // the last query in [lo, hi] whose list starts at or before output p: the owner of p
@@ -572,18 +576,20 @@ lsh_expand_kernel(const uint32_t *__restrict__ raw, const int64_t *__restrict__ 
         }
         return lo;
     };
+    // (a captured fetch may be replayed after another query has rewritten the offsets)
+    auto entry = [&](int64_t at) { return (uint64_t)at < (uint64_t)raw_entries ? (int64_t)raw[at] : (int64_t)-1; };
     for (int64_t s = (blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5)) * span; s < total;
          s += warps * span) {
         const int64_t end = min(total, s + span);
         const int64_t j0 = owner(0, m - 1, s), j1 = owner(j0, m - 1, end - 1);
         if (j0 == j1) {
-            const uint32_t *src = raw + (raw_off ? raw_off[j0] : j0 * raw_stride) - off[j0];
+            const int64_t at = (raw_off ? raw_off[j0] : j0 * raw_stride) - off[j0];
 #pragma unroll 8
-            for (int64_t i = s + lane; i < end; i += 32) out[i] = (int64_t)src[i];
+            for (int64_t i = s + lane; i < end; i += 32) out[i] = entry(at + i);
         } else {
             for (int64_t i = s + lane; i < end; i += 32) {
                 const int64_t j = owner(j0, j1, i);
-                out[i] = (int64_t)raw[(raw_off ? raw_off[j] : j * raw_stride) + (i - off[j])];
+                out[i] = entry((raw_off ? raw_off[j] : j * raw_stride) + (i - off[j]));
             }
         }
     }
@@ -706,18 +712,26 @@ int lsh_run_bitmap1(stag_lsh *h, const int32_t *HQ, int64_t *range, unsigned lon
     return 0;
 }
 
-// Writes the kept lists (int64, query order) to out (device) on stream s.
+// Writes the kept lists (int64, query order) to out (device) on stream s. What it queues reads
+// the handle's buffers after the call has returned, so it leaves an event for the next query
+// (and waits for the one before, which then covers every earlier copy on other streams). A
+// captured copy takes part in neither: its replays read what the buffers hold by then.
 int lsh_write_lists(stag_lsh *h, int64_t total, int64_t *out, cudaStream_t s) {
     if (total == 0) return 0;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    STAG_CUDA_TRY(cudaStreamIsCapturing(s, &st));
+    const bool ordered = st == cudaStreamCaptureStatusNone;
+    if (ordered) STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->lists_read, 0));
     if (!h->raw_lists) {
         STAG_CUDA_TRY(cudaMemcpyAsync(out, h->cand, total * 8, cudaMemcpyDeviceToDevice, s));
-        return 0;
+    } else {
+        count_launch();
+        const int span = (int)std::min<int64_t>(1024, std::max<int64_t>(32, round_up(total / (152 * 32), 32)));
+        lsh_expand_kernel<<<grid_for_elems(ceil_div(total, span) * 32, 256), 256, 0, s>>>(
+            (const uint32_t *)h->raw, h->raw_off, h->n, h->raw_cap / 4, h->own_off, h->last_m, total, span, out);
+        STAG_CUDA_TRY(cudaGetLastError());
     }
-    count_launch();
-    const int span = (int)std::min<int64_t>(1024, std::max<int64_t>(32, round_up(total / (152 * 32), 32)));
-    lsh_expand_kernel<<<grid_for_elems(ceil_div(total, span) * 32, 256), 256, 0, s>>>(
-        (const uint32_t *)h->raw, h->raw_off, h->n, h->own_off, h->last_m, total, span, out);
-    STAG_CUDA_TRY(cudaGetLastError());
+    if (ordered) STAG_CUDA_TRY(cudaEventRecord(h->lists_read, s));
     return 0;
 }
 
@@ -792,6 +806,7 @@ int lsh_run(stag_lsh *h, const float *dQ, int64_t m, int64_t *dOff, cudaStream_t
     // (m + 1 int64 each)
     const int64_t b_hq = round_up(m * nf * 4, 256), b_rng = round_up(m * L * 16, 256);
     const int64_t b_cnt = round_up(m * 8, 256), b_off = round_up((m + 1) * 8, 256);
+    STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->lists_read, 0));
     int rc = grow(&h->scratch, &h->scratch_cap, b_hq + b_rng + b_cnt + 2 * b_off);
     h->raw_lists = h->cand_ready = false;
     if (rc) return rc;
@@ -890,6 +905,7 @@ void free_lsh(stag_lsh *h) {
     cudaFree(h->dir);
     cudaFree(h->sort_buf);
     cudaFree(h->host_q);
+    if (h->lists_read) cudaEventDestroy(h->lists_read);
     if (h->stream) cudaStreamDestroy(h->stream);
     delete h;
 }
@@ -933,7 +949,8 @@ stag_lsh_t *stag_lsh_create(const float *X, int64_t n, int64_t d, int K, int L, 
     };
     cudaError_t e;
     if (!g.ok) return (cuda_fail(cudaErrorInvalidDevice, "cudaSetDevice"), bail(0));
-    if ((e = cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking)) != cudaSuccess)
+    if ((e = cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&h->lists_read, cudaEventDisableTiming)) != cudaSuccess)
         return (cuda_fail(e, "cudaStreamCreate"), bail(0));
     int32_t *H = nullptr;
     void *sortb = nullptr;

@@ -215,3 +215,62 @@ def test_one_pass_lists_at_their_limits(n, m):
         hoff, hidx = lsh.query(Q)
     assert np.array_equal(off.cpu().numpy(), woff) and np.array_equal(idx.cpu().numpy(), widx)
     assert np.array_equal(hoff, woff) and np.array_equal(hidx, widx)
+
+
+@pytest.mark.parametrize("m1", [40, 2000])  # lists at fixed and at measured offsets (m n 4 above 256 MB)
+@pytest.mark.parametrize("then", ["other stream", "host", "fetch on two streams"])
+def test_a_queued_fetch_is_not_overtaken_by_the_next_query(m1, then):
+    # the copy of the kept lists is queued behind 50 ms of other work on its stream; a query
+    # with other rows, on another stream, comes before it has run
+    import ctypes
+    import torch
+    from paper_2407_07096_gb300 import _lib
+    n, lib = 100_000, _lib.load()
+    r = np.random.default_rng(m1)
+    X = (r.standard_normal((n, 3)) * 6).astype(np.float32)
+    Q1 = torch.from_numpy(X[r.integers(0, n, m1)] + np.float32(0.1)).cuda()
+    Q2 = torch.from_numpy(X[r.integers(0, n, 33)] - np.float32(0.2)).cuda()
+    with _cls()(X, 3, 7, seed=4) as lsh:
+        want = [t.cpu().numpy() for Q in (Q1, Q2) for t in lsh.query_dev(Q)]
+        a, b = torch.cuda.Stream(), torch.cuda.Stream()
+        off, total = torch.empty(m1 + 1, dtype=torch.int64, device="cuda"), ctypes.c_int64()
+        torch.cuda.synchronize()
+        _lib.check(lib.stag_lsh_query_dev(lsh._h, Q1.data_ptr(), m1, off.data_ptr(), None, 0, ctypes.byref(total),
+                                          a.cuda_stream))
+        idx = [torch.full((total.value,), -7, dtype=torch.int64, device="cuda") for _ in range(2)]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(a):
+            torch.cuda._sleep(100_000_000)
+        _lib.check(lib.stag_lsh_fetch_dev(lsh._h, idx[0].data_ptr(), total.value, a.cuda_stream))
+        if then == "fetch on two streams":
+            _lib.check(lib.stag_lsh_fetch_dev(lsh._h, idx[1].data_ptr(), total.value, b.cuda_stream))
+        with torch.cuda.stream(b):
+            got2 = lsh.query(Q2.cpu().numpy()) if then == "host" else lsh.query_dev(Q2)
+        torch.cuda.synchronize()
+    assert np.array_equal(off.cpu().numpy(), want[0]) and np.array_equal(idx[0].cpu().numpy(), want[1])
+    if then == "fetch on two streams":
+        assert np.array_equal(idx[1].cpu().numpy(), want[1])
+    got2 = [np.asarray(t.cpu() if isinstance(t, torch.Tensor) else t) for t in got2]
+    assert np.array_equal(got2[0], want[2]) and np.array_equal(got2[1], want[3])
+
+
+def test_captured_fetch():
+    import ctypes
+    import torch
+    from paper_2407_07096_gb300 import _lib
+    lib = _lib.load()
+    X, Q = mixture_inputs(83, 4000, 90, 4)
+    with _cls()(X, 3, 6, seed=6) as lsh:
+        woff, widx = lsh.query(Q)
+        Qd = torch.from_numpy(Q).cuda()
+        off, total = torch.empty(91, dtype=torch.int64, device="cuda"), ctypes.c_int64()
+        idx = torch.zeros(len(widx), dtype=torch.int64, device="cuda")
+        torch.cuda.synchronize()
+        _lib.check(lib.stag_lsh_query_dev(lsh._h, Qd.data_ptr(), 90, off.data_ptr(), None, 0, ctypes.byref(total), None))
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            _lib.check(lib.stag_lsh_fetch_dev(lsh._h, idx.data_ptr(), total.value,
+                                              torch.cuda.current_stream().cuda_stream))
+        g.replay()
+        torch.cuda.synchronize()
+    assert np.array_equal(idx.cpu().numpy(), widx) and np.array_equal(off.cpu().numpy(), woff)
