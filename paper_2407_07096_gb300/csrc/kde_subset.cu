@@ -211,7 +211,9 @@ kde_subset16_kernel(const float *__restrict__ X, int64_t n, int d, int dp, const
                     total = issued;
                     return;
                 }
-                ngroups = gleft = (int)((n1 - n0 + 31) >> 5);
+                // (an end before its start counts as an empty list, as in the gather kernel: a
+                // negative count would take 2^32 steps to come back to 0)
+                ngroups = gleft = (int)((max(n1 - n0, (int64_t)0) + 31) >> 5);
                 ip = idx + n0 + lane;
                 iend = idx + n1;
                 if (kW) wp = W + n0 + lane;

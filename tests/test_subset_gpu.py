@@ -185,3 +185,20 @@ def test_staged_rows_edges(d, m, max_len):
         got = kde.query_subset_dev(torch.from_numpy(Q).cuda(), torch.from_numpy(off).cuda(),
                                    torch.from_numpy(bad).cuda(), torch.from_numpy(W).cuda()).cpu().numpy()
     _check(got, want, np.nan_to_num(kap), d)
+
+
+@pytest.mark.parametrize("d", [3, 16, 20])
+def test_a_list_that_ends_before_it_starts_is_empty(d):
+    # the device call does not check its offsets; such a list adds nothing and the lists
+    # beside it are not disturbed
+    import torch
+    K = _kde_cls()
+    X, Q = mixture_inputs(d, 400, 12, d)
+    off = np.array([0, 70, 69, 120, 89, 150, 118, 160, 127, 300, 20, 6000, 0], dtype=np.int64)
+    idx = np.random.default_rng(d).integers(0, 400, 6000).astype(np.int64)
+    with K(X, 0.3, form="simt_f32") as kde:
+        got = kde.query_subset_dev(torch.from_numpy(Q).cuda(), torch.from_numpy(off).cuda(),
+                                   torch.from_numpy(idx).cuda()).cpu().numpy()
+        for j in range(12):
+            want = kde.query_subset(Q[j:j + 1], np.array([0, max(0, off[j + 1] - off[j])]), idx[off[j]:off[j + 1]])
+            assert got[j] == want[0], j
