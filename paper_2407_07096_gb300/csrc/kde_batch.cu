@@ -245,8 +245,7 @@ int enqueue(BatchPlan *p, cudaStream_t s) {
         rc = tc_launch_multi(tables, n_inst, units, work, p->d_err, p->hs[0]->sm_count, p->wait_ns, s);
         if (!rc)
             rc = fin_launch(FinInst{}, (const FinInst *)p->d_fin, p->n_fin, p->cblocks, p->qblocks, p->max_passes,
-                            p->max_d_pad, p->max_items, p->recompute, p->fin_ctl, p->d_err, p->hs[0]->sm_count,
-                            p->wait_ns, s);
+                            p->max_d_pad, p->max_items, p->recompute, p->fin_ctl, p->d_err, p->hs[0]->sm_count, s);
     }
     if (!rc) rc = join(BatchPlan::kPrep, BatchPlan::kSide);
     return rc;

@@ -1763,7 +1763,7 @@ static int tc_finish(stag_kde *h, const float *dQ, int64_t m, int64_t splits, do
     int cblocks, qblocks;
     fin_number(&f, h->sm_count, 0, 0, &cblocks, &qblocks);
     return fin_launch(f, nullptr, 1, cblocks, qblocks, f.passes, h->d_pad, max_fix_items(m, tc->T), h->tc_check,
-                      tc->fin_ctl, tc->err, h->sm_count, h->wait_ns, s);
+                      tc->fin_ctl, tc->err, h->sm_count, s);
 }
 
 int tc_operand_width(const stag_kde *h) { return h->tc ? h->tc->Kp : 0; }

@@ -56,6 +56,11 @@ constexpr float kPruneLog2 = 64.f;
 // queries kept stay below ~7.2e-5 against the 1e-4 tolerance.
 constexpr double kTcErrThreshold = 7.5e-5;
 constexpr int kErrTimeout = 1;
+// A phase of the recompute gives up when none of its items is finished for this long. What is
+// waited for there is arithmetic, an item at a time (0.7 ms at n = 2e5, d = 128, growing with
+// n d: about half a second where the points fill the device's memory), so the handle's limit on
+// the pairwise kernel's hand-overs, which may be far shorter, does not apply.
+constexpr uint64_t kFixStallNs = 10000000000ull;
 constexpr int kFixThreads = simt::kThreads;  // 128: four warps
 constexpr int kQBlock = 256;                 // queries per block of the flag count
 constexpr int kSortChunk = 4096;             // entries per sort item
@@ -478,7 +483,7 @@ __device__ __forceinline__ void combine_group(const FinInst &I, int g, int F) {
 
 __global__ void __launch_bounds__(kFixThreads, 3)
 fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int n_inst, int qblocks, int max_passes,
-               FinCtl *ctl, int *err, uint64_t wait_ns) {
+               FinCtl *ctl, int *err) {
     extern __shared__ __align__(16) float smem[];
     RadixSmem &radix = *reinterpret_cast<RadixSmem *>(smem);  // (the sort's and the lists' phases take turns)
     __shared__ int s_item, s_ok, wcnt[8], warp_sums[kFixThreads / 32], sq[64];
@@ -510,11 +515,17 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
             }
         }
         if (tid == 0) {
-            const uint64_t t0 = ptx::globaltimer();
-            int ok = 1;
-            while (*reinterpret_cast<volatile int *>(&ctl->done[ph]) < N) {
+            uint64_t t0 = ptx::globaltimer();
+            int ok = 1, seen = 0;
+            while (true) {
+                const int done = *reinterpret_cast<volatile int *>(&ctl->done[ph]);
+                if (done >= N) break;
                 __nanosleep(100);
-                if (ptx::globaltimer() - t0 > wait_ns) {
+                const uint64_t now = ptx::globaltimer();
+                if (done != seen) {
+                    seen = done;
+                    t0 = now;
+                } else if (now - t0 > kFixStallNs) {
                     atomicExch(err, kErrTimeout);
                     ok = 0;
                     break;
@@ -724,7 +735,7 @@ void fin_number(FinInst *inst, int sm_count, int cblock, int qblock, int *cblock
 
 int fin_launch(const FinInst &inst0, const FinInst *table, int n_inst, int cblocks, int qblocks, int max_passes,
                int max_d_pad, int64_t max_items, bool recompute, FinCtl *ctl, int *err, int sm_count,
-               uint64_t wait_ns, cudaStream_t s) {
+               cudaStream_t s) {
     count_launch();
     fin_combine_kernel<<<(unsigned)cblocks, 256, 0, s>>>(inst0, table, n_inst, ctl);
     STAG_CUDA_TRY(cudaGetLastError());
@@ -736,7 +747,7 @@ int fin_launch(const FinInst &inst0, const FinInst *table, int n_inst, int cbloc
     count_launch();
     // (the ring's layout follows each instance's d_pad; the widest layout is the streamed one)
     const size_t smem = std::max(simt::simt_smem(std::min(max_d_pad, kSimtResidentMaxD)), simt::simt_smem(max_d_pad));
-    fin_fix_kernel<<<grid, kFixThreads, smem, s>>>(inst0, table, n_inst, qblocks, max_passes, ctl, err, wait_ns);
+    fin_fix_kernel<<<grid, kFixThreads, smem, s>>>(inst0, table, n_inst, qblocks, max_passes, ctl, err);
     STAG_CUDA_TRY(cudaGetLastError());
     return 0;
 }

@@ -50,6 +50,6 @@ void fin_number(FinInst *inst, int sm_count, int cblock, int qblock, int *cblock
 // NULL. recompute = false leaves the second out (no instance checks its results).
 int fin_launch(const FinInst &inst0, const FinInst *table, int n_inst, int cblocks, int qblocks, int max_passes,
                int max_d_pad, int64_t max_items, bool recompute, FinCtl *ctl, int *err, int sm_count,
-               uint64_t wait_ns, cudaStream_t s);
+               cudaStream_t s);
 
 }  // namespace stagkde

@@ -101,3 +101,25 @@ def test_few_queries_many_ranges(n, m):
     with _kde(X, 0.02) as kde:
         got = kde.query(Q)
     assert np.all(oracle.rel_err(got, want) <= tol_tc(kappa, 20))
+
+
+def test_short_wait_limit_does_not_cut_the_recompute_short():
+    # 5e5 points in 128 dimensions: a work item of the recompute takes more than a
+    # millisecond, three times the limit on the pairwise kernel's hand-overs; the query and
+    # the batch answer as they do at the default limit
+    import torch
+    from paper_2407_07096_gb300.kde import query_batch
+    r = np.random.default_rng(8)
+    X = r.standard_normal((500_000, 128), dtype=np.float32)
+    Q = r.standard_normal((300, 128), dtype=np.float32)
+    with _kde(X, 3.0) as kde:
+        want = kde.query(Q)
+        assert kde.last_recomputed() >= 250
+        kde.set_wait_limit(500_000)
+        got = kde.query(Q)
+        Qd, out = torch.from_numpy(Q).cuda(), torch.empty(300, dtype=torch.float64, device="cuda")
+        for _ in range(2):  # (a batch reports a wait that expired in its previous run)
+            query_batch([kde], [Qd], [out])
+            torch.cuda.synchronize()
+    assert np.array_equal(got, want)
+    assert np.all(np.abs(out.cpu().numpy() - want) <= 2e-4 * want)
