@@ -202,3 +202,41 @@ def test_a_list_that_ends_before_it_starts_is_empty(d):
         for j in range(12):
             want = kde.query_subset(Q[j:j + 1], np.array([0, max(0, off[j + 1] - off[j])]), idx[off[j]:off[j + 1]])
             assert got[j] == want[0], j
+
+
+def _time(f):
+    import torch
+    f()
+    torch.cuda.synchronize()
+    v = []
+    for _ in range(9):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(20):
+            f()
+        b.record()
+        torch.cuda.synchronize()
+        v.append(a.elapsed_time(b))
+    return sorted(v)[4]
+
+
+@pytest.mark.parametrize("d", [5, 16])
+def test_lanes_without_an_entry_cost_nothing_extra(d):
+    # lists of one entry against lists of 30, and lists of which every second entry is out of
+    # range against whole ones: no more time (twice, for the noise) although most lanes of a
+    # stage have nothing to do
+    import torch
+    K = _kde_cls()
+    n, r = 200_000, np.random.default_rng(d)
+    X = r.standard_normal((n, d), dtype=np.float32)
+    with K(X, 0.1, form="simt_f32") as kde:
+        def run(m, per, every=0):
+            off = torch.arange(m + 1, device="cuda") * per
+            idx = torch.from_numpy(r.integers(0, n, m * per)).cuda()
+            if every:
+                idx[::every] = -1
+            Q = torch.from_numpy(X[:m].copy()).cuda()
+            out = torch.empty(m, dtype=torch.float64, device="cuda")
+            return _time(lambda: kde.query_subset_dev(Q, off, idx, out=out))
+        assert run(100_000, 1) <= 2 * run(100_000, 30)
+        assert run(3000, 700, every=2) <= 2 * run(3000, 700)
