@@ -144,14 +144,15 @@ kde_subset_kernel(const float *__restrict__ X, int64_t n, int d, int dp, const f
 
 // Rows of at most 16 coordinates, staged. The instructions around the arithmetic decide. The
 // query stays in registers, the consumer counts its own groups of 32 entries (a query's first
-// stage carries its number and its group count), copies are predicated instead of branched
-// around, and a lane without an entry copies nothing, computes on what the stage held and adds
-// 0. (Copying row 0 for such lanes made every warp of the chip meet on one line of L2. Without
-// that, 1e5 lists of 100 entries, n = 1e6, d = 16: 622 -> 125 us; 1e5 lists of 3, n = 1e5, d = 5:
-// 589 -> 83; 3000 lists of 700 of which half is out of range, n = 1e6, d = 4: 231 -> 23.)
+// stage carries its number and its group count), copies take their size instead of a branch,
+// and a lane without an entry computes and adds 0. It copies a row that is its warp's own: with
+// row 0 for all of them every warp of the chip met on one line of L2. Without that, 1e5 lists of
+// 100 entries, n = 1e6, d = 16: 622 -> 125 us; 1e5 lists of 3, n = 1e5, d = 5: 589 -> 84; 3000
+// lists of 700 of which half is out of range, n = 1e6, d = 4: 231 -> 23. (Predicating the copies
+// instead is 1 to 2 % faster with weights, 3 % slower on long lists without.)
 // Measured, n = 1e6, d = 16, 1e5 lists of 1000 weighted entries: 1417 us with every lane loading
 // its own row, 1203 with staged rows, 909 with scale_down in place of ldexp, 822 in this form,
-// 782 without the branches, 672 with the idle lanes' copies left out. Two stages 50 % slower,
+// 782 without the branches, 669 with the idle lanes' own rows. Two stages 50 % slower,
 // four (three blocks per SM) 2 % slower, the index load outside a branch (it then sinks
 // to its use) twice as slow. X in L2 or not makes no difference: the time goes to L1 (row
 // copies, their reads, shuffles) and to issue.
@@ -162,7 +163,6 @@ struct __align__(128) SubStage16 {
     long long j;  // (first stage of a query)
     int groups;
 };
-constexpr unsigned kNoRow = 0xffffffffu;  // (a row starts at a 16-byte piece below it)
 constexpr size_t kSubSmem16 = sizeof(SubStage16) * kSubStages * kSubsetWarps;
 
 template <int KERN, bool kW, bool kFull>
@@ -183,6 +183,8 @@ kde_subset16_kernel(const float *__restrict__ X, int64_t n, int d, int dp, const
     const unsigned ring_a = (unsigned)__cvta_generic_to_shared(ring);
     const int64_t warps = (int64_t)gridDim.x * kSubsetWarps;
     const unsigned rowq = kFull ? 4u : dp / 4;  // 16-byte pieces per row
+    // what a lane without an entry copies: one row for the warp, another for most other warps
+    const unsigned idle_row = (unsigned)(((uint64_t)blockIdx.x * kSubsetWarps + warp) % (uint64_t)n) * rowq;
     // this lane copies piece `piece` of rows (lane / 4) + 8 i (a piece past the row's end:
     // zero bytes of it, so that the stage holds zeros there)
     const unsigned piece = lane & 3;
@@ -234,23 +236,19 @@ kde_subset16_kernel(const float *__restrict__ X, int64_t n, int d, int dp, const
     unsigned in = 0;      // byte offset of the stage to fill
     auto issue = [&]() {
         const bool ok = (unsigned long long)gi < (unsigned long long)n;
-        // (an entry out of range contributes nothing and is not followed; a lane without an
-        // entry copies nothing)
-        const unsigned row = ok ? (unsigned)gi * rowq : kNoRow;
+        // (an entry out of range contributes nothing and is not followed)
+        const unsigned row = ok ? (unsigned)gi * rowq : idle_row;
         counts = counts + counts + (ok ? 1u : 0u);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const unsigned r = __shfl_sync(0xffffffffu, row, (lane >> 2) + 8 * i);
             if (kFull)
-                asm volatile(
-                    "{\n.reg .pred p;\nsetp.ne.u32 p, %2, %3;\n@p cp.async.cg.shared.global [%0], [%1], 16;\n}\n" ::"r"(
-                        dst0 + in + 8 * i * kSubChunk * 4),
-                    "l"(xp + r), "r"(r), "n"(kNoRow));
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst0 + in + 8 * i * kSubChunk * 4),
+                             "l"(xp + r));
             else
-                asm volatile(
-                    "{\n.reg .pred p;\nsetp.ne.u32 p, %2, %3;\n@p cp.async.cg.shared.global [%0], [%1], 16, %4;\n}\n" ::"r"(
-                        dst0 + in + 8 * i * kSubChunk * 4),
-                    "l"(xp + r), "r"(r), "n"(kNoRow), "r"(bytes));
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst0 + in +
+                                                                                    8 * i * kSubChunk * 4),
+                             "l"(xp + r), "r"(bytes));
         }
         if (kW)
             asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 4, %2, %3;\n" ::"r"(
@@ -318,7 +316,7 @@ kde_subset16_kernel(const float *__restrict__ X, int64_t n, int d, int dp, const
         }
         const bool mine = (counts >> (S - 1)) & 1u;
         // one FP32 chain (the plain form's order; unused pieces add (0 - 0)^2). A lane without
-        // an entry works on the stage's old contents and adds 0.
+        // an entry works on its warp's idle row and adds 0.
         float4 xv[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) xv[v] = *reinterpret_cast<const float4 *>(&st->rows[src0 + ((v ^ swz) << 2)]);
