@@ -68,8 +68,10 @@ struct stag_lsh {
     int64_t host_q_cap = 0;
     int64_t last_total = 0;  // size of the kept candidate lists (device query)
     // after the last queued copy of the kept lists to the caller: the next query, whatever its
-    // stream, waits for it before it touches raw, scratch or cand
+    // stream, waits for it before it touches raw, scratch or cand (reading: one may be queued,
+    // no query has waited for it yet)
     cudaEvent_t lists_read = nullptr;
+    bool reading = false;
     void *sort_buf = nullptr;  // raw candidate keys and radix-sort buffers (grown on demand)
     int64_t sort_cap = 0;
 };
@@ -450,6 +452,7 @@ lsh_bitmap1_kernel(const int64_t *__restrict__ range, int64_t m, int L, const ui
     __shared__ int pref[2][65];
     __shared__ int warp_sums[kThreads / 32];
     constexpr int U = 8;  // members per thread loaded ahead
+    constexpr int R = 4;  // of the rest, members per thread in flight
     const int tid = threadIdx.x, lane = tid & 31;
     const int nsum = kSum ? (words + 31) / 32 : 0;
     uint32_t *sum = bm + words;
@@ -488,19 +491,48 @@ lsh_bitmap1_kernel(const int64_t *__restrict__ range, int64_t m, int L, const ui
         pref[buf][lane + 32] = half + ib - cb;
         if (lane == 31) pref[buf][64] = half + ib;
     };
-    // member f of the item in buffer buf, all ones past its end (indices are below 2^32 - 1)
-    auto member = [&](int buf, int f) -> uint32_t {
-        if (f >= pref[buf][64]) return 0xffffffffu;
-        int t = 0;  // the last table whose members start at or before f
+    // the table that member f of the item in buffer buf belongs to: the last one whose members
+    // start at or before f
+    auto table_of = [&](int buf, int f) {
+        int t = 0;
 #pragma unroll
         for (int step = 32; step; step >>= 1)
             if (pref[buf][t + step] <= f) t += step;
+        return t;
+    };
+    // member f, all ones past the item's end (indices are below 2^32 - 1)
+    auto member = [&](int buf, int f) -> uint32_t {
+        if (f >= pref[buf][64]) return 0xffffffffu;
+        const int t = table_of(buf, f);
         return ids[slo[buf][t] + (f - pref[buf][t])];
     };
     auto mark = [&](uint32_t i) {
         if (i != 0xffffffffu) {
             const uint32_t old = atomicOr(&bm[i >> 5], 1u << (i & 31));
             if (kSum && old == 0u) atomicOr(&sum[i >> 10], 1u << ((i >> 5) & 31));
+        }
+    };
+    // The members past the first U of every thread: the table advances with f (a search for
+    // each made queries with large buckets slower than the two-pass kernel), several loads in
+    // flight.
+    auto mark_rest = [&](int buf) {
+        const int members = pref[buf][64];
+        int f = tid + U * kThreads;
+        if (f >= members) return;
+        int t = table_of(buf, f);
+        for (; f < members; f += R * kThreads) {
+            uint32_t v[R];
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                const int g = f + u * kThreads;
+                v[u] = 0xffffffffu;
+                if (g < members) {
+                    while (pref[buf][t + 1] <= g) ++t;  // (ends: the last prefix is `members`)
+                    v[u] = ids[slo[buf][t] + (g - pref[buf][t])];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < R; ++u) mark(v[u]);
         }
     };
     if (tid < 32) {
@@ -516,7 +548,7 @@ lsh_bitmap1_kernel(const int64_t *__restrict__ range, int64_t m, int L, const ui
     for (int64_t j = blockIdx.x; j < m; j += gridDim.x, buf ^= 1) {
 #pragma unroll
         for (int u = 0; u < U; ++u) mark(iv[u]);
-        for (int f = tid + U * kThreads; f < pref[buf][64]; f += kThreads) mark(member(buf, f));
+        mark_rest(buf);
         if (tid < 32) publish(buf ^ 1);
         __syncthreads();
         // the next item's first members are on their way while this one's words are walked
@@ -577,7 +609,7 @@ lsh_expand_kernel(const uint32_t *__restrict__ raw, const int64_t *__restrict__ 
         return lo;
     };
     // (a captured fetch may be replayed after another query has rewritten the offsets)
-    auto entry = [&](int64_t at) { return (uint64_t)at < (uint64_t)raw_entries ? (int64_t)raw[at] : (int64_t)-1; };
+    auto entry = [&](int64_t at) { return (int64_t)raw[min((uint64_t)at, (uint64_t)raw_entries - 1)]; };
     for (int64_t s = (blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5)) * span; s < total;
          s += warps * span) {
         const int64_t end = min(total, s + span);
@@ -721,7 +753,8 @@ int lsh_write_lists(stag_lsh *h, int64_t total, int64_t *out, cudaStream_t s) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     STAG_CUDA_TRY(cudaStreamIsCapturing(s, &st));
     const bool ordered = st == cudaStreamCaptureStatusNone;
-    if (ordered) STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->lists_read, 0));
+    if (ordered && h->reading) STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->lists_read, 0));
+    h->reading |= ordered;
     if (!h->raw_lists) {
         STAG_CUDA_TRY(cudaMemcpyAsync(out, h->cand, total * 8, cudaMemcpyDeviceToDevice, s));
     } else {
@@ -806,7 +839,7 @@ int lsh_run(stag_lsh *h, const float *dQ, int64_t m, int64_t *dOff, cudaStream_t
     // (m + 1 int64 each)
     const int64_t b_hq = round_up(m * nf * 4, 256), b_rng = round_up(m * L * 16, 256);
     const int64_t b_cnt = round_up(m * 8, 256), b_off = round_up((m + 1) * 8, 256);
-    STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->lists_read, 0));
+    if (h->reading) STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->lists_read, 0));
     int rc = grow(&h->scratch, &h->scratch_cap, b_hq + b_rng + b_cnt + 2 * b_off);
     h->raw_lists = h->cand_ready = false;
     if (rc) return rc;
@@ -1053,6 +1086,7 @@ int stag_lsh_query_dev(stag_lsh_t *h, const float *dQ, int64_t m, int64_t *dOff,
     int rc = lsh_run(h, dQ, m, dOff, s, total);
     if (rc) return rc;
     h->last_total = *total;
+    h->reading = false;
     return dIdx && cap >= *total ? lsh_write_lists(h, *total, dIdx, s) : 0;
 }
 
@@ -1087,6 +1121,7 @@ int stag_lsh_query(stag_lsh_t *h, const float *Q, int64_t m, int64_t *off, int64
     rc = lsh_run(h, dQ, m, dOff, s, total);
     if (rc) return rc;
     h->last_total = *total;
+    h->reading = false;
     STAG_CUDA_TRY(cudaMemcpyAsync(off, dOff, (m + 1) * 8, cudaMemcpyDeviceToHost, s));
     if (idx && cap >= *total && *total > 0 && (rc = lsh_need_cand(h, *total, s))) {
         cudaStreamSynchronize(s);
