@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 
+#include "smem_opt_in.h"
 #include "stag_kde.h"
 
 namespace stagkde {

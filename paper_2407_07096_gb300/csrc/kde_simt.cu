@@ -145,9 +145,8 @@ int simt_prepare_points(stag_kde *h, const float *dX) {
 template <bool kQResident, bool kOneBlock, int KERN>
 int launch_simt_inst(const stag_kde *h, dim3 grid, cudaStream_t s, int64_t m, float negc, int64_t tps) {
     auto kern = kde_simt_f32_kernel<kQResident, kOneBlock, KERN>;
-    // set once per instantiation (before any stream capture can be in progress)
-    static const cudaError_t attr = allow_smem(kern);
-    STAG_CUDA_TRY(attr);
+    static SmemOptIn opt_in;
+    STAG_CUDA_TRY(opt_in((const void *)kern, kMaxSmem));
     kern<<<grid, kThreads, simt_smem(h->d_pad), s>>>(h->xt, h->n, h->n_tiles, h->qt, m, h->d_pad, negc, tps,
                                                      h->part.sum, h->part.shift);
     return 0;

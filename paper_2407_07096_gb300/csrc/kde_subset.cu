@@ -383,10 +383,8 @@ kde_subset16_kernel(const float *__restrict__ X, int64_t n, int d, int dp, const
 template <int KERN, bool kW, bool kFull>
 int launch16(const stag_kde *h, const float *dQ, int64_t m, const int64_t *dOff, const int64_t *dIdx, const float *dW,
              float negc, double scale, double *dOut, cudaStream_t s) {
-    // set once per instantiation (before any stream capture can be in progress)
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        kde_subset16_kernel<KERN, kW, kFull>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSubSmem16);
-    STAG_CUDA_TRY(attr);
+    static SmemOptIn opt_in;
+    STAG_CUDA_TRY(opt_in((const void *)kde_subset16_kernel<KERN, kW, kFull>, (int)kSubSmem16));
     // four blocks per SM are resident; several times as many even out ragged lists
     const unsigned grid =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(m, kSubsetWarps), (int64_t)h->sm_count * 12));

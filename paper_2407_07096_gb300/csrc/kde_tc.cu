@@ -1297,9 +1297,8 @@ int launch_tc(const TcInst &inst0, const TcInst *table, int n_inst, int64_t tota
     static_assert(C::SMEM <= 232448, "shared memory budget");
     // at least 116 KB so that no two CTAs share an SM (each holds up to 512 TMEM columns)
     const int smem = std::max(C::SMEM, 118 * 1024);
-    // set once per instantiation (before any stream capture can be in progress)
-    static cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    STAG_CUDA_TRY(attr);
+    static SmemOptIn opt_in;
+    STAG_CUDA_TRY(opt_in((const void *)kern, smem));
     const int grid = (int)std::min<int64_t>(total_units, sm_count);
     count_launch();
     kern<<<grid, C::THREADS, smem, s>>>(inst0, table, n_inst, total_units, err, wait_ns, stall_ns);
@@ -1331,9 +1330,8 @@ int launch_multi_eg(const TcMulti &mp, int grid, int *err, uint64_t wait_ns, cud
                                    Cfg<64, 256, 2, 8, 1, EG>::SMEM, Cfg<128, 128, 2, 8, 1, EG>::SMEM, 118 * 1024});
     static_assert(smem <= 232448, "shared memory budget");
     auto kern = kde_tc_multi_kernel<EG>;
-    // set once per instantiation (before any stream capture can be in progress)
-    static cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    STAG_CUDA_TRY(attr);
+    static SmemOptIn opt_in;
+    STAG_CUDA_TRY(opt_in((const void *)kern, smem));
     count_launch();
     kern<<<grid, 64 + 128 * EG, smem, s>>>(mp, err, wait_ns, stall_ns);
     STAG_CUDA_TRY(cudaGetLastError());
@@ -1652,12 +1650,8 @@ static int launch_rowterm(int Kp, const RtInst &r0, const RtInst *table, int n_i
     {                                                                                                              \
         auto kern = table ? tc_rowterm_kernel<KPV, KPV / 16, true> : tc_rowterm_kernel<KPV, KSV, false>;          \
         constexpr int smem = RowTermGeo::smem_bytes(KPV);                                                          \
-        static cudaError_t attr0 = cudaFuncSetAttribute(tc_rowterm_kernel<KPV, KSV, false>,                       \
-                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);       \
-        static cudaError_t attr1 = cudaFuncSetAttribute(tc_rowterm_kernel<KPV, KPV / 16, true>,                   \
-                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);       \
-        STAG_CUDA_TRY(attr0);                                                                                      \
-        STAG_CUDA_TRY(attr1);                                                                                      \
+        static SmemOptIn opt_in[2];                                                                                \
+        STAG_CUDA_TRY(opt_in[table ? 1 : 0]((const void *)kern, smem));                                            \
         kern<<<(unsigned)blocks, RowTermGeo::THREADS, smem, s>>>(r0, table, n_inst);                              \
         break;                                                                                                     \
     }

@@ -693,8 +693,8 @@ int launch_bitmap1(const stag_lsh *h, const int64_t *range, int64_t m, unsigned 
     const int words = (int)bitmap_words(h->n);
     const int smem = (words + (kSum ? (words + 31) / 32 : 0)) * 4;
     constexpr int kMost = (int)((kSum ? kMaxSliceWords + (kMaxSliceWords + 31) / 32 : kSumPoints / 32) * 4);
-    static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
-    STAG_CUDA_TRY(attr);
+    static SmemOptIn opt_in;
+    STAG_CUDA_TRY(opt_in((const void *)kern, kMost));
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(m, (int64_t)sms * (2048 / kThreads)));
     count_launch();
     kern<<<grid, kThreads, smem, s>>>(range, m, h->L, h->ids, words, h->raw_off, h->n, (uint32_t *)h->raw, ucount);
@@ -785,23 +785,11 @@ int lsh_run_bitmap(stag_lsh *h, const int32_t *HQ, int64_t *range, int64_t m, in
     const int64_t sw = bitmap_slice_words(h->n);
     const size_t smem = (size_t)(sw + 32) * 4;
     constexpr int kMaxSmem = (int)((kMaxSliceWords + 32) * 4);
-    static const cudaError_t attr = [] {
-        cudaError_t e = cudaFuncSetAttribute(lsh_bitmap_kernel<false, false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(lsh_bitmap_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kMaxSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(lsh_bitmap_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kMaxSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(lsh_bitmap_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kMaxSmem);
-        return e;
-    }();
-    STAG_CUDA_TRY(attr);
     auto count_k = slices > 1 ? lsh_bitmap_kernel<false, true> : lsh_bitmap_kernel<false, false>;
     auto write_k = slices > 1 ? lsh_bitmap_kernel<true, true> : lsh_bitmap_kernel<true, false>;
+    static SmemOptIn count_in[2], write_in[2];
+    STAG_CUDA_TRY(count_in[slices > 1]((const void *)count_k, kMaxSmem));
+    STAG_CUDA_TRY(write_in[slices > 1]((const void *)write_k, kMaxSmem));
     const int64_t b_cnt = round_up(items * 8, 256), b_off = round_up((items + 1) * 8, 256);
     int rc = grow(&h->sort_buf, &h->sort_cap, b_cnt + b_off);
     if (rc) return rc;

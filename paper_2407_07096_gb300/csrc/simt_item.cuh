@@ -311,12 +311,8 @@ inline size_t simt_smem(int d_pad) {
                                       : (size_t)kStages * 3 * kChunkBytes;
 }
 
-template <typename F>
-cudaError_t allow_smem(F *kern) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                std::max<int>(kStages * 3 * kChunkBytes,
-                                              kStages * kChunkBytes + kSimtResidentMaxD * kSimtTile * 8));
-}
+constexpr int kMaxSmem =
+    std::max(kStages * 3 * kChunkBytes, kStages * kChunkBytes + kSimtResidentMaxD * kSimtTile * 8);
 
 }  // namespace simt
 }  // namespace stagkde

@@ -740,9 +740,8 @@ int fin_launch(const FinInst &inst0, const FinInst *table, int n_inst, int cbloc
     fin_combine_kernel<<<(unsigned)cblocks, 256, 0, s>>>(inst0, table, n_inst, ctl);
     STAG_CUDA_TRY(cudaGetLastError());
     if (!recompute) return 0;
-    // set once (before any stream capture can be in progress)
-    static const cudaError_t attr = simt::allow_smem(fin_fix_kernel);
-    STAG_CUDA_TRY(attr);
+    static SmemOptIn opt_in;
+    STAG_CUDA_TRY(opt_in((const void *)fin_fix_kernel, simt::kMaxSmem));
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count * 3, max_items));
     count_launch();
     // (the ring's layout follows each instance's d_pad; the widest layout is the streamed one)
