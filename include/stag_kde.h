@@ -29,6 +29,10 @@
  *   - m = 0 is a valid no-op. n >= 1 and d >= 1 are required.
  *   - A handle may be used by one thread at a time. Results are deterministic: the same
  *     handle, inputs and options give bitwise-identical outputs on every call.
+ *   - The queries of a handle share its scratch memory. FP32 queries of one handle that overlap
+ *     on the device (on different streams, or a replayed graph beside another call) give
+ *     undefined results: queue them on one stream or order the streams. FP64 queries, subset
+ *     sums (device variant) and E2LSH queries may be queued on any streams.
  */
 #ifndef STAG_KDE_H
 #define STAG_KDE_H

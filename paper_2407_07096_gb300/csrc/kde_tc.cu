@@ -102,7 +102,8 @@ struct TcData {
     void *gbuf = nullptr;      // recompute scratch (fin_scratch_bytes), sized for gbuf_m rows
     int64_t gbuf_m = 0;
     int *fix_count = nullptr;  // device: number of queries handed to the plain form
-    FinCtl *fin_ctl = nullptr; // device: the recompute's phase counters
+    void *fin_ctl = nullptr;   // device: the recompute's phase counters, a slot per call (fin_ctl_slot)
+    unsigned fin_calls[2] = {0, 0};
     int *err = nullptr;        // device error code (timeouts): the handle's flag_dev + 1
 };
 
@@ -1517,6 +1518,21 @@ int tc_prepare_points(stag_kde *h, const float *dX) {
     return rc;
 }
 
+// The phase counters of a query's recompute. Its blocks wait for one another by them, so two
+// recomputes that overlap must not share them (one would reset the other's counts): queries
+// take the slots in turn, captured ones, whose replays keep theirs, from a set of their own.
+constexpr size_t kFinSlots = 64, kFinSlotBytes = 512;
+
+static int fin_ctl_slot(TcData *tc, cudaStream_t s, FinCtl **ctl) {
+    static_assert(sizeof(FinCtl) + 7 * sizeof(int) <= kFinSlotBytes, "one instance");
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    STAG_CUDA_TRY(cudaStreamIsCapturing(s, &st));
+    const int set = st != cudaStreamCaptureStatusNone;
+    const size_t slot = set * kFinSlots + tc->fin_calls[set]++ % kFinSlots;
+    *ctl = reinterpret_cast<FinCtl *>(static_cast<char *>(tc->fin_ctl) + slot * kFinSlotBytes);
+    return 0;
+}
+
 static int ensure_query_scratch(stag_kde *h, int64_t m_pad) {
     TcData *tc = h->tc;
     const int Kp = tc->Kp;
@@ -1550,7 +1566,7 @@ static int ensure_query_scratch(stag_kde *h, int64_t m_pad) {
         tc->unorm_cap = m_pad;
     }
     if (!tc->fix_count) STAG_CUDA_TRY(dev_malloc(&tc->fix_count, sizeof(int)));
-    if (!tc->fin_ctl) STAG_CUDA_TRY(dev_malloc(&tc->fin_ctl, fin_ctl_bytes(1)));
+    if (!tc->fin_ctl) STAG_CUDA_TRY(dev_malloc(&tc->fin_ctl, 2 * kFinSlots * kFinSlotBytes));
     const int64_t need = tc->T * m_pad;
     if (tc->rt_cap < need) {
         cudaFree(tc->rowterm);
@@ -1756,8 +1772,11 @@ static int tc_finish(stag_kde *h, const float *dQ, int64_t m, int64_t splits, do
     fill_fin(h, dQ, m, splits, dOut, &f);
     int cblocks, qblocks;
     fin_number(&f, h->sm_count, 0, 0, &cblocks, &qblocks);
-    return fin_launch(f, nullptr, 1, cblocks, qblocks, f.passes, h->d_pad, max_fix_items(m, tc->T), h->tc_check,
-                      tc->fin_ctl, tc->err, h->sm_count, s);
+    FinCtl *ctl;
+    int rc = fin_ctl_slot(tc, s, &ctl);
+    if (rc) return rc;
+    return fin_launch(f, nullptr, 1, cblocks, qblocks, f.passes, h->d_pad, max_fix_items(m, tc->T), h->tc_check, ctl,
+                      tc->err, h->sm_count, s);
 }
 
 int tc_operand_width(const stag_kde *h) { return h->tc ? h->tc->Kp : 0; }

@@ -28,6 +28,11 @@
 //                    at least one member), and its 64 queries in the plain form's layout;
 //   list             the plain form's work item over `seg` kept tiles of one group;
 //   combine          per query, the FP64 sum of its group's segments.
+// Two queries of one handle that overlap on the device (different streams, a replayed graph
+// beside other calls) share this scratch, so their results are undefined; what must not happen
+// is an access out of range or a wait that nobody ends. So each call has counters of its own
+// (fin_ctl_slot in kde_tc.cu), reads the number of flagged queries once, and every index that is
+// read back from the shared scratch is clamped before it is used as one.
 // Per query, from the row terms R_t = c ||q - c_t||^2 and the tiles' max radii rho_t (c = a
 // log2 e, exponents in log2 units):
 //     ub_t = -(max(0, sqrt(R_t) - sqrt(c) rho_t))^2  >= every exponent -c ||q - x||^2 in tile t
@@ -233,6 +238,9 @@ __device__ __forceinline__ void warp_leading_tile(const FinInst &I, float sqc, i
     }
 }
 
+// A row number or a position in the sorted arrays, in range whatever was read.
+__device__ __forceinline__ int clamp_row(const FinInst &I, uint32_t i) { return (int)min(i, (uint32_t)I.m - 1u); }
+
 // The flagged queries of block b (256 queries) in query order, from position w0 on.
 __device__ __forceinline__ void compact_block(const FinInst &I, int b, int w0, int *wcnt) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -278,7 +286,7 @@ __device__ __forceinline__ void compact_block(const FinInst &I, int b, int w0, i
                         }
                     }
                 }
-                const int at = w + __popc(mk & ((1u << lane) - 1u));
+                const int at = clamp_row(I, w + __popc(mk & ((1u << lane) - 1u)));
                 I.key[at] = (uint32_t)bt;
                 I.val[at] = (uint32_t)j;
                 I.thr[j] = best - kPruneLog2;
@@ -291,8 +299,9 @@ __device__ __forceinline__ void compact_block(const FinInst &I, int b, int w0, i
                 int bt;
                 warp_leading_tile(I, sqc, jq, best, bt);
                 if (lane == 0) {
-                    I.key[w] = (uint32_t)bt;
-                    I.val[w] = (uint32_t)jq;
+                    const int at = clamp_row(I, w);
+                    I.key[at] = (uint32_t)bt;
+                    I.val[at] = (uint32_t)jq;
                     I.thr[jq] = best - kPruneLog2;
                 }
             }
@@ -320,8 +329,8 @@ __device__ __forceinline__ void radix_count(RadixSmem &r, const uint32_t *ki, in
     for (int i = a + lane; i < b; i += 32) atomicAdd(&r.cnt[warp][(ki[i] >> shift) & 255u], 1u);
     __syncthreads();
 }
-__device__ __forceinline__ void radix_move(RadixSmem &r, const uint32_t *ki, const uint32_t *vi, uint32_t *ko,
-                                           uint32_t *vo, int e0, int e1, int shift) {
+__device__ __forceinline__ void radix_move(const FinInst &I, RadixSmem &r, const uint32_t *ki, const uint32_t *vi,
+                                           uint32_t *ko, uint32_t *vo, int e0, int e1, int shift) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int a, b;
     radix_range(e0, e1, a, b);
@@ -341,7 +350,7 @@ __device__ __forceinline__ void radix_move(RadixSmem &r, const uint32_t *ki, con
                 const uint32_t dg = (k[u] >> shift) & 255u;
                 const unsigned peers = __match_any_sync(act, dg);
                 const int rank = __popc(peers & ((1u << lane) - 1u));
-                const uint32_t at = r.cnt[warp][dg] + rank;
+                const int at = clamp_row(I, r.cnt[warp][dg] + rank);
                 ko[at] = k[u];
                 vo[at] = v[u];
                 __syncwarp(act);
@@ -375,14 +384,16 @@ __device__ __forceinline__ void sort_small(const FinInst &I, int F, RadixSmem &r
             at += c[u];
         }
         __syncthreads();
-        radix_move(r, ki, vi, ko, vo, 0, F, 8 * p);
+        radix_move(I, r, ki, vi, ko, vo, 0, F, 8 * p);
         __threadfence_block();
         __syncthreads();
     }
 }
 
-// Where an instance's sorted flagged queries end up.
-__device__ __forceinline__ const uint32_t *sorted_queries(const FinInst &I) { return I.passes & 1 ? I.vtmp : I.val; }
+// Flagged query j in sorted order.
+__device__ __forceinline__ int sorted_query(const FinInst &I, int j) {
+    return clamp_row(I, (I.passes & 1 ? I.vtmp : I.val)[j]);
+}
 
 // The tiles some member of group g may need, in increasing order; their number and the
 // group's segment count.
@@ -390,9 +401,8 @@ __device__ __forceinline__ void keep_group(const FinInst &I, int g, int F, int *
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rows = min(64, F - g * 64);
     const float sqc = sqrtf(I.c);
-    const uint32_t *order = sorted_queries(I);
     if (threadIdx.x < rows) {
-        const int q = (int)order[g * 64 + threadIdx.x];
+        const int q = sorted_query(I, g * 64 + threadIdx.x);
         sq[threadIdx.x] = q;
         sthr[threadIdx.x] = I.thr[q];
     }
@@ -432,27 +442,33 @@ __device__ __forceinline__ void keep_group(const FinInst &I, int g, int F, int *
 
 // Group g's queries, tile-transposed, every value twice (rows past the last are zero).
 __device__ __forceinline__ void gather_group(const FinInst &I, int g, int F) {
-    const uint32_t *order = sorted_queries(I);
     float2 *dst = reinterpret_cast<float2 *>(I.qt) + (int64_t)g * I.d_pad * kSimtTile;
     for (int e = threadIdx.x; e < I.d_pad * kSimtTile; e += kFixThreads) {
         const int r = e % kSimtTile, k = e / kSimtTile, j = g * 64 + r;
-        const float v = j < F && k < I.d ? I.Q[(int64_t)order[j] * I.d + k] : 0.f;
+        const float v = j < F && k < I.d ? I.Q[(int64_t)sorted_query(I, j) * I.d + k] : 0.f;
         dst[e] = make_float2(v, v);
     }
 }
 
+// Segments a group can have at most; work items of `groups` groups, from their prefix sum.
+__device__ __forceinline__ int max_segments(const FinInst &I) { return ((int)I.T + I.seg - 1) / I.seg; }
+__device__ __forceinline__ int items_before(const FinInst &I, int g, int groups) {
+    return min(max(I.item_off[g], 0), groups * max_segments(I));
+}
+
 // Work item w of the instance: kept tiles [s * seg, min(kcount, (s + 1) * seg)) of its group g.
 __device__ __forceinline__ void list_item(const FinInst &I, int g, int w, float *smem) {
-    const int k0 = (w - I.item_off[g]) * I.seg;
-    const int k1 = min(I.kcount[g], k0 + I.seg);
+    const int k0 = min(max(w - I.item_off[g], 0), max_segments(I) - 1) * I.seg;
+    const int k1 = min(min(I.kcount[g], (int)I.T), k0 + I.seg);
     const int *list = I.kept + (int64_t)g * I.T + k0;
     const int per_log = I.per_log, per = 1 << per_log;
     // the point set's last tile may cover fewer than `per` 64-point tiles; it can only be
     // the list's last entry (the lists ascend), whose tail is enumerated last
     int64_t nt = (int64_t)(k1 - k0) * per;
     if (k1 > k0) nt -= max((int64_t)0, ((int64_t)list[k1 - k0 - 1] + 1) * per - I.n_tiles);
-    auto tile_at = [list, per_log, per](int64_t i) {
-        return ((int64_t)list[i >> per_log] << per_log) + (i & (per - 1));
+    const uint64_t last = (uint64_t)I.n_tiles - 1;
+    auto tile_at = [list, per_log, per, last](int64_t i) {
+        return (int64_t)min((uint64_t)(((int64_t)list[i >> per_log] << per_log) + (i & (per - 1))), last);
     };
     const float *q = I.qt + (int64_t)g * I.d_pad * (2 * kSimtTile);
     double *ps = I.psum + (int64_t)w * kSimtTile;
@@ -467,9 +483,9 @@ __device__ __forceinline__ void list_item(const FinInst &I, int g, int w, float 
 }
 
 // Group g's results: two lanes per query over the group's segments.
-__device__ __forceinline__ void combine_group(const FinInst &I, int g, int F) {
+__device__ __forceinline__ void combine_group(const FinInst &I, int g, int F, int groups) {
     const int r = threadIdx.x >> 1, sub = threadIdx.x & 1;
-    const int w0 = I.item_off[g], w1 = I.item_off[g + 1];
+    const int w0 = items_before(I, g, groups), w1 = items_before(I, g + 1, groups);
     float smax = -INFINITY;
     for (int w = w0 + sub; w < w1; w += 2) smax = fmaxf(smax, I.pshift[(int64_t)w * 64 + r]);
     smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, 1));
@@ -478,7 +494,7 @@ __device__ __forceinline__ void combine_group(const FinInst &I, int g, int F) {
         tot += kfn::scale_down(I.psum[(int64_t)w * 64 + r], cexp(I.pshift[(int64_t)w * 64 + r] - smax));
     tot += __shfl_xor_sync(0xffffffffu, tot, 1);
     const int j = g * 64 + r;
-    if (sub == 0 && j < F) I.out[sorted_queries(I)[j]] = w1 > w0 ? ldexp(tot, cexp(smax)) * I.scale : 0.0;
+    if (sub == 0 && j < F) I.out[sorted_query(I, j)] = w1 > w0 ? ldexp(tot, cexp(smax)) * I.scale : 0.0;
 }
 
 __global__ void __launch_bounds__(kFixThreads, 3)
@@ -494,7 +510,7 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
     for (int i = tid; i < n_inst; i += kFixThreads) any |= *tab[i].fix_count > 0;
     if (!__syncthreads_or(any)) return;
     int *chunk_begin = reinterpret_cast<int *>(ctl + 1), *group_begin = chunk_begin + n_inst + 1,
-        *item_begin = group_begin + n_inst + 1;
+        *item_begin = group_begin + n_inst + 1, *flagged = item_begin + n_inst + 1;
 
     // One phase: its N items, whoever takes them, are done when this returns true.
     int phase = 0;
@@ -552,8 +568,11 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
             }
             if (tid == 0) I.bcnt[b] = c;
         } else {
-            scan_to(n_inst, [&](int i) { return sort_chunks(*tab[i].fix_count); }, chunk_begin, warp_sums);
-            scan_to(n_inst, [&](int i) { return (*tab[i].fix_count + 63) / 64; }, group_begin, warp_sums);
+            // (a thread scans the entries that it has written)
+            for (int i = tid; i < n_inst; i += kFixThreads)
+                flagged[i] = (int)min((int64_t)max(*tab[i].fix_count, 0), tab[i].m);
+            scan_to(n_inst, [&](int i) { return sort_chunks(flagged[i]); }, chunk_begin, warp_sums);
+            scan_to(n_inst, [&](int i) { return (flagged[i] + 63) / 64; }, group_begin, warp_sums);
         }
     });
     ok = ok && run(qblocks, [&](int it) {
@@ -566,7 +585,7 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
         compact_block(I, b, w0, wcnt);
     });
     ok = ok && run(n_inst, [&](int i) {
-        const int F = *tab[i].fix_count;
+        const int F = flagged[i];
         if (F > 0 && F <= kSortChunk) sort_small(tab[i], F, radix, warp_sums);
     });
     const int chunks = ok ? chunk_begin[n_inst] : 0;
@@ -576,7 +595,7 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
             const int i = find_owner(n_inst, it, [&](int k) { return chunk_begin[k]; });
             const FinInst &I = tab[i];
             if (p >= I.passes) return;
-            const int F = *I.fix_count, nb = sort_chunks(F), ch = it - chunk_begin[i];
+            const int F = flagged[i], nb = sort_chunks(F), ch = it - chunk_begin[i];
             body(I, nb, ch, ch * kSortChunk, min(F, (ch + 1) * kSortChunk));
         };
         ok = run(chunks, [&](int it) {
@@ -589,7 +608,7 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
         });
         ok = ok && run(n_inst, [&](int i) {
             const FinInst &I = tab[i];
-            const int nb = sort_chunks(*I.fix_count);
+            const int nb = sort_chunks(flagged[i]);
             if (nb == 0 || p >= I.passes) return;
             // exclusive scan in place: each thread a run of two digits' entries
             uint32_t *h = I.hist + (int64_t)tid * 2 * nb;
@@ -615,7 +634,7 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
                     }
                 }
                 __syncthreads();
-                radix_move(radix, ki, vi, p & 1 ? I.key : I.ktmp, p & 1 ? I.val : I.vtmp, e0, e1, 8 * p);
+                radix_move(I, radix, ki, vi, p & 1 ? I.key : I.ktmp, p & 1 ? I.val : I.vtmp, e0, e1, 8 * p);
             });
         });
     }
@@ -626,9 +645,9 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
         const int gg = it < groups ? it : it - groups, i = inst_of_group(gg);
         const FinInst &I = tab[i];
         if (it < groups)
-            keep_group(I, gg - group_begin[i], *I.fix_count, sq, sthr, wcnt);
+            keep_group(I, gg - group_begin[i], flagged[i], sq, sthr, wcnt);
         else
-            gather_group(I, gg - group_begin[i], *I.fix_count);
+            gather_group(I, gg - group_begin[i], flagged[i]);
     });
     ok = ok && run(n_inst, [&](int i) {
         const FinInst &I = tab[i];
@@ -639,7 +658,7 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
         scan_to(n_inst,
                 [&](int i) {
                     const int G = group_begin[i + 1] - group_begin[i];
-                    return G > 0 ? tab[i].item_off[G] : 0;
+                    return G > 0 ? items_before(tab[i], G, G) : 0;
                 },
                 item_begin, warp_sums);
     });
@@ -659,7 +678,7 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
     if (ok)
         run(groups, [&](int gg) {
             const int i = inst_of_group(gg);
-            combine_group(tab[i], gg - group_begin[i], *tab[i].fix_count);
+            combine_group(tab[i], gg - group_begin[i], flagged[i], group_begin[i + 1] - group_begin[i]);
         });
 }
 

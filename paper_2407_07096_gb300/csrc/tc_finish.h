@@ -37,8 +37,8 @@ struct FinInst {
 struct FinCtl {
     int claim[32], done[32];
 };
-// (behind it: three arrays of n_inst + 1 prefix sums)
-inline size_t fin_ctl_bytes(int64_t n_inst) { return sizeof(FinCtl) + 3 * (size_t)(n_inst + 1) * sizeof(int); }
+// (behind it: three arrays of n_inst + 1 prefix sums, and the instances' flag counts)
+inline size_t fin_ctl_bytes(int64_t n_inst) { return sizeof(FinCtl) + (4 * (size_t)n_inst + 3) * sizeof(int); }
 
 // Bytes of an instance's recompute scratch for up to m queries; with inst, also sets its
 // scratch pointers into base.

@@ -123,3 +123,34 @@ def test_short_wait_limit_does_not_cut_the_recompute_short():
             torch.cuda.synchronize()
     assert np.array_equal(got, want)
     assert np.all(np.abs(out.cpu().numpy() - want) <= 2e-4 * want)
+
+
+def test_overlapping_recomputes_end_and_leave_the_handle_usable():
+    # heavily flagged queries of one handle on two streams and in replayed graphs: their
+    # results are undefined (they share scratch), but they end promptly, without an error, and
+    # the next query is right
+    import time
+    import torch
+    d, ms = 64, (5000, 700, 4300)
+    X, Q = _flagging(4000, max(ms), d, 77)
+    with _kde(X, 1.0) as kde:
+        Qd = [torch.from_numpy(Q[:m]).cuda() for m in ms]
+        want = kde.query_dev(Qd[0]).clone()
+        assert kde.last_recomputed() > 4096
+        outs = [torch.empty(m, dtype=torch.float64, device="cuda") for m in ms]
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            kde.query_dev(Qd[2], outs[2])
+        streams = [torch.cuda.Stream() for _ in range(3)]
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        for _ in range(20):
+            for i in (0, 1):
+                kde.query_dev(Qd[i], outs[i], stream=streams[i])
+            with torch.cuda.stream(streams[2]):
+                g.replay()
+        torch.cuda.synchronize()
+        assert time.perf_counter() - t0 < 5.0  # (a recompute that waits in vain gives up after 10 s)
+        got = kde.query_dev(Qd[0])
+        assert torch.equal(got, want)
+        assert np.array_equal(kde.query(Q), want.cpu().numpy())  # (no status left behind)
