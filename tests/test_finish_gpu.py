@@ -154,3 +154,17 @@ def test_overlapping_recomputes_end_and_leave_the_handle_usable():
         got = kde.query_dev(Qd[0])
         assert torch.equal(got, want)
         assert np.array_equal(kde.query(Q), want.cpu().numpy())  # (no status left behind)
+
+
+@pytest.mark.parametrize("n,m,d,a", [(3317, 4600, 128, 1.0), (70000, 5000, 32, 3.0), (70000, 9000, 32, 3.0)])
+def test_chunked_sort_is_reached(n, m, d, a):
+    # more than 4096 flagged queries, tile indices of one and of two digits
+    X, Q = _flagging(n, m, d, n + m)
+    sel = np.unique(np.linspace(0, m - 1, 200).astype(int))
+    want = oracle.kde(X, Q[sel], a)
+    _, _, kappa = oracle.kde_log(X, Q[sel], a)
+    with _kde(X, a) as kde:
+        got = kde.query(Q)
+        assert kde.last_recomputed() > 4096
+    ok = want > 1e-290
+    assert np.all(oracle.rel_err(got[sel], want)[ok] <= tol_tc(kappa, d)[ok])
