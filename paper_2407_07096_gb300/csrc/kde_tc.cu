@@ -1561,8 +1561,10 @@ static int ensure_query_scratch(stag_kde *h, int64_t m_pad) {
         STAG_CUDA_TRY(dev_malloc(&tc->qbad, m_pad * sizeof(int)));
         STAG_CUDA_TRY(dev_malloc(&tc->ub, m_pad * sizeof(unsigned)));
         // (zero between calls: the row-term kernel raises them, the combine puts them back)
-        STAG_CUDA_TRY(cudaMemset(tc->ub, 0, m_pad * sizeof(unsigned)));
-        STAG_CUDA_TRY(cudaStreamSynchronize(nullptr));  // (the query's stream may not wait for this one)
+        // (on the handle's stream: one that waits for no other stream, so that a growth neither
+        // waits for work of the caller nor breaks a capture that is going on elsewhere)
+        STAG_CUDA_TRY(cudaMemsetAsync(tc->ub, 0, m_pad * sizeof(unsigned), h->stream));
+        STAG_CUDA_TRY(cudaStreamSynchronize(h->stream));
         tc->unorm_cap = m_pad;
     }
     if (!tc->fix_count) STAG_CUDA_TRY(dev_malloc(&tc->fix_count, sizeof(int)));

@@ -168,3 +168,32 @@ def test_chunked_sort_is_reached(n, m, d, a):
         assert kde.last_recomputed() > 4096
     ok = want > 1e-290
     assert np.all(oracle.rel_err(got[sel], want)[ok] <= tol_tc(kappa, d)[ok])
+
+
+def test_scratch_grows_beside_a_capture():
+    # a blocking stream is being captured when a handle on another stream sets up its scratch:
+    # both succeed (work on the legacy default stream would break the capture)
+    import ctypes
+    import os
+    import torch
+    rt = ctypes.CDLL(os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "lib64", "libcudart.so"))
+    X, Q = _flagging(3000, 200, 16, 5)
+    want = oracle.kde(X, Q, 0.1)
+    s = torch.cuda.Stream()
+    Qd, out = torch.from_numpy(Q).cuda(), torch.empty(200, dtype=torch.float64, device="cuda")
+    blocking, graph = ctypes.c_void_p(), ctypes.c_void_p()
+    with _kde(X, 0.1, form="tc") as kde:
+        torch.cuda.synchronize()
+        assert rt.cudaStreamCreate(ctypes.byref(blocking)) == 0
+        assert rt.cudaStreamBeginCapture(blocking, 2) == 0  # relaxed: allocations are allowed
+        try:
+            kde.query_dev(Qd, out, stream=s)
+        finally:
+            ended = rt.cudaStreamEndCapture(blocking, ctypes.byref(graph))
+            if graph.value:
+                rt.cudaGraphDestroy(graph)
+            rt.cudaStreamDestroy(blocking)
+        assert ended == 0
+        s.synchronize()
+    _, _, kappa = oracle.kde_log(X, Q, 0.1)
+    assert np.all(oracle.rel_err(out.cpu().numpy(), want) <= tol_tc(kappa, 16))
