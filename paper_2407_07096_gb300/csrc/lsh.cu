@@ -62,7 +62,9 @@ struct stag_lsh {
     void *raw = nullptr;
     int64_t raw_cap = 0;
     bool raw_lists = false, cand_ready = false;
-    const int64_t *raw_off = nullptr, *own_off = nullptr;  // (in scratch)
+    const int64_t *raw_off = nullptr;
+    int64_t *own_off = nullptr, *last_range = nullptr;  // (these and raw_off, last_hq: in scratch)
+    const int32_t *last_hq = nullptr;
     int64_t last_m = 0;
     void *host_q = nullptr;  // host API: device copies of Q and the offsets
     int64_t host_q_cap = 0;
@@ -644,6 +646,12 @@ int grow(void **p, int64_t *cap, int64_t bytes) {
     return 0;
 }
 
+void drop_raw(stag_lsh *h) {
+    cudaFree(h->raw);
+    h->raw = nullptr;
+    h->raw_cap = 0;
+}
+
 unsigned hash_grid_y(int64_t rows) { return (unsigned)ceil_div(rows, kHashRows); }
 
 int launch_hash(const stag_lsh *h, const float *X, int64_t rows, int32_t *H, cudaStream_t s) {
@@ -680,8 +688,8 @@ LshTables tables_of(const stag_lsh *h) {
 
 // One pass over the bitmaps: bucket ranges and sizes, their prefix sum, the 32-bit lists at
 // those offsets, the compact offsets. Taken while the upper bounds fit kMaxRawBytes (they
-// exceed the lists by the members that several tables share); *done says whether it was.
-// Synchronises the stream.
+// exceed the lists by the members that several tables share) and could be allocated; *done says
+// whether it was. Synchronises the stream.
 constexpr int64_t kMaxRawBytes = (int64_t)4 << 30;
 constexpr int64_t kFixedRawBytes = (int64_t)256 << 20;
 constexpr int64_t kSumPoints = (int64_t)1 << 17;  // above: summary bitmap, wider blocks
@@ -721,6 +729,10 @@ int lsh_run_bitmap1(stag_lsh *h, const int32_t *HQ, int64_t *range, unsigned lon
         if (R * 4 > kMaxRawBytes) return 0;
     }
     int rc = grow(&h->raw, &h->raw_cap, std::max<int64_t>(R, 1) * 4);
+    if (rc == STAG_KDE_ENOMEM) {  // the two passes need room for the distinct candidates only
+        cudaGetLastError();
+        return 0;
+    }
     if (rc) return rc;
     int sms = 0;
     STAG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
@@ -738,6 +750,8 @@ int lsh_run_bitmap1(stag_lsh *h, const int32_t *HQ, int64_t *range, unsigned lon
     STAG_CUDA_TRY(cudaMemcpyAsync(total, own_off + m, 8, cudaMemcpyDeviceToHost, s));
     STAG_CUDA_TRY(cudaStreamSynchronize(s));
     h->own_off = own_off;
+    h->last_hq = HQ;
+    h->last_range = range;
     h->last_m = m;
     h->raw_lists = true;
     *done = true;
@@ -766,15 +780,6 @@ int lsh_write_lists(stag_lsh *h, int64_t total, int64_t *out, cudaStream_t s) {
     }
     if (ordered) STAG_CUDA_TRY(cudaEventRecord(h->lists_read, s));
     return 0;
-}
-
-// The kept lists in h->cand (for copies to the host).
-int lsh_need_cand(stag_lsh *h, int64_t total, cudaStream_t s) {
-    if (!h->raw_lists || h->cand_ready) return 0;
-    int rc = grow(&h->cand, &h->cand_cap, std::max<int64_t>(total, 1) * 8);
-    if (!rc) rc = lsh_write_lists(h, total, (int64_t *)h->cand, s);
-    if (!rc) h->cand_ready = true;
-    return rc;
 }
 
 // The two-pass bitmap path of lsh_run: bucket ranges, distinct counts per (query, slice), their
@@ -808,6 +813,11 @@ int lsh_run_bitmap(stag_lsh *h, const int32_t *HQ, int64_t *range, int64_t m, in
     STAG_CUDA_TRY(cudaMemcpyAsync(&U, dOff + m, 8, cudaMemcpyDeviceToHost, s));
     STAG_CUDA_TRY(cudaStreamSynchronize(s));
     rc = grow(&h->cand, &h->cand_cap, std::max<int64_t>(U, 1) * 8);
+    if (rc == STAG_KDE_ENOMEM && h->raw) {  // (32-bit lists of an earlier query may take the room)
+        cudaGetLastError();
+        drop_raw(h);
+        rc = grow(&h->cand, &h->cand_cap, std::max<int64_t>(U, 1) * 8);
+    }
     if (rc) return rc;
     count_launch();
     write_k<<<grid, kBmThreads, smem, s>>>(range, m, h->L, h->ids, words, slices, sw, nullptr, item_off,
@@ -816,6 +826,27 @@ int lsh_run_bitmap(stag_lsh *h, const int32_t *HQ, int64_t *range, int64_t m, in
     STAG_CUDA_TRY(cudaStreamSynchronize(s));
     *total = U;
     return 0;
+}
+
+// The kept lists in h->cand (for copies to the host). Where there is no room for them beside the
+// 32-bit ones, those are given up and the two passes write the lists, from what the query left
+// in scratch.
+int lsh_need_cand(stag_lsh *h, int64_t total, cudaStream_t s) {
+    if (!h->raw_lists || h->cand_ready) return 0;
+    int rc = grow(&h->cand, &h->cand_cap, std::max<int64_t>(total, 1) * 8);
+    if (rc == STAG_KDE_ENOMEM) {
+        cudaGetLastError();
+        if (h->reading) STAG_CUDA_TRY(cudaStreamWaitEvent(s, h->lists_read, 0));
+        STAG_CUDA_TRY(cudaStreamSynchronize(s));
+        drop_raw(h);
+        h->raw_lists = false;
+        rc = lsh_run_bitmap(h, h->last_hq, h->last_range, h->last_m, h->own_off, s, &total);
+        if (rc) h->last_total = 0;
+        return rc;
+    }
+    if (!rc) rc = lsh_write_lists(h, total, (int64_t *)h->cand, s);
+    if (!rc) h->cand_ready = true;
+    return rc;
 }
 
 // Candidate lists of the device queries dQ into dOff (m + 1, device) and the handle's
@@ -1110,11 +1141,12 @@ int stag_lsh_query(stag_lsh_t *h, const float *Q, int64_t m, int64_t *off, int64
     if (rc) return rc;
     h->last_total = *total;
     h->reading = false;
-    STAG_CUDA_TRY(cudaMemcpyAsync(off, dOff, (m + 1) * 8, cudaMemcpyDeviceToHost, s));
     if (idx && cap >= *total && *total > 0 && (rc = lsh_need_cand(h, *total, s))) {
         cudaStreamSynchronize(s);
+        *total = 0;
         return rc;
     }
+    STAG_CUDA_TRY(cudaMemcpyAsync(off, dOff, (m + 1) * 8, cudaMemcpyDeviceToHost, s));
     if (idx && cap >= *total && *total > 0)
         STAG_CUDA_TRY(cudaMemcpyAsync(idx, h->cand, *total * 8, cudaMemcpyDeviceToHost, s));
     STAG_CUDA_TRY(cudaStreamSynchronize(s));

@@ -288,3 +288,42 @@ def test_large_buckets(n, L):
         woff, widx = oracle.lsh_candidates(oracle.lsh_hash(X, lsh.A, lsh.B), oracle.lsh_hash(Q, lsh.A, lsh.B), 1, L)
         off, idx = lsh.query_dev(torch.from_numpy(Q).cuda())
     assert np.array_equal(off.cpu().numpy(), woff) and np.array_equal(idx.cpu().numpy(), widx)
+
+
+@pytest.mark.parametrize("m", [60, 1500])  # lists at fixed and at measured offsets
+@pytest.mark.parametrize("way", ["host", "host with room", "device"])
+def test_lists_without_room_for_the_32_bit_copy(m, way, monkeypatch):
+    # each allocation of a first query fails in turn: those that the two-pass kernels can do
+    # without are done without, the others report out of memory; the next query is unharmed
+    import torch
+    from paper_2407_07096_gb300 import _lib as L
+    n = 60_000
+    r = np.random.default_rng(m)
+    X = (r.standard_normal((n, 3)) * 5).astype(np.float32)
+    Q = X[r.integers(0, n, m)] + np.float32(0.1)
+    answered = 0
+    for k in range(1, 8):
+        with _cls()(X, 3, 5, seed=9) as lsh:
+            if k == 1:
+                woff, widx = oracle.lsh_candidates(oracle.lsh_hash(X, lsh.A, lsh.B), oracle.lsh_hash(Q, lsh.A, lsh.B),
+                                                   3, 5)
+                room = (np.empty(m + 1, np.int64), np.empty(len(widx), np.int64))
+
+            def query():
+                if way == "device":
+                    return [t.cpu().numpy() for t in lsh.query_dev(torch.from_numpy(Q).cuda())]
+                return lsh.query(Q, out=room) if way == "host with room" else lsh.query(Q)
+            monkeypatch.setenv("STAG_KDE_INJECT_ALLOC_FAIL", str(k))
+            try:
+                off, idx = query()
+                assert np.array_equal(off, woff) and np.array_equal(idx, widx), k
+                answered |= 1 << k
+            except L.StagKdeError as e:
+                assert e.code == L.ENOMEM, (k, e)
+            finally:
+                monkeypatch.delenv("STAG_KDE_INJECT_ALLOC_FAIL")
+            off, idx = query()
+            assert np.array_equal(off, woff) and np.array_equal(idx, widx), k
+    # device: scratch, then the 32-bit lists; host: queries, scratch, the 32-bit lists, the lists
+    for k in ((2,) if way == "device" else (3, 4)):
+        assert answered >> k & 1, (k, bin(answered))
