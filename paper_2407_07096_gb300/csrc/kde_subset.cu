@@ -26,6 +26,7 @@
 #include <stddef.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 #include "kernel_fn.cuh"
@@ -165,7 +166,8 @@ struct __align__(128) SubStage16 {
 };
 constexpr size_t kSubSmem16 = sizeof(SubStage16) * kSubStages * kSubsetWarps;
 
-template <int KERN, bool kW, bool kFull>
+// kL1: rows are copied through L1 (see few_lines).
+template <int KERN, bool kW, bool kFull, bool kL1>
 __global__ void __launch_bounds__(32 * kSubsetWarps, 4)
 kde_subset16_kernel(const float *__restrict__ X, int64_t n, int d, int dp, const float *__restrict__ Q, int64_t m,
                     const int64_t *__restrict__ off, const int64_t *__restrict__ idx, const float *__restrict__ W,
@@ -242,13 +244,15 @@ kde_subset16_kernel(const float *__restrict__ X, int64_t n, int d, int dp, const
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const unsigned r = __shfl_sync(0xffffffffu, row, (lane >> 2) + 8 * i);
-            if (kFull)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst0 + in + 8 * i * kSubChunk * 4),
-                             "l"(xp + r));
+            const unsigned dst = dst0 + in + 8 * i * kSubChunk * 4;
+            if (kFull && kL1)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(xp + r));
+            else if (kFull)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(xp + r));
+            else if (kL1)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(xp + r), "r"(bytes));
             else
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst0 + in +
-                                                                                    8 * i * kSubChunk * 4),
-                             "l"(xp + r), "r"(bytes));
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(xp + r), "r"(bytes));
         }
         if (kW)
             asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 4, %2, %3;\n" ::"r"(
@@ -380,17 +384,28 @@ kde_subset16_kernel(const float *__restrict__ X, int64_t n, int d, int dp, const
     asm volatile("cp.async.wait_group 0;\n" ::);
 }
 
-template <int KERN, bool kW, bool kFull>
+template <int KERN, bool kW, bool kFull, bool kL1>
 int launch16(const stag_kde *h, const float *dQ, int64_t m, const int64_t *dOff, const int64_t *dIdx, const float *dW,
              float negc, double scale, double *dOut, cudaStream_t s) {
+    auto kern = kde_subset16_kernel<KERN, kW, kFull, kL1>;
     static SmemOptIn opt_in;
-    STAG_CUDA_TRY(opt_in((const void *)kde_subset16_kernel<KERN, kW, kFull>, (int)kSubSmem16));
+    STAG_CUDA_TRY(opt_in((const void *)kern, (int)kSubSmem16));
     // four blocks per SM are resident; several times as many even out ragged lists
     const unsigned grid =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(m, kSubsetWarps), (int64_t)h->sm_count * 12));
-    kde_subset16_kernel<KERN, kW, kFull><<<grid, 32 * kSubsetWarps, kSubSmem16, s>>>(
-        h->xrow, h->n, (int)h->d, h->d_pad, dQ, m, dOff, dIdx, dW, negc, scale, dOut);
+    kern<<<grid, 32 * kSubsetWarps, kSubSmem16, s>>>(h->xrow, h->n, (int)h->d, h->d_pad, dQ, m, dOff, dIdx, dW, negc,
+                                                    scale, dOut);
     return 0;
+}
+
+// Point sets of a few L2 lines, which every warp of the chip would ask for at once: their rows
+// are copied through L1, larger sets past it. Measured, 6e4 lists of 400, past / through L1, and
+// every lane gathering its own row: 32 points of 4 coordinates 3486 / 184 / 317 us, 512 points
+// 844 / 190 / 331, 2048 (32 KB) 251 / 228 / 332, 4096 184 / 235 / 332, 65536 181 / 243 / 334. Rows
+// of 12 coordinates do not divide a line: 170 points 1881 / 201 / 332, 2730 (128 KB) 369 / 269 /
+// 357, 4096 (192 KB) 266 / 272 / 370, 8192 212 / 276 / 391.
+bool few_lines(const stag_kde *h) {
+    return h->n * h->d_pad * 4 < (h->d_pad == 12 ? (int64_t)192 << 10 : (int64_t)64 << 10);
 }
 
 // Rows of at most 16 coordinates are staged (their offsets in 16-byte units must fit 32
@@ -401,12 +416,18 @@ int launch_kern(const stag_kde *h, const float *dQ, int64_t m, const int64_t *dO
     const float negc = (float)(-h->a * 1.4426950408889634);  // -a log2(e)
     const double scale = h->normalise ? 1.0 / (double)h->n : 1.0;
     if (h->d_pad <= kSubChunk && h->n * (h->d_pad / 4) <= 0xffffffffll) {
-        const bool full = h->d_pad == kSubChunk;
-        if (dW)
-            return full ? launch16<KERN, true, true>(h, dQ, m, dOff, dIdx, dW, negc, scale, dOut, s)
-                        : launch16<KERN, true, false>(h, dQ, m, dOff, dIdx, dW, negc, scale, dOut, s);
-        return full ? launch16<KERN, false, true>(h, dQ, m, dOff, dIdx, dW, negc, scale, dOut, s)
-                    : launch16<KERN, false, false>(h, dQ, m, dOff, dIdx, dW, negc, scale, dOut, s);
+        const bool full = h->d_pad == kSubChunk, l1 = few_lines(h);
+        auto go = [&](auto w, auto f, auto l) {
+            return launch16<KERN, decltype(w)::value, decltype(f)::value, decltype(l)::value>(
+                h, dQ, m, dOff, dIdx, dW, negc, scale, dOut, s);
+        };
+        const std::true_type yes{};
+        const std::false_type no{};
+        auto go_w = [&](auto w) {
+            if (full) return l1 ? go(w, yes, yes) : go(w, yes, no);
+            return l1 ? go(w, no, yes) : go(w, no, no);
+        };
+        return dW ? go_w(yes) : go_w(no);
     }
     const unsigned grid =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(m, kSubsetWarps), (int64_t)h->sm_count * 16));

@@ -240,3 +240,34 @@ def test_lanes_without_an_entry_cost_nothing_extra(d):
             return _time(lambda: kde.query_subset_dev(Q, off, idx, out=out))
         assert run(100_000, 1) <= 2 * run(100_000, 30)
         assert run(3000, 700, every=2) <= 2 * run(3000, 700)
+
+
+@pytest.mark.parametrize("d", [2, 11, 16])
+@pytest.mark.parametrize("n", [1, 7, 200, 1023, 1024, 1025, 4095, 4096, 4097])
+def test_few_points(n, d):
+    # point sets of a few cache lines are copied by another path, up to 64 KB (192 KB for rows
+    # of 12 coordinates): the sums on both sides of the line, and no more time than a set of
+    # 100 times as many (twice, for the noise)
+    import torch
+    K = _kde_cls()
+    r = np.random.default_rng(n + d)
+    X = r.standard_normal((n, d), dtype=np.float32)
+    Q = r.standard_normal((300, d), dtype=np.float32)
+    off, idx, W = _ragged(n, 300, n, 90)
+    want = oracle.kde_subset(X, Q, 0.2, off, idx, W)
+    kap = _kappa(X, Q, 0.2, off, idx, W, "gaussian")
+    big = r.standard_normal((100 * n + 20_000, d), dtype=np.float32)
+    with K(X, 0.2, form="simt_f32") as kde, K(big, 0.2, form="simt_f32") as other:
+        for w in (W, None):
+            got = kde.query_subset(Q, off, idx, w)
+            if w is not None:
+                _check(got, want, kap, d)
+            else:
+                _check(got, oracle.kde_subset(X, Q, 0.2, off, idx, np.ones(len(idx), np.float32)),
+                       _kappa(X, Q, 0.2, off, idx, np.ones(len(idx)), "gaussian"), d)
+        m, per = 20_000, 200
+        Qd = torch.randn(m, d, device="cuda")
+        o, out = torch.arange(m + 1, device="cuda") * per, torch.empty(m, dtype=torch.float64, device="cuda")
+        ids = [torch.randint(k.n, (m * per,), device="cuda") for k in (kde, other)]
+        small, large = (_time(lambda: k.query_subset_dev(Qd, o, i, out=out)) for k, i in zip((kde, other), ids))
+        assert small <= 2 * large
