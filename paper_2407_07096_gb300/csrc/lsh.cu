@@ -24,10 +24,10 @@
 // query at a time, sets a bit per bucket member in a shared-memory bitmap of the points and
 // walks it in index order, writing the list at an offset known from the bucket sizes (one
 // pass; the compact int64 lists are written when they are fetched). Up to 2^22 points, and
-// where those offsets would take too much memory, a block takes (query, slice) items in
-// two such walks (a counting pass, a prefix sum over the items, a writing pass). Beyond that, every bucket member is listed
-// (one warp per query) and repeats are removed by a radix sort of (query << 32 | index)
-// keys and a per-query unique pass.
+// where those offsets would take too much memory, a block takes (query, slice) items in two
+// such walks (a counting pass, a prefix sum over the items, a writing pass). Beyond that, every
+// bucket member is listed (one warp per query) and repeats are removed by a radix sort of
+// (query << 32 | index) keys and a per-query unique pass.
 #include <stdint.h>
 #include <stdlib.h>
 
@@ -200,8 +200,8 @@ __global__ void lsh_directory_kernel(const uint64_t *__restrict__ keys, int64_t 
 }
 
 // Per (query, table): the bucket's range in the sorted arrays (empty unless the first
-// member's K values equal the query's: exact membership); per query: the total. Bound by the
-// its scattered loads: n = 1e6, L = 50, 1e4 queries: 469 us with two binary searches over the
+// member's K values equal the query's: exact membership); per query: the total. Bound by its
+// scattered loads: n = 1e6, L = 50, 1e4 queries: 469 us with two binary searches over the
 // whole table and the tuple check reading rows of A per lane, 311 with the key directory,
 // 130 with the functions coordinate-major (a warp's lanes are consecutive tables).
 __global__ void lsh_lookup_kernel(const int32_t *__restrict__ HQ, int64_t m, LshTables t, int64_t *__restrict__ range,
@@ -589,10 +589,10 @@ lsh_bitmap1_kernel(const int64_t *__restrict__ range, int64_t m, int L, const ui
 }
 
 // out[off[j] + i] = raw[r(j) + i], r(j) = raw_off[j], or j * raw_stride: a warp takes `span`
-// consecutive outputs at a time (1024, fewer when that leaves warps idle) and finds the queries of the first and the last of them;
-// one query (long lists): a plain copy, else every lane searches between the two. (Walking
-// from list to list instead takes one latency per query: 287 us for 340 candidates of 1721
-// queries.)
+// consecutive outputs at a time (1024, fewer when that leaves warps idle) and finds the queries
+// of the first and the last of them; one query (long lists): a plain copy, else every lane
+// searches between the two. (Walking from list to list instead takes one latency per query: 287
+// us for 340 candidates of 1721 queries.)
 __global__ void __launch_bounds__(256)
 lsh_expand_kernel(const uint32_t *__restrict__ raw, const int64_t *__restrict__ raw_off, int64_t raw_stride,
                   int64_t raw_entries, const int64_t *__restrict__ off, int64_t m, int64_t total, int span,
@@ -737,7 +737,13 @@ int lsh_run_bitmap1(stag_lsh *h, const int32_t *HQ, int64_t *range, unsigned lon
     int sms = 0;
     STAG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     h->raw_off = fixed ? nullptr : raw_off;
-    if (h->n <= kSumPoints)
+    // (up to one query per SM: nothing shares its SM, so the widest block; m = 20, n = 1e5, K = 2,
+    // L = 40: 182 us with 256 threads, 132 with 1024; m = 3, n = 8e5, L = 20: 612 and 500)
+    if (h->n <= kSumPoints && m <= sms)
+        rc = launch_bitmap1<1024, false>(h, range, m, count, sms, s);
+    else if (m <= sms)
+        rc = launch_bitmap1<1024, true>(h, range, m, count, sms, s);
+    else if (h->n <= kSumPoints)
         rc = launch_bitmap1<256, false>(h, range, m, count, sms, s);
     else if (bitmap_words(h->n) <= 27648)  // two blocks' bitmaps fit one SM
         rc = launch_bitmap1<512, true>(h, range, m, count, sms, s);

@@ -276,14 +276,16 @@ def test_captured_fetch():
     assert np.array_equal(idx.cpu().numpy(), widx) and np.array_equal(off.cpu().numpy(), woff)
 
 
+@pytest.mark.parametrize("copies", [1, 20])  # up to one query per SM (1024 threads each), and more
 @pytest.mark.parametrize("n,L", [(300, 1), (2049, 1), (3000, 63), (140_000, 5), (890_000, 3)])
-def test_large_buckets(n, L):
+def test_large_buckets(n, L, copies):
     # one function per table: buckets of about a third of the points, far more members than the
     # threads load ahead (8 each of 256, 512 and 1024), over one or many tables
     import torch
     r = np.random.default_rng(n)
     X = r.standard_normal((n, 2)).astype(np.float32) * 3
     Q = np.concatenate([X[:5] + np.float32(0.01), np.full((1, 2), 1e6, np.float32), X[5:8]])
+    Q = np.concatenate([Q + np.float32(0.3 * i) for i in range(copies)])
     with _cls()(X, 1, L, seed=3) as lsh:
         woff, widx = oracle.lsh_candidates(oracle.lsh_hash(X, lsh.A, lsh.B), oracle.lsh_hash(Q, lsh.A, lsh.B), 1, L)
         off, idx = lsh.query_dev(torch.from_numpy(Q).cuda())
