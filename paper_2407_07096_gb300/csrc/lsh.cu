@@ -168,7 +168,7 @@ __device__ __forceinline__ int64_t lower_bound(const uint64_t *a, int64_t lo, in
 struct LshTables {
     const uint64_t *keys;
     const uint32_t *ids, *dir;
-    const float *X, *At, *B;  // points; functions, coordinate-major [K][d][L]; offsets
+    const float *X, *A, *At, *B;  // points; functions [L][K][d], and coordinate-major [K][d][L]; offsets
     int64_t n;
     int d, K, L, key_bits, dir_bits;
     uint64_t salt;
@@ -204,12 +204,20 @@ __global__ void lsh_directory_kernel(const uint64_t *__restrict__ keys, int64_t 
 // scattered loads: n = 1e6, L = 50, 1e4 queries: 469 us with two binary searches over the
 // whole table and the tuple check reading rows of A per lane, 311 with the key directory,
 // 130 with the functions coordinate-major (a warp's lanes are consecutive tables).
+// kWarp: a warp per (query, table), a lane per function. A thread alone checks its K d products
+// in one chain of loads, and with few lookups there is nothing beside it (d = 384, K = 16, L = 10,
+// whole calls: one query 391 -> 118 us, 300 queries 415 -> 184; at 11000 lookups 462, where a
+// thread each is as fast).
+template <bool kWarp>
 __global__ void lsh_lookup_kernel(const int32_t *__restrict__ HQ, int64_t m, LshTables t, int64_t *__restrict__ range,
                                   unsigned long long *__restrict__ count) {
     const int K = t.K, L = t.L;
     const int64_t n = t.n;
     const int64_t total = m * L;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    constexpr int kLanes = kWarp ? 32 : 1;
+    const int lane = threadIdx.x % kLanes;
+    for (int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kLanes; e < total;
+         e += (int64_t)gridDim.x * blockDim.x / kLanes) {
         const int64_t j = e / L, l = e % L;
         const int32_t *hq = HQ + j * (int64_t)K * L + l * K;
         const uint64_t bk = bucket_key(hq, K, t.salt, t.key_bits);
@@ -220,7 +228,18 @@ __global__ void lsh_lookup_kernel(const int32_t *__restrict__ HQ, int64_t m, Lsh
         const int64_t d0 = l * n + dir[0], d1 = l * n + dir[1];
         const int64_t lo = lower_bound(t.keys, d0, d1, key);
         int64_t hi = lower_bound(t.keys, lo, d1, key + 1);
-        if (hi > lo) {
+        if (kWarp && hi > lo) {
+            const float *x = t.X + (int64_t)t.ids[lo] * t.d;
+            bool other = false;  // (a tuple with the same key: not this query's bucket)
+            for (int k = lane; k < K; k += kLanes) {
+                const float *a = t.A + (l * K + k) * t.d;
+                float s = 0.f;
+#pragma unroll 8
+                for (int c = 0; c < t.d; ++c) s = __fmaf_rn(x[c], a[c], s);
+                other |= hash_of_dot(s, t.B[l * K + k]) != hq[k];
+            }
+            if (__any_sync(0xffffffffu, other)) hi = lo;
+        } else if (hi > lo) {
             // eight functions at a time, the point's coordinates read once for all of them (the
             // operations of the hash kernel, in its order)
             const float *x = t.X + (int64_t)t.ids[lo] * t.d;
@@ -243,6 +262,7 @@ __global__ void lsh_lookup_kernel(const int32_t *__restrict__ HQ, int64_t m, Lsh
                     if (u < kn && hash_of_dot(acc[u], t.B[l * K + k0 + u]) != hq[k0 + u]) hi = lo;
             }
         }
+        if (lane) continue;
         range[2 * e] = lo;
         range[2 * e + 1] = hi;
         if (count && hi > lo) atomicAdd(&count[j], (unsigned long long)(hi - lo));
@@ -683,7 +703,18 @@ int bits_for(int64_t v) {
 }
 
 LshTables tables_of(const stag_lsh *h) {
-    return LshTables{h->keys, h->ids, h->dir, h->X, h->At, h->B, h->n, (int)h->d, h->K, h->L, h->key_bits, h->dir_bits, h->salt};
+    return LshTables{h->keys, h->ids, h->dir,      h->X,        h->A,   h->At,
+                     h->B,    h->n,   (int)h->d, h->K, h->L, h->key_bits, h->dir_bits, h->salt};
+}
+
+// A warp per lookup while all of them are resident at once.
+void launch_lookup(const stag_lsh *h, const int32_t *HQ, int64_t m, int64_t *range, unsigned long long *count,
+                   cudaStream_t s) {
+    const int64_t lookups = m * h->L;
+    if (lookups <= 152 * 64)
+        lsh_lookup_kernel<true><<<grid_for_elems(lookups * 32, 256), 256, 0, s>>>(HQ, m, tables_of(h), range, count);
+    else
+        lsh_lookup_kernel<false><<<grid_for_elems(lookups, 256), 256, 0, s>>>(HQ, m, tables_of(h), range, count);
 }
 
 // One pass over the bitmaps: bucket ranges and sizes, their prefix sum, the 32-bit lists at
@@ -717,7 +748,7 @@ int lsh_run_bitmap1(stag_lsh *h, const int32_t *HQ, int64_t *range, unsigned lon
     const bool fixed = m * h->n * 4 <= kFixedRawBytes;
     if (!fixed) STAG_CUDA_TRY(cudaMemsetAsync(count, 0, m * 8, s));
     count_launch();
-    lsh_lookup_kernel<<<grid_for_elems(m * h->L, 256), 256, 0, s>>>(HQ, m, tables_of(h), range, fixed ? nullptr : count);
+    launch_lookup(h, HQ, m, range, fixed ? nullptr : count, s);
     STAG_CUDA_TRY(cudaGetLastError());
     int64_t R = m * h->n;
     if (!fixed) {
@@ -810,7 +841,7 @@ int lsh_run_bitmap(stag_lsh *h, const int32_t *HQ, int64_t *range, int64_t m, in
     STAG_CUDA_TRY(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, h->device));
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(items, (int64_t)dev_sms * 2));
     count_launch(4);
-    lsh_lookup_kernel<<<grid_for_elems(m * h->L, 256), 256, 0, s>>>(HQ, m, tables_of(h), range, nullptr);
+    launch_lookup(h, HQ, m, range, nullptr, s);
     count_k<<<grid, kBmThreads, smem, s>>>(range, m, h->L, h->ids, words, slices, sw, ucount, nullptr, nullptr);
     scan_i64_kernel<<<1, 1024, 0, s>>>(ucount, items, item_off);
     lsh_item_to_query_off_kernel<<<grid_for_elems(m + 1, 256), 256, 0, s>>>(item_off, m, slices, dOff);
@@ -884,7 +915,7 @@ int lsh_run(stag_lsh *h, const float *dQ, int64_t m, int64_t *dOff, cudaStream_t
     if (bitmap_fits(h->n)) return lsh_run_bitmap(h, HQ, range, m, dOff, s, total);
     STAG_CUDA_TRY(cudaMemsetAsync(count, 0, m * 8, s));
     count_launch(2);
-    lsh_lookup_kernel<<<grid_for_elems(m * L, 256), 256, 0, s>>>(HQ, m, tables_of(h), range, count);
+    launch_lookup(h, HQ, m, range, count, s);
     scan_i64_kernel<<<1, 1024, 0, s>>>(count, m, raw_off);
     STAG_CUDA_TRY(cudaGetLastError());
     int64_t R = 0;

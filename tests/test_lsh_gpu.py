@@ -329,3 +329,26 @@ def test_lists_without_room_for_the_32_bit_copy(m, way, monkeypatch):
     # device: scratch, then the 32-bit lists; host: queries, scratch, the 32-bit lists, the lists
     for k in ((2,) if way == "device" else (3, 4)):
         assert answered >> k & 1, (k, bin(answered))
+
+
+@pytest.mark.parametrize("K,d", [(1, 3), (9, 7), (33, 4), (40, 2)])
+@pytest.mark.parametrize("m", [60, 3242, 3243])  # a warp per lookup up to 9728 of them (L = 3), then a thread
+def test_lookup_forms(K, d, m, monkeypatch):
+    # fewer and more functions than lanes; with 9-bit keys, lookups that land on another
+    # tuple's key must be rejected by comparing the functions
+    import torch
+    r = np.random.default_rng(K * 10 + m)
+    X = (r.standard_normal((600, d)) * (0.5 if K > 9 else 0.15)).astype(np.float32)
+    near = X[r.integers(0, 600, m // 2)]
+    far = (r.uniform(-100, 100, size=(m - len(near), d))).astype(np.float32)
+    Q = np.concatenate([near, far])
+    A, B = (r.standard_normal((3 * K, d)) * 0.3).astype(np.float32), (4 * r.random(3 * K)).astype(np.float32)
+    HX, HQ = oracle.lsh_hash(X, A, B), oracle.lsh_hash(Q, A, B)
+    tuples = max(len({tuple(v) for v in HX[:, l * K:(l + 1) * K]}) for l in range(3))
+    if tuples <= 12:  # (few enough for a salt that keeps them apart)
+        monkeypatch.setenv("STAG_KDE_LSH_KEY_BITS", "9")
+    with _cls()(X, K, 3, A=A, B=B) as lsh:
+        off, idx = lsh.query_dev(torch.from_numpy(Q).cuda())
+    woff, widx = oracle.lsh_candidates(HX, HQ, K, 3)
+    assert woff[len(near)] > 0
+    assert np.array_equal(off.cpu().numpy(), woff) and np.array_equal(idx.cpu().numpy(), widx)
