@@ -169,7 +169,9 @@ int launch_simt(const stag_kde *h, dim3 grid, cudaStream_t s, int64_t m, int64_t
     }
 }
 
-// Number of point-set splits: enough blocks for several waves of 2 blocks per SM.
+// Points per split: about 12 blocks per SM in all, four waves of the three resident ones. (The
+// last wave may be nearly empty: n = 70000, m = 10000 gives 1884 blocks on 456 slots, 4.13 waves.
+// Another count would regroup the FP32 sums.)
 static int64_t choose_tiles_per_split(const stag_kde *h, int64_t q_tiles) {
     const int64_t target_blocks = (int64_t)h->sm_count * 2 * 6;
     int64_t splits = std::max<int64_t>(1, ceil_div(target_blocks, q_tiles));

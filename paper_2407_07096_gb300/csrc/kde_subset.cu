@@ -42,10 +42,8 @@ constexpr int kFlush = 16;
 constexpr int64_t kSubsetMaxD = 1536;
 constexpr int kSubStages = 3;    // stages of a warp's ring
 constexpr int kSubChunk = 16;    // coordinates a stage holds per row (one summation block)
+
 __device__ __forceinline__ int clampe(float e) { return (int)fminf(fmaxf(e, -4000.f), 4000.f); }
-__device__ __forceinline__ void copy16(void *smem, const void *g) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(g));
-}
 __device__ __forceinline__ void copy4(void *smem, const void *g) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(g));
 }

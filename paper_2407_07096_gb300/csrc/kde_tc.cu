@@ -493,10 +493,10 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
                         constexpr uint32_t HI_AUG = ptx::smem_desc_hi(256, ptx::kSw32);
                         auto issue = [&](uint32_t d_tmem, uint32_t row0) {
                             uint32_t accumulate = 0;
-    #pragma unroll
+#pragma unroll
                             for (int prod = 0; prod < 3; ++prod) {
                                 // (u_hi, v_hi), (u_hi, v_lo), (u_lo, v_hi); B rows row0..
-    #pragma unroll
+#pragma unroll
                                 for (int s = 0; s < KS; ++s) {
                                     const uint32_t aoff = (prod == 2 ? C::A_PLANE : 0) + G::koff(s, BM);
                                     const uint32_t boff =
@@ -510,7 +510,7 @@ __device__ __forceinline__ void tc_body(const TcInst *__restrict__ insts, bool i
                             ptx::mma_f16_w(d_tmem, alo_aug, HI_AUG, blo_aug + ((row0 * 32) >> 4), HI_AUG, C::IDESC, 1);
                         };
                         if constexpr (C::RING) {
-    #pragma unroll
+#pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 const uint32_t k = 2 * tcount + h;  // half tile index, CTA-wide
                                 const int acc = k % C::NACC;

@@ -25,9 +25,9 @@
 // walks it in index order, writing the list at an offset known from the bucket sizes (one
 // pass; the compact int64 lists are written when they are fetched). Up to 2^22 points, and
 // where those offsets would take too much memory, a block takes (query, slice) items in two
-// such walks (a counting pass, a prefix sum over the items, a writing pass). Beyond that, every
-// bucket member is listed (one warp per query) and repeats are removed by a radix sort of
-// (query << 32 | index) keys and a per-query unique pass.
+// such walks (a counting pass, a prefix sum over the items, a writing pass). Beyond 2^22
+// points every bucket member is listed (one warp per query) and repeats are removed by a
+// radix sort of (query << 32 | index) keys and a per-query unique pass.
 #include <stdint.h>
 #include <stdlib.h>
 
