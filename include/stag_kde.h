@@ -130,6 +130,10 @@ int stag_kde_query(stag_kde_t *h, const void *Q, int64_t m, double *out);
  * Scratch memory is owned by the handle and grown on demand (a growth synchronises the
  * handle's device); stag_kde_reserve() pre-sizes it, after which the call allocates
  * nothing for m <= the reserved size.
+ * An FP64 query under stream capture, and an FP64 instance of a batch, uses one block per 32
+ * queries, which walks all points (its replays may overlap other queries of the handle): below
+ * about 39000 queries that is slower than the direct call (n = m = 1000, d = 2: 193 against
+ * 48 us; n = 1e5, m = 1, d = 8: 1.60 ms against 19 us).
  */
 int stag_kde_query_dev(stag_kde_t *h, const void *dQ, int64_t m, double *dOut, void *stream);
 
