@@ -203,7 +203,7 @@ __global__ void lsh_directory_kernel(const uint64_t *__restrict__ keys, int64_t 
 // member's K values equal the query's: exact membership); per query: the total. Bound by its
 // scattered loads: n = 1e6, L = 50, 1e4 queries: 469 us with two binary searches over the
 // whole table and the tuple check reading rows of A per lane, 311 with the key directory,
-// 130 with the functions coordinate-major (a warp's lanes are consecutive tables).
+// 116 with the functions coordinate-major (a warp's lanes are consecutive tables).
 // kWarp: a warp per (query, table), a lane per function. A thread alone checks its K d products
 // in one chain of loads, and with few lookups there is nothing beside it (d = 384, K = 16, L = 10,
 // whole calls: one query 391 -> 118 us, 300 queries 415 -> 184; at 11000 lookups 462, where a
@@ -460,7 +460,7 @@ lsh_bitmap_kernel(const int64_t *__restrict__ range, int64_t m, int L, const uin
 // two tables and the loads in turn), the next query's ranges are loaded meanwhile, and with
 // kSum a summary bitmap (one bit per word) lets the walk visit only the words that hold
 // something. kSum pays above 2^17 points (several blocks of 256 threads per SM without it).
-// Measured, n = 1e6, L = 50, 1e4 queries (7e7 members, 3.9e7 distinct): 431 us, and 109 to
+// Measured, n = 1e6, L = 50, 1e4 queries (7e7 members, 3.9e7 distinct): 413 us, and 134 to
 // expand, against 334 + 678 for the two passes and ~90 for the copy of their lists. Loading
 // the next query's members during the walk made no difference there (the walk and the bits
 // are bound by issue: about 10k of 13k clocks per query) and 24 % at n = 1e5.
