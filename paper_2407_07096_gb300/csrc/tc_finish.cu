@@ -499,7 +499,7 @@ __device__ __forceinline__ void combine_group(const FinInst &I, int g, int F, in
 
 __global__ void __launch_bounds__(kFixThreads, 3)
 fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int n_inst, int qblocks, int max_passes,
-               FinCtl *ctl, int *err) {
+               FinCtl *ctl, int *err, int sms) {
     extern __shared__ __align__(16) float smem[];
     RadixSmem &radix = *reinterpret_cast<RadixSmem *>(smem);  // (the sort's and the lists' phases take turns)
     __shared__ int s_item, s_ok, wcnt[8], warp_sums[kFixThreads / 32], sq[64];
@@ -512,11 +512,21 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
     int *chunk_begin = reinterpret_cast<int *>(ctl + 1), *group_begin = chunk_begin + n_inst + 1,
         *item_begin = group_begin + n_inst + 1, *flagged = item_begin + n_inst + 1;
 
-    // One phase: its N items, whoever takes them, are done when this returns true.
+    // One phase: its N items, whoever takes them, are done when this returns true. `spread`: blocks
+    // are placed on the SMs in turn, and the second and third block of an SM let the first ones
+    // claim before them (waiting 3 us at most), so that few items lie on different SMs. Whoever asked
+    // first took them before, up to three on one SM: the lists of a batch of 7 instances (90
+    // items) 157 us, 80 so; of 200 queries on 20000 points in 128 dimensions (160 items) 114, 81 so.
     int phase = 0;
-    auto run = [&](int N, auto body) -> bool {
+    auto run = [&](int N, auto body, bool spread = false) -> bool {
         const int ph = phase++;
         if (N <= 0) return true;
+        if (spread && tid == 0) {
+            const int before = (int)blockIdx.x / sms * sms;
+            const uint64_t t0 = ptx::globaltimer();
+            while (*reinterpret_cast<volatile int *>(&ctl->claim[ph]) < before && ptx::globaltimer() - t0 < 3000)
+                __nanosleep(100);
+        }
         while (true) {
             __syncthreads();
             if (tid == 0) s_item = atomicAdd(&ctl->claim[ph], 1);
@@ -674,7 +684,7 @@ fin_fix_kernel(const __grid_constant__ FinInst inst0, const FinInst *table, int 
         if (lg < 0 || w < I.item_off[lg] || w >= I.item_off[lg + 1])
             lg = find_owner(group_begin[li + 1] - group_begin[li], w, [&](int k) { return I.item_off[k]; });
         list_item(I, lg, w, smem);
-    });
+    }, true);
     if (ok)
         run(groups, [&](int gg) {
             const int i = inst_of_group(gg);
@@ -765,7 +775,8 @@ int fin_launch(const FinInst &inst0, const FinInst *table, int n_inst, int cbloc
     count_launch();
     // (the ring's layout follows each instance's d_pad; the widest layout is the streamed one)
     const size_t smem = std::max(simt::simt_smem(std::min(max_d_pad, kSimtResidentMaxD)), simt::simt_smem(max_d_pad));
-    fin_fix_kernel<<<grid, kFixThreads, smem, s>>>(inst0, table, n_inst, qblocks, max_passes, ctl, err);
+    fin_fix_kernel<<<grid, kFixThreads, smem, s>>>(inst0, table, n_inst, qblocks, max_passes, ctl, err,
+                                                   sm_count);
     STAG_CUDA_TRY(cudaGetLastError());
     return 0;
 }
